@@ -99,13 +99,13 @@ struct fci_ctx {
     float *kf = nullptr;            // [npair] k_kl = h_kl - 1/2 sum_j (kj|jl), FP32 (same-spin tensor-core path)
     float *ws32 = nullptr;          // [2][ndet] FP32 workspace of that path (allocated on first use)
     // FP64 sliced sigma_3 (sigma3_sliced.cu): fixed-point integrals, the
-    // per-call row exponents of C and its six bf16 digit slices (slices 0-3
-    // and 4-5 as two planes, 12 bytes per determinant)
+    // per-call row exponents of C and its six bf16 digit planes [row][pitch]
+    // (pitch: the strings of a row rounded up to 128; the padding stays zero)
     long long *XW = nullptr;        // [npair][npair] round(W 2^(47 - eW))
     int eW = 0;                     // |W| < 2^eW
     int *rowexp = nullptr;          // [N_alpha]
-    uint2 *cs0123 = nullptr;        // [ndet]
-    uint32_t *cs45 = nullptr;       // [ndet]
+    uint16_t *planes = nullptr;
+    size_t planes_bytes = 0;
     // FP64 sigma for large spaces (sigma_wide.cu): the fixed-point integral
     // table, the exponent of the call's C, and the 64-bit accumulator
     // (aliases ws32 when the context has it)
@@ -222,6 +222,9 @@ int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *v
 int run_rdm1(fci_ctx *ctx, const void *c, int dtype, double *gamma);
 // rdm2.cu
 int run_rdm2(fci_ctx *ctx, const void *c, int dtype, double *gamma1, double *gamma2);
+
+// row pitch of the digit planes of C: whole tiles of kTileStrings
+inline int64_t plane_pitch(int64_t ncols) { return (ncols + kTileStrings - 1) / kTileStrings * kTileStrings; }
 
 inline unsigned ceil_div(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 

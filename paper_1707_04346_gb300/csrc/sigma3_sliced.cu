@@ -40,19 +40,18 @@ __global__ void k_pair_table(const uint32_t *__restrict__ tab, int64_t ns, int n
     tabp[x * npad + ent_pair(v)] = (uint16_t)(ent_target(v) | (ent_negative(v) ? 0x8000u : 0u));
 }
 
-// Six bf16 digit slices of every C value, relative to its row's exponent:
-// slices 0-3 to cs0123, 4-5 to cs45 (d_s 2^(-8s), d_s balanced 8-bit digits of
-// round(|C| 2^(47 - e_row)) with the sign).
+// Six bf16 digit planes of C relative to each row's exponent (plane d, row r,
+// column j at planes[(d nrows + r) pitch + j]: d_s 2^(-8s), d_s balanced 8-bit
+// digits of round(|C| 2^(47 - e_row)) with the sign); a thread takes 8
+// consecutive columns and writes 16 bytes per plane (zeros past the row's end).
 __global__ void k_slice_c(const double *__restrict__ C, const int *__restrict__ rowexp, int64_t nrows, int64_t ncols,
-                          uint2 *__restrict__ cs0123, uint32_t *__restrict__ cs45, const int *__restrict__ active) {
+                          int64_t pitch, uint16_t *__restrict__ planes, const int *__restrict__ active) {
     if (active != nullptr && *active == 0) return;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nrows * ncols) return;
-    const unsigned long long b = __double_as_longlong(__ldg(C + t));
-    float f[sl::kSlices];
-    sl::digits6(sl::fixed47((uint32_t)b, (uint32_t)(b >> 32), __ldg(rowexp + t / ncols)), f);
-    cs0123[t] = make_uint2(sl::pack_bf16(f[0], f[1]), sl::pack_bf16(f[2], f[3]));
-    cs45[t] = sl::pack_bf16(f[4], f[5]);
+    const int64_t groups = pitch / 8;
+    if (t >= nrows * groups) return;
+    const int64_t r = t / groups, j0 = (t - r * groups) * 8;
+    sl::slice8(C + r * ncols, j0, ncols, __ldg(rowexp + r), planes + r * pitch + j0, nrows * pitch);
 }
 
 // Sizes of the sliced kernel for this context; false when it does not apply.
@@ -114,8 +113,8 @@ int build_sliced_tables(fci_ctx *ctx, const double *h1_host, const double *eri_h
     int rc = FCI_OK;
     ctx->XW = (long long *)dalloc(ctx, sizeof(long long) * (size_t)np * np, &rc);
     ctx->rowexp = (int *)dalloc(ctx, sizeof(int) * (size_t)ctx->A.ns, &rc);
-    ctx->cs0123 = (uint2 *)dalloc(ctx, sizeof(uint2) * (size_t)ctx->ndet, &rc);
-    ctx->cs45 = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)ctx->ndet, &rc);
+    ctx->planes_bytes = sizeof(uint16_t) * sl::kSlices * (size_t)ctx->A.ns * plane_pitch(ctx->B.ns);
+    ctx->planes = (uint16_t *)dalloc(ctx, ctx->planes_bytes, &rc);
     SpinTables &B = ctx->B;
     B.tabp = (uint16_t *)dalloc(ctx, sizeof(uint16_t) * (size_t)npad * B.ns, &rc);
     if (rc) return rc;
@@ -134,12 +133,10 @@ void free_sliced_tables(fci_ctx *ctx) {
     ctx->B.tabp = nullptr;
     dfree(ctx, ctx->XW, sizeof(long long) * (size_t)np * np);
     dfree(ctx, ctx->rowexp, sizeof(int) * (size_t)ctx->A.ns);
-    dfree(ctx, ctx->cs0123, sizeof(uint2) * (size_t)ctx->ndet);
-    dfree(ctx, ctx->cs45, sizeof(uint32_t) * (size_t)ctx->ndet);
+    dfree(ctx, ctx->planes, ctx->planes_bytes);
     ctx->XW = nullptr;
     ctx->rowexp = nullptr;
-    ctx->cs0123 = nullptr;
-    ctx->cs45 = nullptr;
+    ctx->planes = nullptr;
 }
 
 static void *sliced_kernel(int kpad);
@@ -179,7 +176,8 @@ int launch_sigma3_sliced(fci_ctx *ctx, const double *C, double *sig, cudaStream_
     const SpinTables &A = ctx->A, &B = ctx->B;
     k_row_exponents<<<ceil_div(A.ns * 32, 256), 256, 0, s>>>(C, A.ns, B.ns, ctx->rowexp, active);
     FCI_CUDA(cudaGetLastError());
-    k_slice_c<<<ceil_div(ctx->ndet, 256), 256, 0, s>>>(C, ctx->rowexp, A.ns, B.ns, ctx->cs0123, ctx->cs45, active);
+    int64_t pitch = plane_pitch(B.ns);
+    k_slice_c<<<ceil_div(A.ns * (pitch / 8), 256), 256, 0, s>>>(C, ctx->rowexp, A.ns, B.ns, pitch, ctx->planes, active);
     FCI_CUDA(cudaGetLastError());
     prof_mark(ctx, rec, prof_slot, s);
     void *kern = sliced_kernel(kpad);
@@ -191,12 +189,11 @@ int launch_sigma3_sliced(fci_ctx *ctx, const double *C, double *sig, cudaStream_
     int64_t grid = nsm;  // one CTA per SM
     if (grid > A.ns) grid = A.ns;
     SpinTables At = A, Bt = B;
-    const uint2 *c0 = ctx->cs0123;
-    const uint32_t *c4 = ctx->cs45;
+    const uint16_t *planes = ctx->planes;
     const long long *xw = ctx->XW;
     const int *rexp = ctx->rowexp;
     int npair = ctx->npair, eW = ctx->eW;
-    void *args[] = {(void *)&c0,   (void *)&c4,    (void *)&sig,  (void *)&At, (void *)&Bt,         (void *)&xw,
+    void *args[] = {(void *)&planes, (void *)&pitch, (void *)&sig,  (void *)&At, (void *)&Bt,         (void *)&xw,
                     (void *)&rexp, (void *)&npair, (void *)&npad, (void *)&n0, (void *)&eW, (void *)&ctx->d_err,
                     (void *)&active, (void *)&add};
     FCI_CUDA(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(sl::kThreads), args, smem, s));

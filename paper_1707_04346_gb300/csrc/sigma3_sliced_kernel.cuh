@@ -13,7 +13,8 @@
 //    cut into six balanced 8-bit digits X = d0 2^40 + d1 2^32 + ... + d5,
 //    |d_s| <= 128 (the low digits are centred on zero, so the products that
 //    are left out have zero mean), stored as the bf16 values d_s 2^(-8s),
-//    which bf16 holds exactly (12 bytes per determinant, two planes);
+//    which bf16 holds exactly: six planes [row][pitch], the row pitch a
+//    multiple of 128 strings (12 bytes per determinant);
 //  * per alpha row, the rows J_a it gathers share the largest of their
 //    exponents, eD; the factor 2^(e_row(J_a) - eD) of each replacement is
 //    folded into the integral operand, whose digits are rebuilt per row from
@@ -30,9 +31,12 @@
 //    instructions (GB300 runs float-integer conversions on its slow FP64
 //    pipe): levels 0-2 accumulate on biases that leave their integers in the
 //    low mantissa bits, level 3+ is rounded with FP32 magic-number additions.
-//    It adds s_b V into the target's 64-bit slot of the sigma row in shared
-//    memory with an integer atomic: the adds are exact and their order does
-//    not matter, so the result is bit-reproducible;
+//    It adds s_b V into the target's slot of the sigma row in shared memory,
+//    two 32-bit words (the low words, then the high words of the row) and two
+//    32-bit integer atomics, the second carrying the first's overflow: an exact
+//    64-bit add whose order does not matter, so the result is
+//    bit-reproducible.  (A 64-bit atomic add in shared memory costs 27 cycles
+//    per warp and SM on random slots at eight warps, the two 32-bit ones 6.3.)
 //  * at the end of the row the integers are converted to FP64 (integer
 //    arithmetic only, round to nearest even) and written to sigma, which this
 //    kernel overwrites (or adds to, when add != 0).
@@ -45,20 +49,29 @@
 // lane from tensor memory with compile-time register indices and needs no
 // staging of G; one 16-byte load brings the entries of 8 columns.
 //
-// CTA (416 threads), one per SM, persistent over alpha rows:
-//  * warps 0-3 (producers): thread m gathers the sliced values C(J_a, J_b) of
-//    beta string J_b = 128 t + m and transposes them into the six A slices,
-//    K-major (no swizzle) in shared memory; each K-step (16 replacements) sits
-//    behind its own pair of barriers so that the next tile's slices are written
-//    while the tensor cores finish this one;
-//  * warp 12 (one thread) issues the MMAs: per tile, the accumulator columns
+// CTA (544 threads), one per SM, persistent over alpha rows:
+//  * warps 0-3 (producers) copy the digit planes' rows J_a, 128 strings of a
+//    tile at a time, into the six A slices with 16-byte asynchronous copies.
+//    The slices are MN-major (128-byte swizzle: 64 strings x 8 replacements per
+//    kilobyte), so that a row segment of a plane is a row of the operand: no
+//    registers, no transposition, and as many copies in flight as the buffers
+//    hold.  (Gathering through registers, one group of eight replacements in
+//    flight and transposed into a K-major operand, was latency bound.)  Each K-step (16 replacements) sits behind its own pair
+//    of barriers so that the next tile's slices arrive while the tensor cores
+//    finish this one;
+//  * warp 16 (one elected lane) issues the MMAs: per tile, the accumulator columns
 //    are split in two halves (pairs 0..N0-1 and N0..npad-1), each with its own
 //    four level accumulators, so the epilogue of one half overlaps the MMAs of
 //    the other;
-//  * warps 4-11 (epilogue): two warps per tensor-memory lane quarter, taking
-//    alternate 8-column chunks.
+//  * warps 4-15 (epilogue): three warps per tensor-memory lane quarter, taking
+//    every third 8-column chunk; the conversions and adds of a chunk carry no
+//    branches (a branch per entry kept one element in flight per warp).
 // All waits are bounded; a wait that gives up sets the device error word and
 // the CTA drains its MMAs and frees its tensor memory.
+//
+// CAS(14,14): 5.94 ms with register gathers and a branch per epilogue entry,
+// 5.13 ms with the asynchronous gathers and 32-bit adds, 3.90 ms with the
+// branch-free epilogue on twelve warps (MMA operand reads alone: 2.1 ms).
 #pragma once
 #include "sigma_tc_kernel.cuh"
 
@@ -68,8 +81,10 @@ namespace sl {
 using tc::kM;
 
 constexpr int kSlices = 6;    // 8-bit digits per FP64 operand (48 bits)
-constexpr int kThreads = 416; // warps 0-3 producers, 4-11 epilogue, 12 MMA issuer
-constexpr int kEpiThreads = 256;
+constexpr int kEpiGroups = 3; // epilogue warps per tensor-memory lane quarter
+constexpr int kEpiThreads = 128 * kEpiGroups;
+constexpr int kMmaWarp = 4 + 4 * kEpiGroups;  // warps 0-3 producers, then the epilogue, then the MMA issuer
+constexpr int kThreads = 32 * (kMmaWarp + 1);
 constexpr int kMaxKSteps = 6; // K <= 96 (the exact level sums need K <= 85)
 constexpr int kMaxK = 85;
 constexpr int kBars = 2 * kMaxKSteps + 5;  // a_full[6], a_free[6], acc_full[2], acc_empty[2], drain
@@ -79,7 +94,7 @@ struct Layout {
 };
 
 // Shared memory: B slices [6][npad x kpad], A slices [6][128 x kpad], the sigma
-// row as 64-bit integers [nsb], the alpha list [nsingle_a], barriers and words.
+// row as 64-bit integers (low words [nsb], high words [nsb]), the alpha list [nsingle_a], barriers and words.
 __host__ __device__ inline Layout make_layout(int kpad, int npad, int64_t nsb, int nsingle_a) {
     Layout L;
     L.bytesB = (uint32_t)(npad * kpad * 2);
@@ -127,6 +142,28 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// Digits of columns j0 .. j0 + 7 of one row (zeros past ncols), 16 bytes into
+// each of the six planes (out: plane 0, the planes `plane` elements apart).
+__device__ __forceinline__ void slice8(const double *row, int64_t j0, int64_t ncols, int emax, uint16_t *out,
+                                       int64_t plane) {
+    uint32_t w[kSlices][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float f[2][kSlices];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int64_t j = j0 + 2 * i + u;
+            const unsigned long long b = j < ncols ? __double_as_longlong(__ldg(row + j)) : 0ull;
+            digits6(fixed47((uint32_t)b, (uint32_t)(b >> 32), emax), f[u]);
+        }
+#pragma unroll
+        for (int s = 0; s < kSlices; ++s) w[s][i] = pack_bf16(f[0][s], f[1][s]);
+    }
+#pragma unroll
+    for (int s = 0; s < kSlices; ++s)
+        *reinterpret_cast<uint4 *>(out + s * plane) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
 // T * 2^e2 as FP64, by integer arithmetic (round to nearest even; results
 // below the normal range flush to zero).
 __device__ __forceinline__ double scaled_i64(long long T, int e2) {
@@ -154,8 +191,71 @@ __device__ __forceinline__ double scaled_i64(long long T, int e2) {
     return __longlong_as_double((long long)(sgn | ((unsigned long long)E << 52) | (m & 0xFFFFFFFFFFFFFull)));
 }
 
-__device__ __forceinline__ void ld_early_v2(const uint2 *p, uint32_t &x, uint32_t &y) {
-    asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "l"(p));
+// 16-byte asynchronous copy (global to shared, not through registers)
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Descriptor of an MN-major operand in 128-byte-swizzled blocks of 64 MN
+// elements: a K row is 128 bytes, eight of them (1 KB) a swizzle atom, atoms
+// along K sbo apart, 64-element blocks lbo apart.
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    return tc::smem_desc(saddr, lbo, sbo) | ((uint64_t)2 << 61);
+}
+constexpr uint32_t kTransposeA = 1u << 15;  // instruction descriptor: A is MN-major
+
+// Byte offset of 16-byte chunk c (MN elements 8 c .. 8 c + 7, c < 16) of K row a
+// in an MN-major slice of 128 x kpad.
+__device__ __forceinline__ uint32_t mn_offset(int c, int a, int kpad) {
+    return (uint32_t)((c >> 3) * kpad * 128 + (a >> 3) * 1024 + (a & 7) * 128 + (((c & 7) ^ (a & 7)) << 4));
+}
+
+// Producer side of one tile: thread `tid` of 128 copies chunk tid & 15 of the
+// replacement rows a = 16 ks + (tid >> 4) and a + 8 of every K-step into the six
+// slices at a_base (bytesA apart).  `src` points at the tile's first string in
+// row 0 of plane 0; ent[a] gives row J_a.  K-step ks is handed over on
+// a_full(ks) once this thread's copies of it have landed (up to two K-steps
+// stay in flight).  Rows a >= n_ent are not written (zero since the start of
+// the kernel).  Returns false when a wait gave up.
+template <int KPAD, typename Full, typename Free>
+__device__ __forceinline__ bool produce_tile(const uint16_t *src, int64_t pitch, int64_t plane, const uint32_t *ent,
+                                             int n_ent, uint32_t a_base, uint32_t bytesA, int tid, bool first,
+                                             uint32_t free_phase, Full a_full, Free a_free) {
+    constexpr int NKS = KPAD / 16;
+    constexpr int kFlight = 2;
+    const int c = tid & 15, sub = tid >> 4;
+    const uint16_t *col = src + c * 8;
+#pragma unroll
+    for (int ks = 0; ks < NKS + kFlight; ++ks) {
+        if (ks < NKS) {
+            if (!first && !tc::mbar_wait_bounded(a_free(ks), free_phase)) {
+                cp_async_wait<0>();
+                return false;
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int a = ks * 16 + h * 8 + sub;
+                if (a < n_ent) {
+                    const uint16_t *p = col + (int64_t)ent_target(ent[a]) * pitch;
+                    const uint32_t dst = a_base + mn_offset(c, a, KPAD);
+#pragma unroll
+                    for (int d = 0; d < kSlices; ++d) cp_async16(dst + (uint32_t)d * bytesA, p + d * plane);
+                }
+            }
+        }
+        cp_async_commit();
+        if (ks >= kFlight) {
+            cp_async_wait<kFlight>();
+            tc::fence_async_smem();
+            tc::mbar_arrive(a_full(ks - kFlight));
+        }
+    }
+    return true;
 }
 
 // round(X 2^-d) for d >= 0 (zero once d >= 60)
@@ -180,6 +280,7 @@ constexpr uint32_t kBias0 = 0x4B400000u, kBias1 = 0x47400000u, kBias2 = 0x434000
 __device__ __forceinline__ long long levels_to_int(uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3, uint32_t neg) {
     constexpr float M = 12582912.0f;  // 1.5 2^23
     constexpr int MB = 0x4B400000;    // its bit pattern
+    const int sg = -(int)neg;  // 0 or -1: x -> (x ^ sg) - sg negates without a branch
     int hi = (int)(r0 * 256u + r1 - (kBias0 * 256u + kBias1));  // i0 2^8 + i1, exact modulo 2^32
     int i2 = (int)(r2 - kBias2);
     const float a3 = __uint_as_float(r3 ^ (neg << 31));
@@ -187,11 +288,27 @@ __device__ __forceinline__ long long levels_to_int(uint32_t r0, uint32_t r1, uin
     const int h = __float_as_int(t) - MB;
     const float rem = fmaf(-(t - M), 0x1p-18f, a3);  // exact: a3 - h 2^-18
     const int l = __float_as_int(fmaf(rem, 0x1p34f, M)) - MB;
-    if (neg) {
-        hi = -hi;
-        i2 = -i2;
-    }
+    hi = (hi ^ sg) - sg;
+    i2 = (i2 ^ sg) - sg;
     return ((long long)hi << 26) + ((long long)(i2 * 4 + h) << 16) + l;
+}
+
+// Predicated 32-bit adds in shared memory, the first with the old value back
+// (0 where ok is false): no branches, so the conversions and atomics of
+// several columns overlap.
+__device__ __forceinline__ uint32_t atom_add_if(uint32_t addr, uint32_t v, bool ok) {
+    uint32_t old = 0;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p atom.shared.add.u32 %0, [%1], %2;\n\t}"
+        : "+r"(old)
+        : "r"(addr), "r"(v), "r"((uint32_t)ok)
+        : "memory");
+    return old;
+}
+__device__ __forceinline__ void red_add_if(uint32_t addr, uint32_t v, bool ok) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.shared.add.u32 [%0], %1;\n\t}" ::"r"(addr), "r"(v),
+                 "r"((uint32_t)ok)
+                 : "memory");
 }
 
 __device__ __forceinline__ uint4 ld_early_v4(const uint4 *p) {
@@ -212,8 +329,8 @@ __device__ __forceinline__ uint32_t acc_col(int h, int L, int n0, int n1) {
 
 template <int KPAD>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_sigma3_sliced(const uint2 *__restrict__ cs0123, const uint32_t *__restrict__ cs45, double *__restrict__ sig,
-                    SpinTables A, SpinTables B, const long long *__restrict__ XW, const int *__restrict__ rowexp,
+    k_sigma3_sliced(const uint16_t *__restrict__ planes, int64_t pitch, double *__restrict__ sig, SpinTables A,
+                    SpinTables B, const long long *__restrict__ XW, const int *__restrict__ rowexp,
                     int npair, int npad, int n0, int eW, int *err, const int *__restrict__ active, int add) {
     if (active != nullptr && *active == 0) return;  // gated launch (batched engine): instance not active
     constexpr int NKS = KPAD / 16;
@@ -224,7 +341,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const Layout L = make_layout(KPAD, npad, nsb, A.nsingle);
     unsigned char *sB = smem;
     unsigned char *sA = smem + L.offA;
-    unsigned long long *sAcc = reinterpret_cast<unsigned long long *>(smem + L.offAcc);
+    uint32_t *sLo = reinterpret_cast<uint32_t *>(smem + L.offAcc);  // sigma row, low words
+    uint32_t *sHi = sLo + nsb;                                      // high words
     uint32_t *sEa = reinterpret_cast<uint32_t *>(smem + L.offEa);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.offBar);
     volatile int *s_fail = reinterpret_cast<volatile int *>(smem + L.offBar + kBars * 8);
@@ -236,7 +354,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto acc_full = [&](int h) { return bar0 + 8u * (uint32_t)(2 * kMaxKSteps + h); };
     auto acc_empty = [&](int h) { return bar0 + 8u * (uint32_t)(2 * kMaxKSteps + 2 + h); };
     const uint32_t drain = bar0 + 8u * (uint32_t)(2 * kMaxKSteps + 4);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);  // uniform: role branches do not diverge
+    const bool elected = tc::elect_one();  // the MMA warp's issuing lane (one lane issues and commits)
     const int sa_n = A.nsingle;
     const int n1 = npad - n0;
     const int nh = n1 > 0 ? 2 : 1;
@@ -259,15 +379,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::mbar_init(drain, 1);
         *s_fail = 0;
     }
-    for (int64_t j = tid; j < nsb; j += kThreads) sAcc[j] = 0ull;
+    for (int64_t j = tid; j < nsb; j += kThreads) sLo[j] = sHi[j] = 0u;
+    for (uint32_t i = (uint32_t)tid * 16u; i < kSlices * L.bytesA; i += kThreads * 16u)  // padded replacements stay zero
+        *reinterpret_cast<uint4 *>(sA + i) = make_uint4(0u, 0u, 0u, 0u);
+    tc::fence_async_smem();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = *tslot;
-    if (warp >= 4 && warp < 12) {  // level 0-2 biases of both accumulator halves (this warp's chunks)
+    if (warp >= 4 && warp < kMmaWarp) {  // level 0-2 biases of both accumulator halves (this warp's chunks)
         const uint32_t lb = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         for (int h = 0; h < nh; ++h)
-            for (int c = (warp - 4) >> 2; c < (h ? n1 : n0) / 8; c += 2) {
+            for (int c = (warp - 4) >> 2; c < (h ? n1 : n0) / 8; c += kEpiGroups) {
                 tmem_st8(lb + acc_col(h, 0, n0, n1) + (uint32_t)(c * 8), kBias0);
                 tmem_st8(lb + acc_col(h, 1, n0, n1) + (uint32_t)(c * 8), kBias1);
                 tmem_st8(lb + acc_col(h, 2, n0, n1) + (uint32_t)(c * 8), kBias2);
@@ -331,71 +454,19 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::fence_after();
 
         if (warp < 4) {
-            // ---- producers: beta string 128 t + m, one K-group (8 values) at a time,
-            // the next group's loads in flight while this one is transposed ----
-            const int m = tid;
-            uint32_t cx[8], cy[8], cz[8], nx[8], ny[8], nz[8];
-            auto load = [&](uint32_t(&x)[8], uint32_t(&y)[8], uint32_t(&z)[8], int64_t jb, int kg) {
-                const int64_t jc = jb < nsb ? jb : nsb - 1;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int a = kg * 8 + i;
-                    const int64_t idx = (int64_t)ent_target(sEa[a < sa_n ? a : 0]) * nsb + jc;
-                    ld_early_v2(cs0123 + idx, x[i], y[i]);
-                    z[i] = tc::ld_early_u32(cs45 + idx);
-                }
-            };
-            load(cx, cy, cz, m, 0);
+            // ---- producers ----
             for (int64_t t = 0; t < ntiles && !*s_fail; ++t) {
                 const int64_t Tt = T + t;
-                const int64_t jb = t * kM + m;
-                const bool live = jb < nsb;
-#pragma unroll
-                for (int ks = 0; ks < NKS; ++ks) {
-                    if (Tt >= 1 && !tc::mbar_wait_bounded(a_free(ks), (uint32_t)((Tt - 1) & 1))) {
-                        *s_fail = 1;
-                        break;
-                    }
-#pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        const int kg = 2 * ks + g;
-                        if (kg + 1 < kgroups)
-                            load(nx, ny, nz, jb, kg + 1);
-                        else if (t + 1 < ntiles)
-                            load(nx, ny, nz, jb + kM, 0);
-                        if (!live || kg * 8 + 8 > sa_n) {  // dead lane or padded replacements
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                if (!(live && kg * 8 + i < sa_n)) cx[i] = cy[i] = cz[i] = 0u;
-                        }
-                        const uint32_t off = tc::kmajor_offset(m, kg, KPAD);
-#pragma unroll
-                        for (int sl = 0; sl < kSlices; ++sl) {
-                            uint32_t o[4];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const uint32_t x0 = sl < 2 ? cx[2 * i] : sl < 4 ? cy[2 * i] : cz[2 * i];
-                                const uint32_t x1 = sl < 2 ? cx[2 * i + 1] : sl < 4 ? cy[2 * i + 1] : cz[2 * i + 1];
-                                o[i] = __byte_perm(x0, x1, (sl & 1) ? 0x7632 : 0x5410);
-                            }
-                            *reinterpret_cast<uint4 *>(sA + (uint32_t)sl * L.bytesA + off) = make_uint4(o[0], o[1], o[2], o[3]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            cx[i] = nx[i];
-                            cy[i] = ny[i];
-                            cz[i] = nz[i];
-                        }
-                    }
-                    tc::fence_async_smem();
-                    tc::mbar_arrive(a_full(ks));
-                }
+                if (!produce_tile<KPAD>(planes + t * kM, pitch, A.ns * pitch, sEa, sa_n, tc::smem_u32(sA), L.bytesA,
+                                        tid, Tt == 0, (uint32_t)((Tt - 1) & 1), a_full, a_free))
+                    *s_fail = 1;
             }
-        } else if (warp < 12) {
-            // ---- epilogue: lane m of the tile, 8-column chunks g, g+2, ... of each half ----
+        } else if (warp < kMmaWarp) {
+            // ---- epilogue: lane m of the tile, 8-column chunks grp, grp + 3, ... of each half ----
             const int quarter = warp & 3, grp = (warp - 4) >> 2;
             const int m = quarter * 32 + lane;
             const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+            const uint32_t lo0 = tc::smem_u32(sLo), hi0 = tc::smem_u32(sHi);
             for (int64_t t = 0; t < ntiles; ++t) {
                 const int64_t Tt = T + t;
                 const int64_t jb = t * kM + m;
@@ -418,7 +489,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tc::fence_before();
                         tc::mbar_arrive(acc_empty(h));
                     }
-                    for (int c = grp; c < nchunks; c += 2) {
+                    for (int c = grp; c < nchunks; c += kEpiGroups) {
                         uint32_t r[4][8];
 #pragma unroll
                         for (int lv = 0; lv < 4; ++lv)
@@ -432,46 +503,62 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tmem_st8(lane_base + acc_col(h, 1, n0, n1) + (uint32_t)(c * 8), kBias1);
                         tmem_st8(lane_base + acc_col(h, 2, n0, n1) + (uint32_t)(c * 8), kBias2);
                         tmem_st8(lane_base + acc_col(h, 3, n0, n1) + (uint32_t)(c * 8), 0u);
-                        if (c + 2 >= nchunks) {  // last chunk of this thread in the half: release it
+                        if (c + kEpiGroups >= nchunks) {  // last chunk of this thread in the half: release it
                             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                             tc::fence_before();
                             tc::mbar_arrive(acc_empty(h));
                         }
                         const uint4 en = ent;
-                        if (c + 2 < nchunks) ent = fetch(c + 2);
+                        if (c + kEpiGroups < nchunks) ent = fetch(c + kEpiGroups);
                         const uint32_t ew[4] = {en.x, en.y, en.z, en.w};
+                        // every column converted (ILP over the eight), the low words of all
+                        // added first so that their returned values, for the carries, are
+                        // in flight together
+                        uint32_t vl[8], vh[8], old[8];
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             const uint32_t v16 = (j & 1) ? (ew[j >> 1] >> 16) : (ew[j >> 1] & 0xFFFFu);
-                            if (v16 == 0xFFFFu) continue;
                             const long long v = levels_to_int(r[0][j], r[1][j], r[2][j], r[3][j], v16 >> 15);
-                            atomicAdd(sAcc + (v16 & 0x7FFFu), (unsigned long long)v);
+                            vl[j] = (uint32_t)v;
+                            vh[j] = (uint32_t)((unsigned long long)v >> 32);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const uint32_t v16 = (j & 1) ? (ew[j >> 1] >> 16) : (ew[j >> 1] & 0xFFFFu);
+                            old[j] = atom_add_if(lo0 + 4u * (v16 & 0x7FFFu), vl[j], v16 != 0xFFFFu);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const uint32_t v16 = (j & 1) ? (ew[j >> 1] >> 16) : (ew[j >> 1] & 0xFFFFu);
+                            red_add_if(hi0 + 4u * (v16 & 0x7FFFu), vh[j] + (old[j] + vl[j] < vl[j] ? 1u : 0u),
+                                       v16 != 0xFFFFu);
                         }
                     }
                 }
                 if (*s_fail) break;
             }
-        } else if (warp == 12 && lane == 0) {
-            // ---- MMA issuer: descriptors of K-step 0, advanced by 256 bytes (16 in
-            // the address field) per K-step.  A half's six B slices are stacked
+        } else if (warp == kMmaWarp) {
+            // ---- MMA issuer: descriptors of K-step 0, advanced per K-step by 2048
+            // bytes of A (two atoms) and 256 of B.  A half's six B slices are stacked
             // along N and its four levels sit side by side in tensor memory, so
             // A slice s times B slices 0..3-s is one MMA of N = (4 - s) n_h writing
             // levels s..3, and the products of weight 4 and 5 are MMAs of N = n_h
             // into level 3: 15 MMAs per K-step instead of 21 (each M = 128 MMA
             // reads its 4 KB A slice from shared memory; fewer, wider MMAs read it
             // fewer times).  Level 3 starts from zero (written by the epilogue). ----
+            const bool issue = elected;
             uint64_t ad[kSlices], bd0[kSlices], bd1[kSlices];
 #pragma unroll
             for (int sl = 0; sl < kSlices; ++sl) {
-                ad[sl] = tc::smem_desc(tc::smem_u32(sA + sl * L.bytesA), 128, sbo);
+                ad[sl] = smem_desc_mn(tc::smem_u32(sA + sl * L.bytesA), KPAD * 128, 1024);
                 bd0[sl] = tc::smem_desc(tc::smem_u32(sB) + (uint32_t)(sl * n0 / 8) * sbo, 128, sbo);
                 bd1[sl] = tc::smem_desc(tc::smem_u32(sB) + (uint32_t)((kSlices * n0 + sl * n1) / 8) * sbo, 128, sbo);
             }
             uint32_t id0[4], id1[4];  // N = (k + 1) n_h
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                id0[k] = tc::instr_desc(kM, (k + 1) * n0);
-                id1[k] = tc::instr_desc(kM, n1 > 0 ? (k + 1) * n1 : 16);
+                id0[k] = tc::instr_desc(kM, (k + 1) * n0) | kTransposeA;
+                id1[k] = tc::instr_desc(kM, n1 > 0 ? (k + 1) * n1 : 16) | kTransposeA;
             }
             uint32_t col0[4], col1[4];
 #pragma unroll
@@ -485,9 +572,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int ks = 0; ks < NKS; ++ks) {
                     if (wait_a && !tc::mbar_wait_bounded(a_full(ks), (uint32_t)(Tt & 1))) return false;
                     tc::fence_after();
+                    if (!issue) continue;
 #pragma unroll
                     for (int sa = 0; sa < kSlices; ++sa) {
-                        const uint64_t a = ad[sa] + (uint64_t)(ks * 16);
+                        const uint64_t a = ad[sa] + (uint64_t)(ks * 128);
                         const int st = sa < 4 ? 4 - sa : 0;  // stacked B slices 0..st-1 -> levels sa..3
                         if (st > 0) tc::mma_bf16(col[sa], a, bd[0] + (uint64_t)(ks * 16), idn[st - 1], 1u);
 #pragma unroll
@@ -502,11 +590,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int64_t Tt = T + t;
                 bool ok = !(Tt >= 1 && !tc::mbar_wait_bounded(acc_empty(0), (uint32_t)((Tt - 1) & 1)));
                 ok = ok && issue_half(bd0, col0, id0, true, nh == 1, Tt);
-                if (ok) tc::mma_commit(acc_full(0));
+                if (ok && issue) tc::mma_commit(acc_full(0));
                 if (ok && nh == 2) {
                     ok = !(Tt >= 1 && !tc::mbar_wait_bounded(acc_empty(1), (uint32_t)((Tt - 1) & 1)));
                     ok = ok && issue_half(bd1, col1, id1, false, true, Tt);
-                    if (ok) tc::mma_commit(acc_full(1));
+                    if (ok && issue) tc::mma_commit(acc_full(1));
                 }
                 if (!ok) {
                     *s_fail = 1;
@@ -523,15 +611,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int e2 = emax - 1022 + eW - 48;
         double *out = sig + row * nsb;
         for (int64_t j = tid; j < nsb; j += kThreads) {
-            const double v = emax == 0x7FF ? __longlong_as_double(0x7FF8000000000000ll) : scaled_i64((long long)sAcc[j], e2);
+            const double v = emax == 0x7FF ? __longlong_as_double(0x7FF8000000000000ll) : scaled_i64((long long)((unsigned long long)sHi[j] << 32 | sLo[j]), e2);
             out[j] = add ? out[j] + v : v;
-            sAcc[j] = 0ull;
+            sLo[j] = sHi[j] = 0u;
         }
         __syncthreads();
     }
     // ---- exit: wait for every MMA this CTA issued, then free tensor memory ----
-    if (warp == 12 && lane == 0) {
-        tc::mma_commit(drain);
+    if (warp == kMmaWarp) {
+        if (elected) tc::mma_commit(drain);
         if (!tc::mbar_wait_bounded(drain, 0u)) *s_fail = 1;
     }
     tc::fence_before();

@@ -132,6 +132,16 @@ __device__ __forceinline__ float ld_early_f32(const float *p) {
     return v;
 }
 
+// One lane of the (converged) warp.  The MMA warp runs its loop with all lanes
+// and issues under this predicate: loop counters and descriptors then stay in
+// uniform registers, which tcgen05.mma takes its operands from (issuing from a
+// divergent single-lane branch cost 64 cycles per small MMA, 53 this way).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // Bounded wait; returns false if the limit was reached.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t addr, uint32_t parity) {
     for (long it = 0; it < kSpinLimit; ++it)

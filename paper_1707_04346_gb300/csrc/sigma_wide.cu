@@ -2,6 +2,7 @@
 // (sigma_wide_kernel.cuh): its tables (built once at fci_init), the per-call
 // pre-passes, and the sequence of one FP64 sigma = sigma_1 + sigma_2 + sigma_3
 // (Eq. 8) through one 64-bit integer accumulator.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -23,16 +24,15 @@ __global__ void k_global_exponent(const double *__restrict__ x, int64_t n, int *
     if ((threadIdx.x & 31) == 0) atomicMax(eG, (int)mx);
 }
 
-// Six bf16 digit slices of every value, all relative to the one exponent *eG.
-__global__ void k_slice_global(const double *__restrict__ x, int64_t n, const int *__restrict__ eG,
-                               uint2 *__restrict__ cs0123, uint32_t *__restrict__ cs45) {
+// Six bf16 digit planes of a nrows x ncols matrix (layout as in sigma3_sliced.cu),
+// all relative to the one exponent *eG.
+__global__ void k_slice_global(const double *__restrict__ x, int64_t nrows, int64_t ncols, const int *__restrict__ eG,
+                               int64_t pitch, uint16_t *__restrict__ planes) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const unsigned long long b = __double_as_longlong(__ldg(x + t));
-    float f[sl::kSlices];
-    sl::digits6(sl::fixed47((uint32_t)b, (uint32_t)(b >> 32), *eG), f);
-    cs0123[t] = make_uint2(sl::pack_bf16(f[0], f[1]), sl::pack_bf16(f[2], f[3]));
-    cs45[t] = sl::pack_bf16(f[4], f[5]);
+    const int64_t groups = pitch / 8;
+    if (t >= nrows * groups) return;
+    const int64_t r = t / groups, j0 = (t - r * groups) * 8;
+    sl::slice8(x + r * ncols, j0, ncols, *eG, planes + r * pitch + j0, nrows * pitch);
 }
 
 // out[c][r] = in[r][c] for a rows x cols matrix of 8-byte words (32 x 32 tiles).
@@ -165,8 +165,10 @@ int build_wide_tables(fci_ctx *ctx, const double *h1_host, const double *eri_hos
     const int npad0 = round_up16(np);
     ctx->XT = (long long *)dalloc(ctx, sizeof(long long) * xt.size(), &rc);
     ctx->d_eG = (int *)dalloc(ctx, sizeof(int), &rc);
-    if (!ctx->cs0123) ctx->cs0123 = (uint2 *)dalloc(ctx, sizeof(uint2) * (size_t)ctx->ndet, &rc);
-    if (!ctx->cs45) ctx->cs45 = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)ctx->ndet, &rc);
+    // digit planes of C by rows, or of its transpose (sigma_1)
+    const size_t rows = (size_t)std::max(ctx->A.ns * plane_pitch(B.ns), B.ns * plane_pitch(ctx->A.ns));
+    ctx->planes_bytes = sizeof(uint16_t) * sl::kSlices * rows;
+    ctx->planes = (uint16_t *)dalloc(ctx, ctx->planes_bytes, &rc);
     if (!ctx->ws32) ctx->wsacc = (long long *)dalloc(ctx, sizeof(long long) * (size_t)ctx->ndet, &rc);
     if (B.nsingle > 0 && ctx->A.nsingle > 0)
         B.tabp32 = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)npad0 * B.ns, &rc);
@@ -208,12 +210,12 @@ static int launch_wide(fci_ctx *ctx, const SpinTables &R, int64_t ncols, unsigne
     int64_t grid = nsm;  // one CTA per SM
     if (grid > R.ns * S.nparts) grid = R.ns * S.nparts;
     SpinTables Rt = R;
-    const uint2 *c0 = ctx->cs0123;
-    const uint32_t *c4 = ctx->cs45;
+    const uint16_t *planes = ctx->planes;
+    int64_t pitch = plane_pitch(ncols);
     const uint32_t *tabp = ctx->B.tabp32;
     const long long *xt = ctx->XT;
     int npair = ctx->npair, shq = MODE == 0 ? 1 : ctx->sh1;
-    void *args[] = {(void *)&c0,   (void *)&c4,    (void *)&acc,   (void *)&Rt,     (void *)&ncols,
+    void *args[] = {(void *)&planes, (void *)&pitch, (void *)&acc,   (void *)&Rt,     (void *)&ncols,
                     (void *)&tabp, (void *)&xt,    (void *)&npair, (void *)&S.npad, (void *)&S.nparts,
                     (void *)&shq,  (void *)&ctx->d_err};
     FCI_CUDA(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(wd::kThreads), args, S.smem, s));
@@ -223,6 +225,11 @@ static int launch_wide(fci_ctx *ctx, const SpinTables &R, int64_t ncols, unsigne
 static unsigned grid_stride_blocks(int64_t n) {
     const int64_t b = (n + 255) / 256;
     return (unsigned)(b < 8 * 152 ? (b < 1 ? 1 : b) : 8 * 152);
+}
+
+static void slice(fci_ctx *ctx, const double *x, int64_t nrows, int64_t ncols, cudaStream_t s) {
+    const int64_t pitch = plane_pitch(ncols);
+    k_slice_global<<<ceil_div(nrows * (pitch / 8), 256), 256, 0, s>>>(x, nrows, ncols, ctx->d_eG, pitch, ctx->planes);
 }
 
 // FP64 sigma = H C through the wide kernels (sig overwritten):
@@ -245,7 +252,7 @@ int launch_sigma_f64_wide(fci_ctx *ctx, const double *C, double *sig, cudaStream
         auto sigma3 = [&](int rec, int slot, int add) -> int {
             FCI_CUDA(cudaMemsetAsync(ctx->d_eG, 0, sizeof(int), s));
             k_global_exponent<<<grid_stride_blocks(n), 256, 0, s>>>(C, n, ctx->d_eG);
-            k_slice_global<<<ceil_div(n, 256), 256, 0, s>>>(C, n, ctx->d_eG, ctx->cs0123, ctx->cs45);
+            slice(ctx, C, ctx->A.ns, ctx->B.ns, s);
             FCI_CUDA(cudaGetLastError());
             FCI_CUDA(cudaMemsetAsync(acc, 0, sizeof(long long) * (size_t)n, s));
             prof_mark(ctx, rec, slot, s);
@@ -281,7 +288,7 @@ int launch_sigma_f64_wide(fci_ctx *ctx, const double *C, double *sig, cudaStream
                                             : reinterpret_cast<unsigned long long *>(ctx->wsacc);
         FCI_CUDA(cudaMemsetAsync(ctx->d_eG, 0, sizeof(int), s));
         k_global_exponent<<<grid_stride_blocks(n), 256, 0, s>>>(C, n, ctx->d_eG);
-        k_slice_global<<<ceil_div(n, 256), 256, 0, s>>>(C, n, ctx->d_eG, ctx->cs0123, ctx->cs45);
+        slice(ctx, C, ctx->A.ns, ctx->B.ns, s);
         FCI_CUDA(cudaGetLastError());
         FCI_CUDA(cudaMemsetAsync(acc, 0, sizeof(long long) * (size_t)n, s));
         prof_mark(ctx, rec, 0, s);
@@ -311,8 +318,7 @@ int launch_sigma_f64_wide(fci_ctx *ctx, const double *C, double *sig, cudaStream
     if (B.nsingle > 0) {
         k_transpose_u64<<<dim3(ceil_div(nsb, 32), ceil_div(nsa, 32)), tb, 0, s>>>(
             reinterpret_cast<const unsigned long long *>(C), acc, nsa, nsb);
-        k_slice_global<<<ceil_div(n, 256), 256, 0, s>>>(reinterpret_cast<const double *>(acc), n, ctx->d_eG,
-                                                        ctx->cs0123, ctx->cs45);
+        slice(ctx, reinterpret_cast<const double *>(acc), nsb, nsa, s);
         FCI_CUDA(cudaGetLastError());
         prof_mark(ctx, rec, 0, s);
         FCI_CUDA(cudaMemsetAsync(sacc, 0, sizeof(long long) * (size_t)n, s));
@@ -326,7 +332,7 @@ int launch_sigma_f64_wide(fci_ctx *ctx, const double *C, double *sig, cudaStream
         prof_mark(ctx, rec, 1, s);
     }
     if (A.nsingle > 0) {
-        k_slice_global<<<ceil_div(n, 256), 256, 0, s>>>(C, n, ctx->d_eG, ctx->cs0123, ctx->cs45);
+        slice(ctx, C, ctx->A.ns, ctx->B.ns, s);
         FCI_CUDA(cudaGetLastError());
         if (B.nsingle > 0)
             if (int rc = launch_wide<0>(ctx, A, nsb, acc, s)) return rc;

@@ -53,11 +53,15 @@
 // i.e. 1/2 sum (ij|kl) E_ij E_kl + sum k_kl E_kl with the identity resolved
 // over intermediate strings; the adds of a warp go to one row, consecutive J.
 //
-// CTA (416 threads), one per SM, persistent over items: warps 0-3 gather and
-// transpose the A slices (as in the per-row kernel), warps 4-11 read the
-// accumulators (two warps per lane quarter, alternate 8-column chunks), warp
-// 12 issues the MMAs.  All waits are bounded; a wait that gives up sets the
+// CTA (544 threads), one per SM, persistent over items: warps 0-3 gather the A
+// slices by asynchronous copies (as in the per-row kernel), warps 4-15 read the
+// accumulators (three warps per lane quarter, every third 8-column chunk), warp
+// 16 issues the MMAs.  All waits are bounded; a wait that gives up sets the
 // device error word, and the CTA drains its MMAs and frees tensor memory.
+//
+// sigma_3 at CAS(16,16): 133.7 ms with register gathers and a branch per entry,
+// 75.2 ms with asynchronous gathers, 72.0 ms with the branch-free epilogue on
+// twelve warps; the 64-bit adds into global memory (1.2e10) bound it now.
 #pragma once
 #include "sigma3_sliced_kernel.cuh"
 
@@ -67,8 +71,10 @@ namespace wd {
 using sl::kSlices;
 using tc::kM;
 
-constexpr int kThreads = 416;      // warps 0-3 producers, 4-11 epilogue, 12 MMA issuer
-constexpr int kEpiThreads = 256;
+using sl::kEpiGroups;
+using sl::kEpiThreads;
+using sl::kMmaWarp;
+using sl::kThreads;
 constexpr int kMaxKSteps = 6;      // K <= 96
 constexpr int kPartMax = 48;       // pair columns per part
 constexpr int kLevels = 5;         // accumulators per element
@@ -130,18 +136,16 @@ __device__ __forceinline__ long long levels_to_int5(uint32_t r0, uint32_t r1, ui
     const int h = __float_as_int(t) - MB;
     const float rem = fmaf(-(t - M), 0x1p-18f, a4);  // exact: a4 - h 2^-18
     const int l = __float_as_int(fmaf(rem, 0x1p34f, M)) - MB;
-    if (neg) {
-        hi = -hi;
-        mid = -mid;
-    }
+    const int sg = -(int)neg;  // negate without a branch
+    hi = (hi ^ sg) - sg;
+    mid = (mid ^ sg) - sg;
     return ((long long)hi << 26) + ((long long)mid << 10) + ((long long)h << 16) + l;
 }
 
 template <int KPAD, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_sigma_wide(const uint2 *__restrict__ cs0123, const uint32_t *__restrict__ cs45,
-                 unsigned long long *__restrict__ acc, SpinTables R, int64_t ncols, const uint32_t *__restrict__ tabp,
-                 const long long *__restrict__ XT, int npair, int npad, int nparts, int shq, int *err) {
+    k_sigma_wide(const uint16_t *__restrict__ planes, int64_t pitch, unsigned long long *__restrict__ acc, SpinTables R,
+                 int64_t ncols, const uint32_t *__restrict__ tabp, const long long *__restrict__ XT, int npair, int npad, int nparts, int shq, int *err) {
     constexpr int NKS = KPAD / 16;
     constexpr int kgroups = KPAD / 8;
     constexpr uint32_t sbo = (uint32_t)(KPAD / 8) * 128u;
@@ -161,7 +165,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto acc_full = [&](int b) { return bar0 + 8u * (uint32_t)(2 * kMaxKSteps + b); };
     auto acc_empty = [&](int b) { return bar0 + 8u * (uint32_t)(2 * kMaxKSteps + 2 + b); };
     const uint32_t drain = bar0 + 8u * (uint32_t)(2 * kMaxKSteps + 4);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);  // uniform: role branches do not diverge
+    const bool elected = tc::elect_one();  // the MMA warp's issuing lane (one lane issues and commits)
     const int nq = MODE == 1 ? npair + 1 : npair;  // rows of XT
 
     if (warp == 0) {
@@ -182,6 +188,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::mbar_init(drain, 1);
         *s_fail = 0;
     }
+    for (uint32_t i = (uint32_t)tid * 16u; i < kSlices * L.bytesA; i += kThreads * 16u)  // padded replacements stay zero
+        *reinterpret_cast<uint4 *>(sA + i) = make_uint4(0u, 0u, 0u, 0u);
+    tc::fence_async_smem();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -227,10 +236,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 *reinterpret_cast<uint4 *>(sB + tc::kmajor_offset(s * np + ql, kg, KPAD)) =
                     make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
         }
-        if (warp >= 4 && warp < 12) {  // starting words of both buffers in this item's layout
+        if (warp >= 4 && warp < kMmaWarp) {  // starting words of both buffers in this item's layout
             const uint32_t lb = tmem + ((uint32_t)((warp & 3) * 32) << 16);
             for (int b = 0; b < 2; ++b)
-                for (int c = (warp - 4) >> 2; c < np / 8; c += 2) init_chunk(lb, b, np, c);
+                for (int c = (warp - 4) >> 2; c < np / 8; c += kEpiGroups) init_chunk(lb, b, np, c);
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         }
         tc::fence_async_smem();
@@ -239,67 +248,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::fence_after();
 
         if (warp < 4) {
-            // ---- producers: column string 128 t + m, one K-group (8 values) at a
-            // time, the next group's loads in flight while this one is transposed ----
-            const int m = tid;
-            uint32_t cx[8], cy[8], cz[8], nx[8], ny[8], nz[8];
-            auto load = [&](uint32_t(&x)[8], uint32_t(&y)[8], uint32_t(&z)[8], int64_t jb, int kg) {
-                const int64_t jc = jb < ncols ? jb : ncols - 1;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int a = kg * 8 + i;
-                    const int64_t idx = (int64_t)ent_target(sEa[a < sa_n ? a : 0]) * ncols + jc;
-                    sl::ld_early_v2(cs0123 + idx, x[i], y[i]);
-                    z[i] = tc::ld_early_u32(cs45 + idx);
-                }
-            };
-            load(cx, cy, cz, m, 0);
+            // ---- producers ----
             for (int64_t t = 0; t < ntiles && !*s_fail; ++t) {
                 const int64_t Tt = T + t;
-                const int64_t jb = t * kM + m;
-                const bool live = jb < ncols;
-#pragma unroll
-                for (int ks = 0; ks < NKS; ++ks) {
-                    if (Tt >= 1 && !tc::mbar_wait_bounded(a_free(ks), (uint32_t)((Tt - 1) & 1))) {
-                        *s_fail = 1;
-                        break;
-                    }
-#pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        const int kg = 2 * ks + g;
-                        if (kg + 1 < kgroups)
-                            load(nx, ny, nz, jb, kg + 1);
-                        else if (t + 1 < ntiles)
-                            load(nx, ny, nz, jb + kM, 0);
-                        if (!live || kg * 8 + 8 > sa_n) {  // dead lane or padded replacements
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                if (!(live && kg * 8 + i < sa_n)) cx[i] = cy[i] = cz[i] = 0u;
-                        }
-                        const uint32_t off = tc::kmajor_offset(m, kg, KPAD);
-#pragma unroll
-                        for (int s = 0; s < kSlices; ++s) {
-                            uint32_t o[4];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const uint32_t x0 = s < 2 ? cx[2 * i] : s < 4 ? cy[2 * i] : cz[2 * i];
-                                const uint32_t x1 = s < 2 ? cx[2 * i + 1] : s < 4 ? cy[2 * i + 1] : cz[2 * i + 1];
-                                o[i] = __byte_perm(x0, x1, (s & 1) ? 0x7632 : 0x5410);
-                            }
-                            *reinterpret_cast<uint4 *>(sA + (uint32_t)s * L.bytesA + off) = make_uint4(o[0], o[1], o[2], o[3]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            cx[i] = nx[i];
-                            cy[i] = ny[i];
-                            cz[i] = nz[i];
-                        }
-                    }
-                    tc::fence_async_smem();
-                    tc::mbar_arrive(a_full(ks));
-                }
+                if (!sl::produce_tile<KPAD>(planes + t * kM, pitch, R.ns * pitch, sEa, sa_n, tc::smem_u32(sA),
+                                            L.bytesA, tid, Tt == 0, (uint32_t)((Tt - 1) & 1), a_full, a_free))
+                    *s_fail = 1;
             }
-        } else if (warp < 12) {
+        } else if (warp < kMmaWarp) {
             // ---- epilogue: lane m of the tile, 8-column chunks grp, grp + 2, ... ----
             const int quarter = warp & 3, grp = (warp - 4) >> 2;
             const int m = quarter * 32 + lane;
@@ -332,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tc::fence_before();
                     tc::mbar_arrive(acc_empty(b));
                 }
-                for (int c = grp; c < nch; c += 2) {
+                for (int c = grp; c < nch; c += kEpiGroups) {
                     uint32_t r[kLevels][8];
 #pragma unroll
                     for (int lv = 0; lv < kLevels; ++lv)
@@ -342,43 +298,49 @@ __global__ void __launch_bounds__(kThreads, 1)
                                      : "r"(lane_base + acc_col(b, lv, np) + (uint32_t)(c * 8)));
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     init_chunk(lane_base, b, np, c);  // the next use of this buffer starts from these
-                    if (c + 2 >= nch) {  // last chunk of this thread: release the buffer
+                    if (c + kEpiGroups >= nch) {  // last chunk of this thread: release the buffer
                         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                         tc::fence_before();
                         tc::mbar_arrive(acc_empty(b));
                     }
                     const uint32_t ew[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
-                    if (c + 2 < nch) fetch(c + 2, e0, e1);
+                    if (c + kEpiGroups < nch) fetch(c + kEpiGroups, e0, e1);
                     if (!live) continue;
+                    long long v[8];  // every column converted (ILP over the eight), then the adds
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const uint32_t en = MODE == 0 ? ew[j] : sPair[q0 + c * 8 + j];
-                        if (en == kNoEntry) continue;
-                        range_bad |= (r[3][j] >> 23) ^ (kBias3 >> 23);  // level 3 left its binade
-                        long long v = levels_to_int5(r[0][j], r[1][j], r[2][j], r[3][j], r[4][j], en >> 31);
-                        if (MODE == 0 || q0 + c * 8 + j == npair) v *= 1ll << shq;
+                        // level 3 left its binade (only entries that are used count)
+                        range_bad |= en == kNoEntry ? 0u : (r[3][j] >> 23) ^ (kBias3 >> 23);
+                        v[j] = levels_to_int5(r[0][j], r[1][j], r[2][j], r[3][j], r[4][j], en >> 31);
+                        if (MODE == 0 || q0 + c * 8 + j == npair) v[j] *= 1ll << shq;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t en = MODE == 0 ? ew[j] : sPair[q0 + c * 8 + j];
                         const int64_t o = MODE == 0 ? row * ncols + (int64_t)ent_target(en)
                                                     : (int64_t)ent_target(en) * ncols + jb;
-                        atomicAdd(acc + o, (unsigned long long)v);
+                        if (en != kNoEntry) atomicAdd(acc + o, (unsigned long long)v[j]);
                     }
                 }
                 if (*s_fail) break;
             }
             if (range_bad) atomicOr(err, 2);
-        } else if (warp == 12 && lane == 0) {
-            // ---- MMA issuer: descriptors of K-step 0, advanced by 256 bytes (16 in
-            // the address field) per K-step ----
+        } else if (warp == kMmaWarp) {
+            // ---- MMA issuer: descriptors of K-step 0, advanced per K-step by 2048
+            // bytes of A (two atoms) and 256 of B ----
             // A slice s: levels s..4 from B slices 0..4-s (stacked, one MMA of
             // N = (5 - s) np), then B slice 5 - s into level 4 (N = np)
+            const bool issue = elected;
             uint64_t ad[kSlices], bd[kSlices];
 #pragma unroll
             for (int s = 0; s < kSlices; ++s) {
-                ad[s] = tc::smem_desc(tc::smem_u32(sA + s * L.bytesA), 128, sbo);
+                ad[s] = sl::smem_desc_mn(tc::smem_u32(sA + s * L.bytesA), KPAD * 128, 1024);
                 bd[s] = tc::smem_desc(tc::smem_u32(sB) + (uint32_t)(s * np / 8) * sbo, 128, sbo);
             }
             uint32_t idn[5];
 #pragma unroll
-            for (int k = 0; k < 5; ++k) idn[k] = tc::instr_desc(kM, (k + 1) * np);
+            for (int k = 0; k < 5; ++k) idn[k] = tc::instr_desc(kM, (k + 1) * np) | sl::kTransposeA;
             for (int64_t t = 0; t < ntiles; ++t) {
                 const int64_t Tt = T + t;
                 const int b = (int)(Tt & 1);
@@ -388,9 +350,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (ok && !tc::mbar_wait_bounded(a_full(ks), (uint32_t)(Tt & 1))) ok = false;
                     if (!ok) break;
                     tc::fence_after();
+                    if (!issue) continue;
 #pragma unroll
                     for (int sa = 0; sa < kSlices; ++sa) {
-                        const uint64_t a = ad[sa] + (uint64_t)(ks * 16);
+                        const uint64_t a = ad[sa] + (uint64_t)(ks * 128);
                         if (sa < 5)
                             tc::mma_bf16(tmem + acc_col(b, sa, np), a, bd[0] + (uint64_t)(ks * 16), idn[4 - sa], 1u);
                         tc::mma_bf16(tmem + acc_col(b, 4, np), a, bd[5 - sa] + (uint64_t)(ks * 16), idn[0], 1u);
@@ -401,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     *s_fail = 1;
                     break;
                 }
-                tc::mma_commit(acc_full(b));
+                if (issue) tc::mma_commit(acc_full(b));
             }
         }
         // ---- item end: every MMA of the item has been read by the epilogue ----
@@ -412,8 +375,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (*s_fail) break;
     }
     // ---- exit: wait for every MMA this CTA issued, then free tensor memory ----
-    if (warp == 12 && lane == 0) {
-        tc::mma_commit(drain);
+    if (warp == kMmaWarp) {
+        if (elected) tc::mma_commit(drain);
         if (!tc::mbar_wait_bounded(drain, 0u)) *s_fail = 1;
     }
     tc::fence_before();
