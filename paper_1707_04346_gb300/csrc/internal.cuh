@@ -82,6 +82,17 @@ struct SpinTables {
     bool owner = true;         // false when aliasing the alpha tables
 };
 
+// Digit planes of one spin's G_s (sigma_ss.cu): blocks of nb rows, each with the
+// K-steps that hold a nonzero.
+struct SsOperand {
+    unsigned char *planes = nullptr;
+    size_t plane_bytes = 0;
+    int *lists = nullptr;  // offsets [nnb + 1] into the K-step list, K-steps
+    size_t list_bytes = 0;
+    int *e = nullptr;      // biased exponent of each row
+    int nb = 0, nnb = 0;
+};
+
 }  // namespace fci
 
 struct fci_ctx {
@@ -114,12 +125,11 @@ struct fci_ctx {
     int sh1 = 0;
     int *d_eG = nullptr;            // device: largest biased exponent of C
     long long *wsacc = nullptr;     // [ndet] when ws32 is absent
-    // FP64 same-spin terms as dense sliced products (sigma_ss.cu): digit planes
-    // of each spin's same-spin Hamiltonian G_s with per-row exponents (the
-    // beta ones alias the alpha ones when both spins share one string space),
-    // and the per-call planes of C by rows and by columns with their exponents
-    unsigned char *ssG_a = nullptr, *ssG_b = nullptr;
-    int *ssE_a = nullptr, *ssE_b = nullptr;
+    // FP64 same-spin terms as dense sliced products (sigma_ss.cu): each spin's
+    // same-spin Hamiltonian G_s (beta aliases alpha when both spins share one
+    // string space), and the per-call planes of C by rows and by columns with
+    // their exponents
+    fci::SsOperand ssGa, ssGb;
     unsigned char *ssCr = nullptr, *ssCc = nullptr;
     int *ssEr = nullptr, *ssEc = nullptr;
     double *hdiag = nullptr;        // [ndet]

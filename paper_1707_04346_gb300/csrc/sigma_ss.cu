@@ -18,16 +18,42 @@
 // integers every 256 terms, and at the end one FP64 conversion per element
 // with the two scales of its row and column.
 //
-// One kernel computes out[n ldo + m] += sum_k A(m, k) B(n, k) for two plane
-// sets A (rows m, the MMA's M: 128 per tile) and B (rows n: 48 per tile), each
+// One kernel computes out(m, n) += sum_k A(m, k) B(n, k) for a plane set A of C
+// (rows m, the MMA's M: 128 per tile) and one B of G (rows n: NB per tile), each
 // row with its own exponent:
-//   sigma_1: A = G_b (m = I_b), B = C by rows (n = I_a, k = J_b);
-//   sigma_2: A = C by columns (m = I_b, k = J_a), B = G_a (n = I_a);
-// both write sigma(I_a, I_b) at I_a n_b + I_b, consecutive across the lanes of
-// a warp.  Plane sets are laid out like the 2-RDM's digit planes: per K-step
-// of 16, six planes of rows x 16 bf16 in the K-major no-swizzle core-matrix
-// layout; rows padded to a multiple of 384 (both tile heights), K to 16.
+//   sigma_1: A = C by rows (m = I_a, k = J_b), B = G_b (n = I_b);
+//   sigma_2: A = C by columns (m = I_b, k = J_a), B = G_a (n = I_a); its epilogue
+//            also applies the FP64 diagonal of both spins.
+// Layout: an operand tile (six digit planes of its rows x 16 columns in the
+// K-major no-swizzle core-matrix layout) is contiguous, so that one bulk copy
+// stages it: A [K-step][128-row block][6][4 KB], B [row block][K-step][6][32 NB].
+// (An SM issues a bulk copy about every 100 cycles whatever its size, and the
+// twelve copies of 1.5 to 4 KB per K-step of a plane-by-plane layout were the
+// 1190 cycles that a K-step of 48 columns took.)
+// G_s between strings that differ by more than two replacements is zero, and
+// strings in address order share their high orbitals: of the K-steps of a
+// 96-row block of G, 12 % (CAS(14,14)) and 34 % (CAS(16,16)) hold only zeros.
+// B keeps the others, with their list per block; rows of G as the narrow side
+// of the tile skip more than as the 128-row side.
+// NB = 96 where the tiles fill the chip: the digit products run as MMAs of N =
+// 192 (two digits stacked along N, writing two neighbouring weights) or 96;
+// 575 cycles per K-step and 48 columns against 730 to 800 for NB = 48 (an M =
+// 128 MMA reads its 4 KB of A each time, so narrow ones wait for shared
+// memory).  The five accumulators of 96 columns fill tensor memory once, so
+// the next flush group cannot simply alternate buffers: the epilogue releases
+// weight by weight, last first, and the first three K-steps of a group are
+// issued weight by weight in that order (the eleven products of weights 4 and
+// 5 first), which hides the read-out.  NB = 16 for small spaces, where 96-row
+// tiles would leave most SMs idle.
 // G_s's planes are built once at fci_init; C's two plane sets per call.
+//
+// sigma_1 + sigma_2 with their passes over C: CAS(14,14) 3.74 -> 2.59 ms,
+// CAS(16,16) 179 -> 82 ms.  At CAS(16,16) the product runs at 1500 TFLOP/s of
+// executed MMA work (cuBLAS sustains 1705 there, at the power cap); at CAS(14,14)
+// its 972 tiles are 6.4 waves of 152.
+#include <algorithm>
+#include <vector>
+
 #include "sliced_mma.cuh"
 
 namespace fci {
@@ -36,38 +62,38 @@ namespace ss {
 using sl::kSlices;
 using tc::kM;
 using sm::bulk_g2s;
-using sm::levels_to_int_f;
 using sm::mbar_expect_tx;
 
-constexpr int kThreads = 448;        // warp 0 copies, warp 1 issues the MMAs, warps 2-13 epilogue
-constexpr int kEpiThreads = 384;
-constexpr int kBN = 48;              // B rows per tile
-constexpr int kStages = 6;           // K-steps of operands in flight
 constexpr int kKTile = 16;           // K-steps (256 terms) per accumulator flush
-constexpr int kRowPad = 384;         // plane rows: a multiple of 128 and of 48
+constexpr int kLead = 3;             // K-steps of a flush group issued weight by weight
+constexpr int kLevels = 5;
 constexpr int kF = 34;               // integer unit 2^-34 of the accumulator scale
 constexpr uint32_t kBytesA = 6 * 4096;
-constexpr uint32_t kBytesB = 6 * kBN * 32;
-constexpr uint32_t kStageBytes = kBytesA + kBytesB;
-constexpr int kBars = 2 * kStages + 5;
-constexpr uint32_t kSmem = kStages * kStageBytes + kBars * 8 + 16;
 
-inline int64_t pad_rows(int64_t r) { return (r + kRowPad - 1) / kRowPad * kRowPad; }
-inline size_t plane_bytes(int64_t rows, int64_t k) { return (size_t)((k + 15) / 16) * 6 * pad_rows(rows) * 32; }
+// Tile shape of NB rows of G: stages of operands in flight, epilogue warps per
+// lane quarter, weights per MMA (N = kWide NB <= 256), tensor-memory columns.
+template <int NB>
+struct Shape {
+    static constexpr uint32_t kBytesB = 6 * NB * 32;
+    static constexpr uint32_t kStageBytes = kBytesA + kBytesB;
+    static constexpr int kStages = NB == 96 ? 5 : 8;
+    static constexpr int kSub = NB == 96 ? 3 : 1;
+    static constexpr int kCols = NB / kSub;  // columns per epilogue thread
+    static constexpr int kWide = NB == 96 ? 2 : 5;
+    static constexpr int kEpiThreads = 128 * kSub;
+    static constexpr int kThreads = 64 + kEpiThreads;  // warp 0 copies, warp 1 issues the MMAs
+    static constexpr uint32_t kTmem = NB == 96 ? 512 : 128;
+    static constexpr int kBars = 2 * kStages + 1 + kLevels + 1;  // full, free, acc_full, acc_empty[level], drain
+    static constexpr uint32_t kSmem = kStages * kStageBytes + kBars * 8 + 16;
+};
 
-// six digits of X into the planes at (row r, column k): plane t of K-step k/16
-// at byte ((k/16) 6 + t) rows_pad 32, then the core-matrix offset of (r, k%16)
-__device__ __forceinline__ void put_digits(unsigned char *planes, int64_t rows_pad, int64_t r, int64_t k, long long X) {
-    float f[kSlices];
-    sl::digits6(X, f);
-    const int64_t ks = k >> 4;
-    const int kk = (int)(k & 15);
-    const uint32_t off = (uint32_t)((r >> 3) * 256 + (kk >> 3) * 128 + (r & 7) * 16 + (kk & 7) * 2);
-#pragma unroll
-    for (int t = 0; t < kSlices; ++t) {
-        const __nv_bfloat16 b = __float2bfloat16_rn(f[t]);  // exact: an 8-bit integer times a power of two
-        *reinterpret_cast<__nv_bfloat16 *>(planes + ((size_t)ks * 6 + t) * rows_pad * 32 + off) = b;
-    }
+inline int64_t nblocks(int64_t rows, int nb) { return (rows + nb - 1) / nb; }
+inline int64_t ksteps(int64_t k) { return (k + 15) / 16; }
+inline size_t c_bytes(int64_t rows, int64_t k) { return (size_t)ksteps(k) * nblocks(rows, kM) * kBytesA; }
+
+// byte offset of (row r, column kk) of a K-step inside one plane of a tile
+__device__ __forceinline__ uint32_t core_offset(int r, int kk) {
+    return (uint32_t)((r >> 3) * 256 + (kk >> 3) * 128 + (r & 7) * 16 + (kk & 7) * 2);
 }
 
 __device__ __forceinline__ long long fixed46(double x, int emax) {
@@ -86,16 +112,34 @@ __global__ void k_ss_rowexp(const double *__restrict__ gval, int64_t ns, int nsa
     e[x] = (int)m;
 }
 
-// dense G planes: every off-diagonal ELL entry (row x, column gcol, value
-// gval) scattered (each row's columns are distinct; the planes start at zero)
-__global__ void k_ss_gplanes(const int32_t *__restrict__ gcol, const double *__restrict__ gval, int64_t ns, int nsame,
-                             const int *__restrict__ e, int64_t rows_pad, unsigned char *__restrict__ planes) {
+// used[nb * nks + ks] = 1 for every K-step of every block of NB rows that holds
+// an off-diagonal nonzero
+__global__ void k_ss_used(const int32_t *__restrict__ gcol, const double *__restrict__ gval, int64_t ns, int nsame,
+                          int NB, int64_t nks, unsigned char *__restrict__ used) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < ns || t >= ns * (int64_t)nsame) return;  // slot 0 (t < ns): the diagonal
+    if (gval[t] != 0.0) used[(t % ns) / NB * nks + (gcol[t] >> 4)] = 1;
+}
+
+// G planes: every off-diagonal ELL entry (row x, column gcol, value gval)
+// scattered into the kept K-step slot[nb * nks + ks] (each row's columns are
+// distinct; the planes start at zero)
+__global__ void k_ss_gplanes(const int32_t *__restrict__ gcol, const double *__restrict__ gval, int64_t ns, int nsame,
+                             const int *__restrict__ e, int NB, int64_t nks, const int *__restrict__ slot,
+                             unsigned char *__restrict__ planes) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < ns || t >= ns * (int64_t)nsame) return;
     const int64_t x = t % ns;
     const double v = gval[t];
     if (v == 0.0) return;
-    put_digits(planes, rows_pad, x, gcol[t], fixed46(v, e[x]));
+    const int col = gcol[t];
+    float f[kSlices];
+    sl::digits6(fixed46(v, e[x]), f);
+    unsigned char *tile = planes + (size_t)slot[x / NB * nks + (col >> 4)] * 6 * NB * 32;
+    const uint32_t off = core_offset((int)(x % NB), col & 15);
+#pragma unroll
+    for (int s = 0; s < kSlices; ++s)  // exact: an 8-bit integer times a power of two
+        *reinterpret_cast<__nv_bfloat16 *>(tile + s * NB * 32 + off) = __float2bfloat16_rn(f[s]);
 }
 
 // largest biased exponent of each row (erow) and each column (ecol) of the
@@ -126,86 +170,106 @@ __global__ void k_ss_cexp(const double *__restrict__ C, int64_t nrows, int64_t n
     }
 }
 
-// C's planes by rows (row i of the planes = row i of C, k = column) or by
-// columns (row j of the planes = column j of C, k = row of C): one thread per
-// (plane row, 8 consecutive k), 16-byte stores of each digit plane
-__global__ void k_ss_cplanes(const double *__restrict__ C, int64_t nrows, int64_t ncols, int cols,
-                             const int *__restrict__ e, int64_t rows_pad, unsigned char *__restrict__ planes) {
-    const int64_t prow_n = cols ? ncols : nrows, klen = cols ? nrows : ncols;
-    const int64_t groups = (klen + 7) / 8;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= prow_n * groups) return;
-    // cols: consecutive threads take consecutive plane rows (consecutive C columns: coalesced reads)
-    const int64_t r = cols ? t % prow_n : t / groups, g = cols ? t / prow_n : t % groups;
-    const int er = e[r];
-    uint32_t w[kSlices][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float f0[kSlices], f1[kSlices];
-        const int64_t k0 = g * 8 + 2 * i, k1 = k0 + 1;
-        const double v0 = k0 < klen ? (cols ? C[k0 * ncols + r] : C[r * ncols + k0]) : 0.0;
-        const double v1 = k1 < klen ? (cols ? C[k1 * ncols + r] : C[r * ncols + k1]) : 0.0;
-        sl::digits6(fixed46(v0, er), f0);
-        sl::digits6(fixed46(v1, er), f1);
-#pragma unroll
-        for (int s = 0; s < kSlices; ++s) w[s][i] = sl::pack_bf16(f0[s], f1[s]);
+// C's planes by rows (plane row = row of C, k = column; nullptr: not wanted) and
+// by columns (plane row = column of C, k = row), both from one read of a 64 x 64
+// tile of C through shared memory; 8 threads write the 128 bytes of 8 rows' core
+// matrix.  Rows past the matrix are written as zeros up to the end of a 64-row
+// tile (the planes' padding beyond starts at zero), columns past it as zeros.
+__global__ void __launch_bounds__(256) k_ss_cplanes(const double *__restrict__ C, int64_t nrows, int64_t ncols,
+                                                    const int *__restrict__ erow, const int *__restrict__ ecol,
+                                                    unsigned char *__restrict__ prow, unsigned char *__restrict__ pcol) {
+    __shared__ double t[64][65];
+    const int64_t c0 = (int64_t)blockIdx.x * 64, r0 = (int64_t)blockIdx.y * 64;
+    for (int i = threadIdx.x; i < 64 * 64; i += 256) {
+        const int64_t r = r0 + (i >> 6), c = c0 + (i & 63);
+        t[i >> 6][i & 63] = (r < nrows && c < ncols) ? C[r * ncols + c] : 0.0;
     }
-    const int64_t ks = g >> 1;
-    const uint32_t off = (uint32_t)((r >> 3) * 256 + (g & 1) * 128 + (r & 7) * 16);
+    __syncthreads();
+    for (int it = threadIdx.x; it < 1024; it += 256) {
+        const bool cols = it >= 512;
+        unsigned char *planes = cols ? pcol : prow;
+        if (planes == nullptr) continue;
+        const int x = it & 63, g = (it >> 6) & 7;  // plane row of the tile, group of 8 k
+        const int64_t r = (cols ? c0 : r0) + x, k0 = (cols ? r0 : c0) + g * 8;
+        const int64_t rows = cols ? ncols : nrows, klen = cols ? nrows : ncols;
+        if (k0 >= (klen + 15) / 16 * 16) continue;
+        const int e = r < rows ? (cols ? ecol[r] : erow[r]) : 0;
+        uint32_t w[kSlices][4];
 #pragma unroll
-    for (int s = 0; s < kSlices; ++s)
-        *reinterpret_cast<uint4 *>(planes + ((size_t)ks * 6 + s) * rows_pad * 32 + off) =
-            make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
-}
-
-// sigma(I_a, I_b) += (G_a(I_a, I_a) + G_b(I_b, I_b)) C(I_a, I_b) in FP64 (the
-// diagonal of the same-spin Hamiltonians, ELL slot 0; a null da or db leaves
-// that spin out)
-__global__ void k_ss_diag(const double *__restrict__ C, double *__restrict__ sig, const double *__restrict__ da,
-                          const double *__restrict__ db, int64_t nsa, int64_t nsb) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nsa * nsb; i += stride) {
-        const int64_t ia = i / nsb, ib = i - ia * nsb;
-        const double d = (da ? da[ia] : 0.0) + (db ? db[ib] : 0.0);
-        sig[i] = fma(d, C[i], sig[i]);
+        for (int i = 0; i < 4; ++i) {
+            float f0[kSlices], f1[kSlices];
+            const int k = g * 8 + 2 * i;
+            sl::digits6(fixed46(cols ? t[k][x] : t[x][k], e), f0);
+            sl::digits6(fixed46(cols ? t[k + 1][x] : t[x][k + 1], e), f1);
+#pragma unroll
+            for (int s = 0; s < kSlices; ++s) w[s][i] = sl::pack_bf16(f0[s], f1[s]);
+        }
+        unsigned char *tile = planes + ((size_t)(k0 >> 4) * ((rows + kM - 1) / kM) + (r >> 7)) * kBytesA;
+        const uint32_t off = core_offset((int)(r & 127), (int)(k0 & 15));
+#pragma unroll
+        for (int s = 0; s < kSlices; ++s)
+            *reinterpret_cast<uint4 *>(tile + s * 4096 + off) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
     }
 }
 
 struct SsArgs {
     const unsigned char *A, *B;  // plane sets
-    int64_t rowsA, rowsB;        // padded plane rows
+    const int *koff, *kidx;      // K-steps of row block nb of B: kidx[koff[nb] .. koff[nb + 1])
     int M, N;                    // rows of A (output lanes) and of B (output columns) in use
-    int64_t nks;                 // K-steps
     const int *eA, *eB;          // biased exponent of each row
     double *out;
-    int64_t ldo;                 // out[n ldo + m] +=
+    int64_t sm, sn;              // out[m sm + n sn] +=
+    const double *C;             // with it, out += (dn[n] + dm[m]) C at the same place first (dm may be null)
+    const double *dn, *dm;
     int *err;
 };
 
-// Tiles: 128 rows of A x 48 rows of B, t = nb * nmb + mb; CTA b takes tiles
+// value = V 2^(eA + eB - 12 - f), eA/eB the unbiased exponents of the row maxima
+// (given biased); a non-finite operand row (exponent 0x7FF) gives NaN
+__device__ __forceinline__ double element(long long V, int ea, int eb) {
+    if (ea == 0x7FF || eb == 0x7FF) return __longlong_as_double(0x7FF8000000000000ll);
+    return sl::scaled_i64(V, (ea - 1022) + (eb - 1022) - 12 - kF);
+}
+
+// The integer i of an FP32 value holding i 2^-k exactly, |i| <= 2^24, as
+// 4 h + r with h = round(i / 4): both from magic-number additions, which are
+// exact up to 2^22; no conversion instructions.
+__device__ __forceinline__ int exact_int(float v, float quarter_scale, float unit) {
+    constexpr float M = 12582912.0f;  // 1.5 2^23
+    constexpr int MB = 0x4B400000;
+    const float t = fmaf(v, quarter_scale, M);          // round(i / 4)
+    const float r = fmaf(-(t - M), 4.0f * unit, v);     // (i - 4 h) 2^-k, exact
+    const float u = fmaf(r, 4.0f * quarter_scale, M);   // i - 4 h
+    return 4 * (__float_as_int(t) - MB) + (__float_as_int(u) - MB);
+}
+
+// Tiles: 128 rows of A x NB rows of B, t = nb * nmb + mb; CTA b takes tiles
 // b, b + grid, ...  (the CTAs of one wave share A and B K-steps through L2,
 // advancing through K at one rate).
-__global__ void __launch_bounds__(kThreads, 1) k_ss_tc(SsArgs P) {
+template <int NB>
+__global__ void __launch_bounds__(Shape<NB>::kThreads, 1) k_ss_tc(SsArgs P) {
+    using S = Shape<NB>;
+    constexpr int kStages = S::kStages;
     extern __shared__ __align__(1024) unsigned char smem[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
-    volatile int *s_fail = reinterpret_cast<volatile int *>(smem + kStages * kStageBytes + kBars * 8);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + kStages * kStageBytes + kBars * 8 + 4);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * S::kStageBytes);
+    volatile int *s_fail = reinterpret_cast<volatile int *>(smem + kStages * S::kStageBytes + S::kBars * 8);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + kStages * S::kStageBytes + S::kBars * 8 + 4);
     const uint32_t sbase = tc::smem_u32(smem);
     const uint32_t bar0 = tc::smem_u32(bars);
     auto full = [&](int st) { return bar0 + 8u * (uint32_t)st; };
     auto freeb = [&](int st) { return bar0 + 8u * (uint32_t)(kStages + st); };
-    auto acc_full = [&](int b) { return bar0 + 8u * (uint32_t)(2 * kStages + b); };
-    auto acc_empty = [&](int b) { return bar0 + 8u * (uint32_t)(2 * kStages + 2 + b); };
-    const uint32_t drain = bar0 + 8u * (uint32_t)(2 * kStages + 4);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nmb = (P.M + 127) / 128, nnb = (P.N + kBN - 1) / kBN;
+    const uint32_t acc_full = bar0 + 8u * (uint32_t)(2 * kStages);
+    auto acc_empty = [&](int lv) { return bar0 + 8u * (uint32_t)(2 * kStages + 1 + lv); };
+    const uint32_t drain = bar0 + 8u * (uint32_t)(2 * kStages + 1 + kLevels);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    const bool elected = tc::elect_one();
+    const int nmb = (P.M + 127) / 128, nnb = (P.N + NB - 1) / NB;
     const int ntiles = nmb * nnb;
 
-    for (uint32_t i = (uint32_t)tid * 16u; i < kStages * kStageBytes; i += kThreads * 16u)
-        *reinterpret_cast<uint4 *>(smem + i) = make_uint4(0u, 0u, 0u, 0u);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(tslot)),
-                     "r"(512)
+                     "r"(S::kTmem)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -214,14 +278,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ss_tc(SsArgs P) {
             tc::mbar_init(full(i), 1);
             tc::mbar_init(freeb(i), 1);
         }
-        for (int b = 0; b < 2; ++b) {
-            tc::mbar_init(acc_full(b), 1);
-            tc::mbar_init(acc_empty(b), kEpiThreads);
-        }
+        tc::mbar_init(acc_full, 1);
+        for (int lv = 0; lv < kLevels; ++lv) tc::mbar_init(acc_empty(lv), S::kEpiThreads);
         tc::mbar_init(drain, 1);
         *s_fail = 0;
     }
-    tc::fence_async_smem();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -229,153 +290,205 @@ __global__ void __launch_bounds__(kThreads, 1) k_ss_tc(SsArgs P) {
 
     int64_t G_copied = 0;
     if (warp == 0 && lane == 0) {
-        // ---- copies: the A and B planes of one K-step per stage ----
+        // ---- copies: the A and B tiles of one K-step per stage ----
         int64_t &G = G_copied;
         for (int t = blockIdx.x; t < ntiles && !*s_fail; t += gridDim.x) {
             const int mb = t % nmb, nb = t / nmb;
-            const uint32_t ba = 128u * 32u, bb = (uint32_t)kBN * 32u;  // rows padded: whole tiles
-            for (int64_t ks = 0; ks < P.nks; ++ks, ++G) {
+            const int k1 = __ldg(P.koff + nb + 1);
+            for (int k = __ldg(P.koff + nb); k < k1; ++k, ++G) {
                 const int st = (int)(G % kStages);
+                const size_t ks = (size_t)__ldg(P.kidx + k);
                 if (G >= kStages && !tc::mbar_wait_bounded(freeb(st), (uint32_t)((G / kStages - 1) & 1))) {
                     *s_fail = 1;
                     break;
                 }
-                mbar_expect_tx(full(st), 6u * (ba + bb));
-                const unsigned char *sa = P.A + ((size_t)ks * 6 * P.rowsA + (size_t)mb * 128) * 32;
-                const unsigned char *sb = P.B + ((size_t)ks * 6 * P.rowsB + (size_t)nb * kBN) * 32;
-                const uint32_t dst = sbase + (uint32_t)st * kStageBytes;
-#pragma unroll
-                for (int p = 0; p < 6; ++p) {
-                    bulk_g2s(dst + (uint32_t)p * 4096u, sa + (size_t)p * P.rowsA * 32, ba, full(st));
-                    bulk_g2s(dst + kBytesA + (uint32_t)p * kBN * 32u, sb + (size_t)p * P.rowsB * 32, bb, full(st));
-                }
+                mbar_expect_tx(full(st), S::kStageBytes);
+                const uint32_t dst = sbase + (uint32_t)st * S::kStageBytes;
+                bulk_g2s(dst, P.A + (ks * nmb + mb) * kBytesA, kBytesA, full(st));
+                bulk_g2s(dst + kBytesA, P.B + (size_t)k * S::kBytesB, S::kBytesB, full(st));
             }
         }
-    } else if (warp == 1 && lane == 0) {
-        // ---- MMAs: A digit s times the stacked B digits 0..4-s into weights
-        // s..4 (N = (5 - s) 48), then B digit 5 - s into weight 4 ----
-        uint64_t ad[kSlices], bd[kSlices];
-#pragma unroll
-        for (int s = 0; s < kSlices; ++s) {
-            ad[s] = tc::smem_desc(sbase + (uint32_t)s * 4096u, 128, 256);
-            bd[s] = tc::smem_desc(sbase + kBytesA + (uint32_t)s * kBN * 32u, 128, 256);
-        }
-        uint32_t idn[5];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) idn[k] = tc::instr_desc(kM, (k + 1) * kBN);
+    } else if (warp == 1) {
+        // ---- MMAs (all lanes run the loop, the elected one issues) ----
+        const uint64_t a0 = tc::smem_desc(sbase, 128, 256), b0 = tc::smem_desc(sbase + kBytesA, 128, 256);
+        auto A = [&](int st, int s) { return a0 + (uint64_t)((st * S::kStageBytes + s * 4096) >> 4); };
+        auto B = [&](int st, int d) { return b0 + (uint64_t)((st * S::kStageBytes + d * NB * 32) >> 4); };
         int64_t G = 0, Tt = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
-            for (int64_t kt = 0; kt < P.nks && ok; kt += kKTile, ++Tt) {
-                const int b = (int)(Tt & 1);
-                if (Tt >= 2 && !tc::mbar_wait_bounded(acc_empty(b), (uint32_t)(((Tt - 2) >> 1) & 1))) {
-                    ok = false;
-                    break;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+            const int nb = t / nmb;
+            const int nk = __ldg(P.koff + nb + 1) - __ldg(P.koff + nb);
+            for (int kt = 0; kt < nk && ok; kt += kKTile, ++Tt) {
+                const int ke = min(nk - kt, kKTile), lead = min(ke, kLead);
+                // the first K-steps of the group weight by weight, as the epilogue
+                // releases the accumulators of the group before (weights 4 and 5
+                // share one); each accumulator's first MMA overwrites it
+#pragma unroll
+                for (int lv = kLevels - 1; lv >= 0; --lv) {
+                    if (ok && Tt >= 1 && !tc::mbar_wait_bounded(acc_empty(lv), (uint32_t)((Tt - 1) & 1))) ok = false;
+                    for (int j = 0; j < lead && ok; ++j) {
+                        const int st = (int)((G + j) % kStages);
+                        if (lv == kLevels - 1 &&
+                            !tc::mbar_wait_bounded(full(st), (uint32_t)(((G + j) / kStages) & 1))) {
+                            ok = false;
+                            break;
+                        }
+                        tc::fence_after();
+                        if (!elected) continue;
+#pragma unroll
+                        for (int s = 0; s < kSlices; ++s) {
+                            if (s <= lv)
+                                tc::mma_bf16(tmem + lv * NB, A(st, s), B(st, lv - s), tc::instr_desc(kM, NB),
+                                             (j == 0 && s == 0) ? 0u : 1u);
+                            if (lv == kLevels - 1)
+                                tc::mma_bf16(tmem + lv * NB, A(st, s), B(st, 5 - s), tc::instr_desc(kM, NB), 1u);
+                        }
+                        if (lv == 0) tc::mma_commit(freeb(st));
+                    }
                 }
-                tc::fence_after();
-                const int64_t ke = min(P.nks, kt + kKTile);
-                for (int64_t ks = kt; ks < ke; ++ks, ++G) {
+                G += lead;
+                // the others digit by digit of A, kWide weights per MMA
+                for (int j = lead; j < ke && ok; ++j, ++G) {
                     const int st = (int)(G % kStages);
                     if (!tc::mbar_wait_bounded(full(st), (uint32_t)((G / kStages) & 1))) {
                         ok = false;
                         break;
                     }
                     tc::fence_after();
-                    const uint64_t so = (uint64_t)((st * kStageBytes) >> 4);
+                    if (!elected) continue;
 #pragma unroll
-                    for (int sa = 0; sa < kSlices; ++sa) {
-                        // the first MMA of a flush group writes every accumulator column
-                        if (sa < 5)
-                            tc::mma_bf16(tmem + wd::acc_col(b, sa, kBN), ad[sa] + so, bd[0] + so, idn[4 - sa],
-                                         (sa == 0 && ks == kt) ? 0u : 1u);
-                        tc::mma_bf16(tmem + wd::acc_col(b, 4, kBN), ad[sa] + so, bd[5 - sa] + so, idn[0], 1u);
+                    for (int s = 0; s < kSlices; ++s) {
+#pragma unroll
+                        for (int d = 0; d < kSlices; d += S::kWide)
+                            if (s + d < kLevels) {
+                                const int w = kLevels - s - d < S::kWide ? kLevels - s - d : S::kWide;
+                                tc::mma_bf16(tmem + (s + d) * NB, A(st, s), B(st, d), tc::instr_desc(kM, w * NB), 1u);
+                            }
+                        tc::mma_bf16(tmem + (kLevels - 1) * NB, A(st, s), B(st, 5 - s), tc::instr_desc(kM, NB), 1u);
                     }
                     tc::mma_commit(freeb(st));
                 }
-                if (!ok) break;
-                tc::mma_commit(acc_full(b));
+                if (ok && elected) tc::mma_commit(acc_full);
             }
+        }
         if (!ok) *s_fail = 1;
     } else if (warp >= 2) {
-        // ---- epilogue: three warps per lane quarter (warp % 4); lane m of the
-        // tile, columns 16 sub .. 16 sub + 15 read as two groups of 8 ----
+        // ---- epilogue: kSub warps per lane quarter (warp % 4); lane m of the
+        // tile, columns kCols sub .. ----
+        constexpr int kCols = S::kCols;
         const int quarter = warp & 3, sub = (warp - 2) >> 2;
         const int ml = quarter * 32 + lane;
-        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-        const float two_f = __int_as_float((127 + kF) << 23);
-        bool range_bad = false;
+        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(sub * kCols);
+        float top2 = 0.f, top3 = 0.f;
         int64_t Tt = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
             const int mb = t % nmb, nb = t / nmb;
+            const int nk = __ldg(P.koff + nb + 1) - __ldg(P.koff + nb);
             const int m = mb * 128 + ml;
-            long long acc[2][8];
+            long long acc[kCols];
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[h][j] = 0;
-            for (int64_t kt = 0; kt < P.nks; kt += kKTile, ++Tt) {
-                const int b = (int)(Tt & 1);
-                if (!tc::mbar_wait_bounded(acc_full(b), (uint32_t)((Tt >> 1) & 1))) {
+            for (int j = 0; j < kCols; ++j) acc[j] = 0;
+            for (int kt = 0; kt < nk; kt += kKTile, ++Tt) {
+                if (!tc::mbar_wait_bounded(acc_full, (uint32_t)(Tt & 1))) {
                     ok = false;
                     break;
                 }
                 tc::fence_after();
+                // weights 0-3 hold integers in units 2^-8L (|.| <= 2^20, 2^22, 2^23
+                // and 3 2^22: top digits within +-64, others within +-128, 256
+                // terms), weights 4 and 5 FP32 below 2^-6; units of the sum 2^-34
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t r[wd::kLevels][8];
+                for (int lv = kLevels - 1; lv >= 0; --lv)
 #pragma unroll
-                    for (int lv = 0; lv < wd::kLevels; ++lv)
-                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                                     : "=r"(r[lv][0]), "=r"(r[lv][1]), "=r"(r[lv][2]), "=r"(r[lv][3]), "=r"(r[lv][4]),
-                                       "=r"(r[lv][5]), "=r"(r[lv][6]), "=r"(r[lv][7])
-                                     : "r"(lane_base + wd::acc_col(b, lv, kBN) + (uint32_t)(16 * sub + 8 * h)));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (h == 1) {  // the buffer is read: the next flush group may overwrite it
-                        tc::fence_before();
-                        tc::mbar_arrive(acc_empty(b));
-                    }
+                    for (int h = 0; h < kCols; h += 16) {
+                        uint32_t r[16];
+                        asm volatile(
+                            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                              "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+                              "=r"(r[14]), "=r"(r[15])
+                            : "r"(lane_base + (uint32_t)(lv * NB + h)));
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        if (h + 16 >= kCols) {  // this weight is read: the next group may overwrite it
+                            tc::fence_before();
+                            tc::mbar_arrive(acc_empty(lv));
+                        }
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float v2 = __uint_as_float(r[2][j]), v3 = __uint_as_float(r[3][j]);
-                        range_bad |= !(fabsf(v2) <= 256.f) || !(fabsf(v3) <= 1.f);  // |.| <= 2^24 units
-                        acc[h][j] += levels_to_int_f(__uint_as_float(r[0][j]), __uint_as_float(r[1][j]), v2, v3,
-                                                     __uint_as_float(r[4][j]), kF, two_f);
-                    }
-                }
-            }
-            if (!ok) break;
-            if (m < P.M) {
-                const int eam = P.eA[m];
-                const int ea = eam - 1022;
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int n = nb * kBN + 16 * sub + 8 * h + j;
-                        if (n < P.N) {
-                            // value = V 2^(eA + eB - 12 - f), eA/eB the unbiased exponents of the row
-                            // maxima; a non-finite operand row (exponent 0x7FF) gives NaN
-                            const int ebn = P.eB[n];
-                            const double v = (eam == 0x7FF || ebn == 0x7FF)
-                                                 ? __longlong_as_double(0x7FF8000000000000ll)
-                                                 : sl::scaled_i64(acc[h][j], ea + (ebn - 1022) - 12 - kF);
-                            double *o = P.out + (int64_t)n * P.ldo + m;
-                            *o += v;
+                        for (int j = 0; j < 16; ++j) {
+                            constexpr float M = 12582912.0f;
+                            constexpr int MB = 0x4B400000;
+                            const float v = __uint_as_float(r[j]);
+                            if (lv == 4) {
+                                const float t1 = fmaf(v, 262144.f, M);              // round(2^18 v)
+                                const float q1 = fmaf(-(t1 - M), 0x1p-18f, v);      // exact rest
+                                const float t2 = fmaf(q1, 0x1p34f, M);
+                                acc[h + j] += (long long)((__float_as_int(t1) - MB) * 65536 + (__float_as_int(t2) - MB));
+                            } else if (lv == 3) {
+                                top3 = fmaxf(top3, fabsf(v));
+                                acc[h + j] += (long long)exact_int(v, 0x1p22f, 0x1p-24f) << 10;
+                            } else if (lv == 2) {
+                                top2 = fmaxf(top2, fabsf(v));
+                                acc[h + j] += (long long)exact_int(v, 0x1p14f, 0x1p-16f) << 18;
+                            } else if (lv == 1) {
+                                acc[h + j] += (long long)(__float_as_int(fmaf(v, 256.f, M)) - MB) << 26;
+                            } else {
+                                acc[h + j] += (long long)(__float_as_int(v + M) - MB) << 34;
+                            }
                         }
                     }
             }
+            if (!ok) break;
+            if (kCols == 32 && P.sn == 1) {
+                // a thread holds consecutive columns of one row: transpose the warp's
+                // 32 x 32 block so that its stores run along the row
+#pragma unroll
+                for (int d = kCols / 2; d > 0; d >>= 1)
+#pragma unroll
+                    for (int j = 0; j < kCols; ++j)
+                        if (!(j & d)) {
+                            const bool up = (lane & d) != 0;
+                            const long long got = __shfl_xor_sync(0xFFFFFFFFu, up ? acc[j] : acc[j + d], d);
+                            acc[j] = up ? got : acc[j];
+                            acc[j + d] = up ? acc[j + d] : got;
+                        }
+                const int n = nb * NB + sub * kCols + lane, m0 = mb * 128 + quarter * 32;
+                if (n < P.N) {
+                    const int ebn = P.eB[n];
+#pragma unroll
+                    for (int j = 0; j < kCols; ++j)
+                        if (m0 + j < P.M) {
+                            const int eam = P.eA[m0 + j];
+                            P.out[(m0 + j) * P.sm + n] += element(acc[j], eam, ebn);
+                        }
+                }
+            } else if (m < P.M) {
+                const int eam = P.eA[m];
+                const double dm = P.dm ? P.dm[m] : 0.0;
+#pragma unroll
+                for (int j = 0; j < kCols; ++j) {
+                    const int n = nb * NB + sub * kCols + j;
+                    if (n < P.N) {
+                        const double v = element(acc[j], eam, P.eB[n]);
+                        double *o = P.out + m * P.sm + n * P.sn;
+                        if (P.C)
+                            *o = fma(P.dn[n] + dm, P.C[m * P.sm + n * P.sn], *o) + v;
+                        else
+                            *o += v;
+                    }
+                }
+            }
         }
         if (!ok) *s_fail = 1;
-        if (range_bad) atomicOr(P.err, 2);
+        if (top2 > 256.f || top3 > 1.f) atomicOr(P.err, 2);  // beyond 2^24 units: not reached with these digits
     }
     // ---- exit: wait for every MMA this CTA issued and every copy it started,
     // then free tensor memory ----
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    if (warp == 1 && lane == 0) {
-        tc::mma_commit(drain);
+    if (warp == 1) {
+        if (elected) tc::mma_commit(drain);
         if (!tc::mbar_wait_bounded(drain, 0u)) *s_fail = 1;
     }
     if (warp == 0 && lane == 0) {
@@ -389,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ss_tc(SsArgs P) {
     tc::fence_after();
     if (*s_fail && tid == 0) atomicOr(P.err, 1);
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::kTmem) : "memory");
 }
 
 }  // namespace ss
@@ -397,120 +510,157 @@ __global__ void __launch_bounds__(kThreads, 1) k_ss_tc(SsArgs P) {
 // The dense path applies when both spins have replacements, no string space
 // exceeds 16384 strings (the planes of G stay below 2 GB) and the context asks
 // for it (fci_options.f64_same_spin).
-bool sigma_ss_ok(const fci_ctx *ctx) { return ctx->ssG_a != nullptr; }
+bool sigma_ss_ok(const fci_ctx *ctx) { return ctx->ssGa.planes != nullptr; }
+
+// Rows of G per tile: 96 where its tiles fill half of the chip, else 16.
+static int tile_rows(int64_t M, int64_t N, int nsm) { return ss::nblocks(M, ss::kM) * ss::nblocks(N, 96) * 2 >= nsm ? 96 : 16; }
 
 int build_ss_tables(fci_ctx *ctx) {
     const SpinTables &A = ctx->A, &B = ctx->B;
     if (ctx->opt.f64_same_spin == FCI_SS_FAMILY) return FCI_OK;
     if (A.nsingle == 0 || B.nsingle == 0 || A.ns > 16384 || B.ns > 16384) return FCI_OK;
-    int rc = FCI_OK;
+    int rc = FCI_OK, nsm = 0;
     cudaStream_t s = ctx->stream;
+    FCI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     const bool shared = (&A == &B) || (A.gval == B.gval);
-    auto build = [&](const SpinTables &T, unsigned char **planes, int **e) -> int {
-        const size_t pb = ss::plane_bytes(T.ns, T.ns);
-        *planes = (unsigned char *)dalloc(ctx, pb, &rc);
-        *e = (int *)dalloc(ctx, sizeof(int) * (size_t)T.ns, &rc);
-        if (rc) return rc;
-        FCI_CUDA(cudaMemsetAsync(*planes, 0, pb, s));
-        ss::k_ss_rowexp<<<ceil_div(T.ns, 256), 256, 0, s>>>(T.gval, T.ns, T.nsame, *e);
-        ss::k_ss_gplanes<<<ceil_div(T.ns * (int64_t)T.nsame, 256), 256, 0, s>>>(T.gcol, T.gval, T.ns, T.nsame, *e,
-                                                                                ss::pad_rows(T.ns), *planes);
-        FCI_CUDA(cudaGetLastError());
-        return FCI_OK;
+    auto build = [&](const SpinTables &T, int64_t M, SsOperand &O) -> int {
+        const int nb = O.nb = tile_rows(M, T.ns, nsm);
+        const int64_t nks = ss::ksteps(T.ns), nnb = ss::nblocks(T.ns, nb);
+        const unsigned ell = ceil_div(T.ns * (int64_t)T.nsame, 256);
+        // the K-steps of each row block that hold a nonzero (every block keeps at
+        // least one)
+        std::vector<unsigned char> used((size_t)(nnb * nks));
+        std::vector<int> slot(used.size(), 0), tab;
+        O.list_bytes = sizeof(int) * (size_t)(nnb + 1 + nnb * nks);
+        O.lists = (int *)dalloc(ctx, O.list_bytes, &rc);  // koff [nnb + 1], kidx
+        O.e = (int *)dalloc(ctx, sizeof(int) * (size_t)T.ns, &rc);
+        int *dslot = (int *)dalloc(ctx, sizeof(int) * slot.size(), &rc);
+        unsigned char *dused = reinterpret_cast<unsigned char *>(dslot);  // read back before the slots go there
+        auto done = [&](int code) {
+            dfree(ctx, dslot, sizeof(int) * slot.size());
+            return code;
+        };
+        if (rc) return done(rc);
+        cudaError_t e = cudaMemsetAsync(dused, 0, used.size(), s);
+        if (e == cudaSuccess) {
+            ss::k_ss_used<<<ell, 256, 0, s>>>(T.gcol, T.gval, T.ns, T.nsame, nb, nks, dused);
+            ss::k_ss_rowexp<<<ceil_div(T.ns, 256), 256, 0, s>>>(T.gval, T.ns, T.nsame, O.e);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(used.data(), dused, used.size(), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return done(cuda_fail(e, "same-spin K-step lists"));
+        std::vector<int> koff(1, 0), kidx;
+        for (int64_t b = 0; b < nnb; ++b) {
+            for (int64_t k = 0; k < nks; ++k)
+                if (used[b * nks + k] || (k == nks - 1 && (int)kidx.size() == koff.back())) {
+                    slot[b * nks + k] = (int)kidx.size();
+                    kidx.push_back((int)k);
+                }
+            koff.push_back((int)kidx.size());
+        }
+        tab = koff;
+        tab.insert(tab.end(), kidx.begin(), kidx.end());
+        O.nnb = (int)nnb;
+        O.plane_bytes = kidx.size() * (size_t)(6 * nb * 32);
+        O.planes = (unsigned char *)dalloc(ctx, O.plane_bytes, &rc);
+        if (rc) return done(rc);
+        e = cudaMemcpyAsync(O.lists, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dslot, slot.data(), sizeof(int) * slot.size(), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(O.planes, 0, O.plane_bytes, s);
+        if (e == cudaSuccess) {
+            ss::k_ss_gplanes<<<ell, 256, 0, s>>>(T.gcol, T.gval, T.ns, T.nsame, O.e, nb, nks, dslot, O.planes);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        return done(e == cudaSuccess ? FCI_OK : cuda_fail(e, "same-spin planes"));
     };
-    if ((rc = build(A, &ctx->ssG_a, &ctx->ssE_a))) return rc;
-    if (shared) {
-        ctx->ssG_b = ctx->ssG_a;
-        ctx->ssE_b = ctx->ssE_a;
-    } else if ((rc = build(B, &ctx->ssG_b, &ctx->ssE_b))) {
+    if ((rc = build(A, B.ns, ctx->ssGa))) return rc;
+    if (shared)
+        ctx->ssGb = ctx->ssGa;
+    else if ((rc = build(B, A.ns, ctx->ssGb)))
         return rc;
-    }
     // per-call workspace: C by rows (K = J_b) and by columns (K = J_a), and their exponents
-    ctx->ssCr = (unsigned char *)dalloc(ctx, ss::plane_bytes(A.ns, B.ns), &rc);
-    ctx->ssCc = (unsigned char *)dalloc(ctx, ss::plane_bytes(B.ns, A.ns), &rc);
+    ctx->ssCr = (unsigned char *)dalloc(ctx, ss::c_bytes(A.ns, B.ns), &rc);
+    ctx->ssCc = (unsigned char *)dalloc(ctx, ss::c_bytes(B.ns, A.ns), &rc);
     ctx->ssEr = (int *)dalloc(ctx, sizeof(int) * (size_t)(A.ns + B.ns + 1), &rc);
     if (rc) return rc;
     ctx->ssEc = ctx->ssEr + A.ns;
     // plane padding (rows past the strings, K past the last string) stays zero
-    FCI_CUDA(cudaMemsetAsync(ctx->ssCr, 0, ss::plane_bytes(A.ns, B.ns), s));
-    FCI_CUDA(cudaMemsetAsync(ctx->ssCc, 0, ss::plane_bytes(B.ns, A.ns), s));
-    FCI_CUDA(opt_in_max_smem((const void *)ss::k_ss_tc, ctx->device));
+    FCI_CUDA(cudaMemsetAsync(ctx->ssCr, 0, ss::c_bytes(A.ns, B.ns), s));
+    FCI_CUDA(cudaMemsetAsync(ctx->ssCc, 0, ss::c_bytes(B.ns, A.ns), s));
+    FCI_CUDA(opt_in_max_smem((const void *)ss::k_ss_tc<96>, ctx->device));
+    FCI_CUDA(opt_in_max_smem((const void *)ss::k_ss_tc<16>, ctx->device));
     FCI_CUDA(cudaStreamSynchronize(s));
     return FCI_OK;
 }
 
 void free_ss_tables(fci_ctx *ctx) {
     const SpinTables &A = ctx->A, &B = ctx->B;
-    if (ctx->ssG_b && ctx->ssG_b != ctx->ssG_a) {
-        dfree(ctx, ctx->ssG_b, ss::plane_bytes(B.ns, B.ns));
-        dfree(ctx, ctx->ssE_b, sizeof(int) * (size_t)B.ns);
-    }
-    if (ctx->ssG_a) {
-        dfree(ctx, ctx->ssG_a, ss::plane_bytes(A.ns, A.ns));
-        dfree(ctx, ctx->ssE_a, sizeof(int) * (size_t)A.ns);
-    }
-    dfree(ctx, ctx->ssCr, ss::plane_bytes(A.ns, B.ns));
-    dfree(ctx, ctx->ssCc, ss::plane_bytes(B.ns, A.ns));
+    auto drop = [&](SsOperand &O, int64_t ns) {
+        dfree(ctx, O.planes, O.plane_bytes);
+        dfree(ctx, O.lists, O.list_bytes);
+        dfree(ctx, O.e, sizeof(int) * (size_t)ns);
+        O = SsOperand{};
+    };
+    if (ctx->ssGb.e != ctx->ssGa.e) drop(ctx->ssGb, B.ns);
+    ctx->ssGb = SsOperand{};
+    drop(ctx->ssGa, A.ns);
+    dfree(ctx, ctx->ssCr, ss::c_bytes(A.ns, B.ns));
+    dfree(ctx, ctx->ssCc, ss::c_bytes(B.ns, A.ns));
     dfree(ctx, ctx->ssEr, sizeof(int) * (size_t)(A.ns + B.ns + 1));
-    ctx->ssG_a = ctx->ssG_b = ctx->ssCr = ctx->ssCc = nullptr;
-    ctx->ssE_a = ctx->ssE_b = ctx->ssEr = ctx->ssEc = nullptr;
+    ctx->ssCr = ctx->ssCc = nullptr;
+    ctx->ssEr = ctx->ssEc = nullptr;
 }
 
-// sigma += sigma_1 (which = 1), sigma_2 (which = 2) or both (which = 3), in
-// that order, from the dense planes.
-static unsigned grid_stride(int64_t n) { return (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8); }
-
+// sigma += sigma_1 (which = 1), sigma_2 (which = 2) or both (which = 3), in that
+// order, from the dense planes; sigma_2's pass also applies the diagonal of the
+// alpha strings' Hamiltonian and, with sigma_1, of the beta strings'.
 int launch_sigma_ss(fci_ctx *ctx, const double *C, double *sig, int which, cudaStream_t s, int rec, int slot) {
     const SpinTables &A = ctx->A, &B = ctx->B;
     const int64_t nsa = A.ns, nsb = B.ns;
     int nsm = 0;
     FCI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-    auto gemm = [&](const unsigned char *Ap, int64_t rowsA, int M, const int *eA, const unsigned char *Bp, int64_t rowsB,
-                    int N, const int *eB, int64_t K) -> int {
+    auto gemm = [&](const unsigned char *Ap, int64_t M, const int *eA, const SsOperand &O, int64_t N, int64_t sm, int64_t sn,
+                    const double *dn, const double *dm) -> int {
         ss::SsArgs P;
         P.A = Ap;
-        P.B = Bp;
-        P.rowsA = rowsA;
-        P.rowsB = rowsB;
-        P.M = M;
-        P.N = N;
-        P.nks = (K + 15) / 16;
+        P.B = O.planes;
+        P.koff = O.lists;
+        P.kidx = O.lists + O.nnb + 1;
+        P.M = (int)M;
+        P.N = (int)N;
         P.eA = eA;
-        P.eB = eB;
+        P.eB = O.e;
         P.out = sig;
-        P.ldo = nsb;
+        P.sm = sm;
+        P.sn = sn;
+        P.C = dn ? C : nullptr;
+        P.dn = dn;
+        P.dm = dm;
         P.err = ctx->d_err;
-        const int64_t tiles = (int64_t)((M + 127) / 128) * ((N + ss::kBN - 1) / ss::kBN);
-        const unsigned grid = (unsigned)std::min<int64_t>(tiles, nsm);
-        ss::k_ss_tc<<<grid, ss::kThreads, ss::kSmem, s>>>(P);
+        const unsigned grid = (unsigned)std::min<int64_t>(ss::nblocks(M, ss::kM) * O.nnb, nsm);
+        if (O.nb == 96)
+            ss::k_ss_tc<96><<<grid, ss::Shape<96>::kThreads, ss::Shape<96>::kSmem, s>>>(P);
+        else
+            ss::k_ss_tc<16><<<grid, ss::Shape<16>::kThreads, ss::Shape<16>::kSmem, s>>>(P);
         FCI_CUDA(cudaGetLastError());
         return FCI_OK;
     };
-    // exponents of C's rows (I_a) and columns (I_b)
+    // exponents of C's rows (I_a) and columns (I_b), then its planes
     FCI_CUDA(cudaMemsetAsync(ctx->ssEr, 0, sizeof(int) * (size_t)(nsa + nsb), s));
     ss::k_ss_cexp<<<dim3(ceil_div(nsb, 32), ceil_div(nsa, 32)), dim3(32, 8), 0, s>>>(C, nsa, nsb, ctx->ssEr, ctx->ssEc);
     FCI_CUDA(cudaGetLastError());
-    if (which & 1) {  // sigma_1: A = G_b (m = I_b), B = C by rows (n = I_a), K = J_b
-        ss::k_ss_cplanes<<<ceil_div(nsa * ((nsb + 7) / 8), 256), 256, 0, s>>>(C, nsa, nsb, 0, ctx->ssEr,
-                                                                             ss::pad_rows(nsa), ctx->ssCr);
-        FCI_CUDA(cudaGetLastError());
-        if (int rc = gemm(ctx->ssG_b, ss::pad_rows(nsb), (int)nsb, ctx->ssE_b, ctx->ssCr, ss::pad_rows(nsa), (int)nsa,
-                          ctx->ssEr, nsb))
-            return rc;
+    ss::k_ss_cplanes<<<dim3(ceil_div(nsb, 64), ceil_div(nsa, 64)), 256, 0, s>>>(
+        C, nsa, nsb, ctx->ssEr, ctx->ssEc, which & 1 ? ctx->ssCr : nullptr, which & 2 ? ctx->ssCc : nullptr);
+    FCI_CUDA(cudaGetLastError());
+    if (which & 1) {  // sigma_1: A = C by rows (m = I_a), B = G_b (n = I_b), K = J_b
+        if (int rc = gemm(ctx->ssCr, nsa, ctx->ssEr, ctx->ssGb, nsb, nsb, 1, nullptr, nullptr)) return rc;
         prof_mark(ctx, rec, slot, s);
         ++slot;
     }
-    // the diagonal: both spins (which = 3), alpha only (which = 2: sigma_1 follows
-    // as the parity transpose of sigma_2), beta only (which = 1)
-    ss::k_ss_diag<<<grid_stride(nsa * nsb), 256, 0, s>>>(C, sig, which & 2 ? A.gval : nullptr,
-                                                        which & 1 ? B.gval : nullptr, nsa, nsb);
-    FCI_CUDA(cudaGetLastError());
-    if (which & 2) {  // sigma_2: A = C by columns (m = I_b), B = G_a (n = I_a), K = J_a
-        ss::k_ss_cplanes<<<ceil_div(nsb * ((nsa + 7) / 8), 256), 256, 0, s>>>(C, nsa, nsb, 1, ctx->ssEc,
-                                                                             ss::pad_rows(nsb), ctx->ssCc);
-        FCI_CUDA(cudaGetLastError());
-        if (int rc = gemm(ctx->ssCc, ss::pad_rows(nsb), (int)nsb, ctx->ssEc, ctx->ssG_a, ss::pad_rows(nsa), (int)nsa,
-                          ctx->ssE_a, nsa))
+    if (which & 2) {  // sigma_2: A = C by columns (m = I_b), B = G_a (n = I_a), K = J_a, and the diagonal
+        if (int rc = gemm(ctx->ssCc, nsb, ctx->ssEc, ctx->ssGa, nsa, 1, nsb, A.gval, which & 1 ? B.gval : nullptr))
             return rc;
         prof_mark(ctx, rec, slot, s);
     }
