@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "small_dense.cuh"
 
 namespace fci {
 namespace bt {
@@ -289,43 +290,31 @@ __global__ void __launch_bounds__(kBlock) k_bdots(const Chunk *__restrict__ ch, 
         }
     __shared__ double red[8][kBlock / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        double v = acc[j];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[j][warp] = v;
-    }
+    const double v = sd::warp_reduce8(acc, lane);
+    if ((lane & 3) == 0) red[sd::reduce8_index(lane)][warp] = v;
     __syncthreads();
     if (threadIdx.x < mg) {
-        double v = 0.0;
-        for (int w = 0; w < kBlock / 32; ++w) v += red[threadIdx.x][w];
-        partial[(int64_t)cidx * 32 + i0 + threadIdx.x] = v;
+        double t = 0.0;
+        for (int w = 0; w < kBlock / 32; ++w) t += red[threadIdx.x][w];
+        partial[(int64_t)cidx * 32 + i0 + threadIdx.x] = t;
     }
 }
 
-// out[i*os + j*js] = sum of partial[c*STRIDE + j] over instance i's chunks:
-// one CTA per instance, a strided sum per thread and a fixed-order tree.
+// out[i*os + j*js] = sum of partial[c*STRIDE + j] over instance i's chunks in a
+// fixed order: one CTA per instance, a warp per j (j, j + 8, ...).
 template <int STRIDE>
 __global__ void __launch_bounds__(kBlock) k_breduce(const int *__restrict__ cfirst, const int *__restrict__ on,
                                                     const double *__restrict__ partial, int m,
                                                     double *__restrict__ out, int64_t os, int64_t js) {
     const int i = blockIdx.x;
     if (!on[i]) return;
-    __shared__ double red[kBlock / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c0 = cfirst[i], c1 = cfirst[i + 1];
-    for (int j = 0; j < m; ++j) {
+    for (int j = warp; j < m; j += kBlock / 32) {
         double v = 0.0;
-        for (int c = c0 + threadIdx.x; c < c1; c += kBlock) v += partial[(int64_t)c * STRIDE + j];
+        for (int c = c0 + lane; c < c1; c += 32) v += partial[(int64_t)c * STRIDE + j];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[warp] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < kBlock / 32; ++w) t += red[w];
-            out[i * os + j * js] = t;
-        }
-        __syncthreads();
+        if (lane == 0) out[i * os + j * js] = v;
     }
 }
 
@@ -442,113 +431,14 @@ __global__ void k_bpad(const int *__restrict__ on, const double *__restrict__ nr
     Ai[j * kMaxSub + j] = kPad;
 }
 
-// Cyclic Jacobi per instance (textbook; ascending order, stable).
-__global__ void k_bjacobi(const int *__restrict__ on, const double *__restrict__ Aall, int m,
-                          double *__restrict__ wall, double *__restrict__ Vall) {
+// Eigenvalues and eigenvectors of each instance's projected matrix (small_dense.cuh).
+__global__ void __launch_bounds__(kBlock) k_bjacobi(const int *__restrict__ on, const double *__restrict__ Aall, int m,
+                                                    double *__restrict__ wall, double *__restrict__ Vall) {
     const int i = blockIdx.x;
     if (!on[i]) return;
-    const double *A = Aall + (int64_t)i * kMaxSub * kMaxSub;
-    double *w = wall + (int64_t)i * kMaxSub;
-    double *V = Vall + (int64_t)i * kMaxSub * kMaxSub;
-    __shared__ double a[kMaxSub][kMaxSub + 1];
-    __shared__ double v[kMaxSub][kMaxSub + 1];
-    __shared__ int order[kMaxSub];
-    const int tid = threadIdx.x;
-    for (int t = tid; t < m * m; t += blockDim.x) {
-        const int r = t / m, c = t % m;
-        a[r][c] = 0.5 * (A[r * kMaxSub + c] + A[c * kMaxSub + r]);
-        v[r][c] = (r == c) ? 1.0 : 0.0;
-    }
-    __syncthreads();
-    // Parallel cyclic Jacobi with round-robin pair ordering: each step rotates
-    // m/2 disjoint pairs at once (rotations on disjoint index pairs commute).
-    // A rotation is skipped when |a_pq| < 1e-14 (|a_pp| + |a_qq|); the sweeps
-    // stop after a sweep without rotation (60 at most).
-    __shared__ int rotated;
-    __shared__ int pos[kMaxSub + 1];
-    __shared__ int pp[kMaxSub / 2 + 1], pq[kMaxSub / 2 + 1];
-    __shared__ double pc[kMaxSub / 2 + 1], psn[kMaxSub / 2 + 1];
-    const int me = m + (m & 1);  // even number of players; index m is a dummy when m is odd
-    const int half = me / 2;
-    for (int t = tid; t < me; t += blockDim.x) pos[t] = t;
-    __syncthreads();
-    for (int sweep = 0; sweep < 60; ++sweep) {
-        if (tid == 0) rotated = 0;
-        __syncthreads();
-        for (int step = 0; step < me - 1; ++step) {
-            for (int k = tid; k < half; k += blockDim.x) {
-                int p = pos[k], q = pos[me - 1 - k];
-                if (p > q) { const int t2 = p; p = q; q = t2; }
-                double c = 1.0, sn = 0.0;
-                if (q < m) {
-                    const double apq = a[p][q];
-                    if (fabs(apq) > 1e-14 * (fabs(a[p][p]) + fabs(a[q][q]))) {
-                        rotated = 1;
-                        const double theta = (a[q][q] - a[p][p]) / (2.0 * apq);
-                        const double tt = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                        c = 1.0 / sqrt(tt * tt + 1.0);
-                        sn = tt * c;
-                    }
-                }
-                pp[k] = p;
-                pq[k] = q;
-                pc[k] = c;
-                psn[k] = sn;
-            }
-            __syncthreads();
-            // columns: a <- a J
-            for (int t = tid; t < half * m; t += blockDim.x) {
-                const int k = t / m, r = t % m;
-                if (psn[k] == 0.0) continue;
-                const int p = pp[k], q = pq[k];
-                const double c = pc[k], sn = psn[k];
-                const double arp = a[r][p], arq = a[r][q];
-                a[r][p] = c * arp - sn * arq;
-                a[r][q] = sn * arp + c * arq;
-            }
-            __syncthreads();
-            // rows: a <- J^T a ; eigenvectors v <- v J
-            for (int t = tid; t < half * m; t += blockDim.x) {
-                const int k = t / m, r = t % m;
-                if (psn[k] == 0.0) continue;
-                const int p = pp[k], q = pq[k];
-                const double c = pc[k], sn = psn[k];
-                const double apr = a[p][r], aqr = a[q][r];
-                a[p][r] = c * apr - sn * aqr;
-                a[q][r] = sn * apr + c * aqr;
-                const double vrp = v[r][p], vrq = v[r][q];
-                v[r][p] = c * vrp - sn * vrq;
-                v[r][q] = sn * vrp + c * vrq;
-            }
-            __syncthreads();
-            // next round-robin pairing: player 0 stays, the others rotate
-            if (tid == 0) {
-                const int last = pos[me - 1];
-                for (int t = me - 1; t > 1; --t) pos[t] = pos[t - 1];
-                pos[1] = last;
-            }
-            __syncthreads();
-        }
-        if (!rotated) break;
-    }
-    if (tid == 0) {
-        for (int r = 0; r < m; ++r) order[r] = r;
-        for (int r = 1; r < m; ++r) {
-            const int o = order[r];
-            int j = r - 1;
-            while (j >= 0 && a[order[j]][order[j]] > a[o][o]) {
-                order[j + 1] = order[j];
-                --j;
-            }
-            order[j + 1] = o;
-        }
-    }
-    __syncthreads();
-    for (int t = tid; t < m; t += blockDim.x) w[t] = a[order[t]][order[t]];
-    for (int t = tid; t < m * m; t += blockDim.x) {
-        const int r = t / m, k = t % m;
-        V[r * m + k] = v[r][order[k]];
-    }
+    __shared__ sd::EigShared S;
+    sd::eig_symmetric(Aall + (int64_t)i * kMaxSub * kMaxSub, kMaxSub, m, wall + (int64_t)i * kMaxSub,
+                      Vall + (int64_t)i * kMaxSub * kMaxSub, S);
 }
 
 // nroots smallest diagonal entries per instance (ties: lower index) -> unit vectors in B_k
@@ -1263,7 +1153,7 @@ static int batch_davidson_run(fci_batch *b, int nroots, double tol, double *ener
     const int keep = std::min(keepn, maxsub);
     const unsigned gi = (unsigned)((ninst + 127) / 128);
     auto iteration = [&](int mi, bool can_refine, int *sig_launches) -> int {
-        k_bjacobi<<<ninst, 128, 0, s>>>(W.on, W.A, mi, W.w, W.V);
+        k_bjacobi<<<ninst, kBlock, 0, s>>>(W.on, W.A, mi, W.w, W.V);
         for (int k = 0; k < nroots; ++k) {
             k_blincomb<<<b->nchunks, kBlock, 0, s>>>(b->d_chunks, W.on, W.Bv, ntot, mi, W.V + k, kMaxSub * kMaxSub, mi,
                                                       1.0, 0.0, W.X + (size_t)k * ntot);

@@ -42,22 +42,37 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "small_dense.cuh"
 
 namespace fci {
 
 constexpr int kMaxSub = 32;   // subspace limit (vectors)
 constexpr int kDotBlocks = 304;  // 2 x 152 SMs
 
-// partial[b][g*8 + j] = sum over stripe b of X_{g*8+j} . y, j < 8.  The
-// vectors are split into groups of 8 (blockIdx.x % groups) so that each
-// thread keeps 8 accumulators and many blocks fit on an SM; the groups of one
-// stripe run side by side and share y through L2.  On GB300 these products are
-// bound by the FP64 pipe (about 1.2 TFLOP/s against 2 FLOP per 8-byte element),
-// so each element costs exactly one FMA (a single chain per accumulator).
-// VEC = 4 reads 32-byte vectors (n % 4 == 0, 32-byte aligned rows).
+// One set of dot products out[i stride] = X_i . y, i < count <= m, of a launch.
+struct DotSet {
+    const double *X, *y;
+    double *out;
+    int stride, count;
+};
+
+// Dot products of one or two sets (blockIdx.y).  The vectors are split into
+// groups of 8 (blockIdx.x % groups) so that each thread keeps 8 accumulators and
+// many blocks fit on an SM; the groups of one stripe run side by side and share
+// y through L2.  On GB300 these products are bound by the FP64 pipe (about 1.2
+// TFLOP/s against 2 FLOP per 8-byte element), so each element costs exactly one
+// FMA (a single chain per accumulator), the accumulators of a warp are summed
+// together (sd::warp_reduce8) and there are no more stripes than give every
+// thread a few elements: at 3920 elements 912 blocks spent 18.6 us reducing
+// zeros.  The last block sums the stripes in a fixed order (a second launch whose
+// one warp did took 27 us).  VEC = 4 reads 32-byte vectors (n % 4 == 0, 32-byte
+// aligned rows).  gate: null, or a device flag; 0 skips the launch.
 template <int VEC>
-__global__ void __launch_bounds__(256) k_multidot(const double *__restrict__ X, int m, const double *__restrict__ y,
-                                                  int64_t n, int groups, double *__restrict__ partial) {
+__global__ void __launch_bounds__(256) k_multidot(DotSet s0, DotSet s1, int m, int64_t n, int groups, double *partial,
+                                                  int *counter, const int *__restrict__ gate) {
+    if (gate != nullptr && *gate == 0) return;
+    const DotSet D = blockIdx.y ? s1 : s0;
+    partial += (size_t)blockIdx.y * kDotBlocks * 32;
     const int g = blockIdx.x % groups;
     const int stripe = blockIdx.x / groups;
     const int nstripes = gridDim.x / groups;
@@ -69,13 +84,13 @@ __global__ void __launch_bounds__(256) k_multidot(const double *__restrict__ X, 
     const int64_t stride = (int64_t)nstripes * blockDim.x;
     if (VEC == 4) {
         const int64_t n4 = n / 4;
-        const double4_32a *y4 = reinterpret_cast<const double4_32a *>(y);
+        const double4_32a *y4 = reinterpret_cast<const double4_32a *>(D.y);
         for (int64_t r = stripe * (int64_t)blockDim.x + threadIdx.x; r < n4; r += stride) {
             const double4_32a yr = y4[r];
 #pragma unroll
             for (int j = 0; j < 8; ++j)
                 if (j < mg) {
-                    const double4_32a x = reinterpret_cast<const double4_32a *>(X + (int64_t)(i0 + j) * n)[r];
+                    const double4_32a x = reinterpret_cast<const double4_32a *>(D.X + (int64_t)(i0 + j) * n)[r];
                     double a = acc[j];
                     a = fma(x.x, yr.x, a);
                     a = fma(x.y, yr.y, a);
@@ -86,37 +101,59 @@ __global__ void __launch_bounds__(256) k_multidot(const double *__restrict__ X, 
         }
     } else {
         for (int64_t r = stripe * (int64_t)blockDim.x + threadIdx.x; r < n; r += stride) {
-            const double yr = y[r];
+            const double yr = D.y[r];
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (j < mg) acc[j] = fma(X[(int64_t)(i0 + j) * n + r], yr, acc[j]);
+                if (j < mg) acc[j] = fma(D.X[(int64_t)(i0 + j) * n + r], yr, acc[j]);
         }
     }
-    __shared__ double red[8][8];
+    __shared__ double red[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        double v = acc[j];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[j][warp] = v;
-    }
+    const double v = sd::warp_reduce8(acc, lane);
+    if ((lane & 3) == 0) red[sd::reduce8_index(lane)][warp] = v;
     __syncthreads();
     if (threadIdx.x < mg) {
-        double v = 0.0;
-        for (int w = 0; w < 8; ++w) v += red[threadIdx.x][w];
-        partial[(int64_t)stripe * 32 + i0 + threadIdx.x] = v;
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[threadIdx.x][w];
+        partial[(int64_t)stripe * 32 + i0 + threadIdx.x] = t;
+    }
+    if (!sd::last_block(counter + blockIdx.y, gridDim.x)) return;
+    // eight threads per dot product, then their sum
+    double t = 0.0;
+    if (lane < m)
+        for (int b = warp; b < nstripes; b += 8) t += partial[(int64_t)b * 32 + lane];
+    red[warp][lane] = t;
+    __syncthreads();
+    if (threadIdx.x < D.count) {
+        t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+        D.out[(int64_t)threadIdx.x * D.stride] = t;
     }
 }
 
-// out[i] = sum_b partial[b][i] (fixed order), optionally written to a matrix slot.
+// out[i] = sum_b partial[b][i] in a fixed order, one block of 256 threads; row
+// stride of partial and number of values at most MAXM (1 or 32).
 template <int MAXM>
-__global__ void k_reduce_partials(const double *__restrict__ partial, int nb, int m, double *__restrict__ out,
-                                  int out_stride) {
-    int i = threadIdx.x;
-    if (i >= m) return;
+__global__ void __launch_bounds__(256) k_reduce_partials(const double *__restrict__ partial, int nb, int m,
+                                                         double *__restrict__ out, int out_stride) {
+    __shared__ double red[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double v = 0.0;
-    for (int b = 0; b < nb; ++b) v += partial[(int64_t)b * MAXM + i];
-    out[(int64_t)i * out_stride] = v;
+    if (MAXM == 1) {
+        for (int b = threadIdx.x; b < nb; b += 256) v += partial[b];
+        v = sd::block_sum256(v, &red[0][0]);
+        if (threadIdx.x == 0) out[0] = v;
+    } else {
+        if (lane < m)
+            for (int b = warp; b < nb; b += 8) v += partial[(int64_t)b * MAXM + lane];
+        red[warp][lane] = v;
+        __syncthreads();
+        if (threadIdx.x < m) {
+            v = 0.0;
+            for (int w = 0; w < 8; ++w) v += red[w][threadIdx.x];
+            out[(int64_t)threadIdx.x * out_stride] = v;
+        }
+    }
 }
 
 // y[r] = beta*y[r] + sum_i coef[i] X_i[r]; pairs of elements per thread
@@ -153,11 +190,19 @@ __global__ void k_lincomb(const double *__restrict__ X, int m, const double *__r
     }
 }
 
-// y -= sum_i coef[i] X_i (Gram-Schmidt update with device coefficients);
-// partial[block] = this block's share of ||y||^2 after the update.
+// y -= sum_i coef[i] X_i (Gram-Schmidt update with device coefficients); the
+// last block leaves *nrm = ||y||^2 after the update and, for the first pass
+// (again != null), *again = 1 when the pass removed more than half of it
+// (||y1||^2 < sum c_i^2, or a NaN): the second pass is launched gated by it.
 template <int VEC>
 __global__ void __launch_bounds__(256) k_sub_proj(const double *__restrict__ X, int m, const double *__restrict__ coef,
-                                                  double *__restrict__ y, int64_t n, double *__restrict__ partial) {
+                                                  double *__restrict__ y, int64_t n, double *__restrict__ partial,
+                                                  double *__restrict__ nrm_out, int *__restrict__ again, int *counter,
+                                                  const int *__restrict__ gate) {
+    if (gate != nullptr && *gate == 0) return;
+    __shared__ double c[32];
+    if (threadIdx.x < m) c[threadIdx.x] = coef[threadIdx.x];
+    __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     double nrm = 0.0;
     if (VEC == 2) {
@@ -166,10 +211,9 @@ __global__ void __launch_bounds__(256) k_sub_proj(const double *__restrict__ X, 
             double2 v = reinterpret_cast<const double2 *>(y)[r];
 #pragma unroll 8
             for (int i = 0; i < m; ++i) {
-                const double c = coef[i];
                 const double2 x = reinterpret_cast<const double2 *>(X + (int64_t)i * n)[r];
-                v.x = fma(-c, x.x, v.x);
-                v.y = fma(-c, x.y, v.y);
+                v.x = fma(-c[i], x.x, v.x);
+                v.y = fma(-c[i], x.y, v.y);
             }
             reinterpret_cast<double2 *>(y)[r] = v;
             nrm = fma(v.x, v.x, nrm);
@@ -179,46 +223,91 @@ __global__ void __launch_bounds__(256) k_sub_proj(const double *__restrict__ X, 
         for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += stride) {
             double v = y[r];
 #pragma unroll 8
-            for (int i = 0; i < m; ++i) v = fma(-coef[i], X[(int64_t)i * n + r], v);
+            for (int i = 0; i < m; ++i) v = fma(-c[i], X[(int64_t)i * n + r], v);
             y[r] = v;
             nrm = fma(v, v, nrm);
         }
     }
     __shared__ double red[8];
-    for (int o = 16; o > 0; o >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = nrm;
+    nrm = sd::block_sum256(nrm, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = nrm;
+    if (!sd::last_block(counter, gridDim.x)) return;
+    double t = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) t += partial[b];
     __syncthreads();
+    t = sd::block_sum256(t, red);
     if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int w = 0; w < 8; ++w) v += red[w];
-        partial[blockIdx.x] = v;
+        *nrm_out = t;
+        if (again != nullptr) {
+            double c2 = 0.0;
+            for (int i = 0; i < m; ++i) c2 += c[i] * c[i];
+            *again = t >= c2 ? 0 : 1;
+        }
     }
 }
 
-// r = hx - e x; t = -r / (d - e) with the denominator floor; partial ||r||^2
-__global__ void __launch_bounds__(256) k_residual_precond(const double *__restrict__ x, const double *__restrict__ hx,
-                                                          const double *__restrict__ diag, const double *__restrict__ ev,
-                                                          int k, double *__restrict__ t, int64_t n,
-                                                          double *__restrict__ partial) {
+// One root's Ritz vector x = B v, its sigma hx = S v, the residual r = hx - e x
+// and the correction t = -r / (d - e) with the denominator floor, in one pass
+// over the subspace; *rn2 = ||r||^2 (last block, fixed order).
+template <int VEC>
+__global__ void __launch_bounds__(256) k_ritz(const double *__restrict__ B, const double *__restrict__ S, int m,
+                                              const double *__restrict__ V, const double *__restrict__ ev, int k,
+                                              const double *__restrict__ diag, double *__restrict__ X,
+                                              double *__restrict__ HX, double *__restrict__ T, int64_t n,
+                                              double *__restrict__ partial, double *__restrict__ rn2, int *counter) {
+    __shared__ double c[32];
+    if (threadIdx.x < m) c[threadIdx.x] = V[(int64_t)threadIdx.x * m + k];
+    __syncthreads();
     const double e = ev[k];
-    double acc = 0.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        double r = hx[i] - e * x[i];
-        double d = diag[i] - e;
+    double acc = 0.0;
+    auto finish = [&](double x, double h, double dd) {
+        const double r = h - e * x;
+        double d = dd - e;
         if (fabs(d) < 1e-8) d = d < 0 ? -1e-8 : 1e-8;
-        t[i] = -r / d;
-        acc += r * r;
+        acc = fma(r, r, acc);
+        return -r / d;
+    };
+    if (VEC == 2) {
+        const int64_t n2 = n / 2;
+        for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n2; r += stride) {
+            double2 x = make_double2(0.0, 0.0), h = x;
+#pragma unroll 4
+            for (int i = 0; i < m; ++i) {
+                const double2 b = reinterpret_cast<const double2 *>(B + (int64_t)i * n)[r];
+                const double2 s = reinterpret_cast<const double2 *>(S + (int64_t)i * n)[r];
+                x.x = fma(c[i], b.x, x.x);
+                x.y = fma(c[i], b.y, x.y);
+                h.x = fma(c[i], s.x, h.x);
+                h.y = fma(c[i], s.y, h.y);
+            }
+            const double2 d = reinterpret_cast<const double2 *>(diag)[r];
+            reinterpret_cast<double2 *>(X)[r] = x;
+            reinterpret_cast<double2 *>(HX)[r] = h;
+            reinterpret_cast<double2 *>(T)[r] = make_double2(finish(x.x, h.x, d.x), finish(x.y, h.y, d.y));
+        }
+    } else {
+        for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += stride) {
+            double x = 0.0, h = 0.0;
+#pragma unroll 4
+            for (int i = 0; i < m; ++i) {
+                x = fma(c[i], B[(int64_t)i * n + r], x);
+                h = fma(c[i], S[(int64_t)i * n + r], h);
+            }
+            X[r] = x;
+            HX[r] = h;
+            T[r] = finish(x, h, diag[r]);
+        }
     }
     __shared__ double red[8];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    acc = sd::block_sum256(acc, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = acc;
+    if (!sd::last_block(counter, gridDim.x)) return;
+    double t = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) t += partial[b];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int w = 0; w < 8; ++w) v += red[w];
-        partial[blockIdx.x] = v;
-    }
+    t = sd::block_sum256(t, red);
+    if (threadIdx.x == 0) *rn2 = t;
 }
 
 // S_j += V[j][k] * delta for j < m (rank-1 correction of the subspace sigma vectors)
@@ -257,108 +346,24 @@ __global__ void k_scale(double *__restrict__ y, const double *__restrict__ nrm2,
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) y[i] *= s;
 }
 
-// Cyclic Jacobi on the symmetric m x m matrix A (row-major, ld = lda); writes
-// ascending eigenvalues to w and eigenvectors (columns) to V[m][m].
-__global__ void k_jacobi(const double *__restrict__ A, int lda, int m, double *__restrict__ w, double *__restrict__ V) {
-    __shared__ double a[kMaxSub][kMaxSub + 1];
-    __shared__ double v[kMaxSub][kMaxSub + 1];
-    __shared__ int order[kMaxSub];
-    const int tid = threadIdx.x;
-    for (int t = tid; t < m * m; t += blockDim.x) {
-        int i = t / m, j = t % m;
-        a[i][j] = 0.5 * (A[i * lda + j] + A[j * lda + i]);
-        v[i][j] = (i == j) ? 1.0 : 0.0;
+// Eigenvalues w (ascending) and eigenvectors (columns of V[m][m]) of the
+// projected matrix (small_dense.cuh).
+__global__ void __launch_bounds__(256) k_jacobi(const double *__restrict__ A, int lda, int m, double *__restrict__ w,
+                                                double *__restrict__ V) {
+    __shared__ sd::EigShared S;
+    sd::eig_symmetric(A, lda, m, w, V, S);
+}
+
+// What the host reads per iteration, into pinned host memory: Ritz values,
+// squared residual norms, the device error word.
+__global__ void k_publish(const double *__restrict__ w, const double *__restrict__ rn2, int nr, const int *__restrict__ err,
+                          double *__restrict__ host) {
+    const int i = threadIdx.x;
+    if (i < nr) {
+        host[i] = w[i];
+        host[8 + i] = rn2[i];
     }
-    __syncthreads();
-    // Parallel cyclic Jacobi with round-robin pair ordering: each step rotates
-    // m/2 disjoint pairs at once (rotations on disjoint index pairs commute).
-    // A rotation is skipped when |a_pq| < 1e-14 (|a_pp| + |a_qq|); the sweeps
-    // stop after a sweep without rotation (60 at most).
-    __shared__ int rotated;
-    __shared__ int pos[kMaxSub + 1];
-    __shared__ int pp[kMaxSub / 2 + 1], pq[kMaxSub / 2 + 1];
-    __shared__ double pc[kMaxSub / 2 + 1], psn[kMaxSub / 2 + 1];
-    const int me = m + (m & 1);  // even number of players; index m is a dummy when m is odd
-    const int half = me / 2;
-    for (int t = tid; t < me; t += blockDim.x) pos[t] = t;
-    __syncthreads();
-    for (int sweep = 0; sweep < 60; ++sweep) {
-        if (tid == 0) rotated = 0;
-        __syncthreads();
-        for (int step = 0; step < me - 1; ++step) {
-            for (int k = tid; k < half; k += blockDim.x) {
-                int p = pos[k], q = pos[me - 1 - k];
-                if (p > q) { const int t2 = p; p = q; q = t2; }
-                double c = 1.0, sn = 0.0;
-                if (q < m) {
-                    const double apq = a[p][q];
-                    if (fabs(apq) > 1e-14 * (fabs(a[p][p]) + fabs(a[q][q]))) {
-                        rotated = 1;
-                        const double theta = (a[q][q] - a[p][p]) / (2.0 * apq);
-                        const double tt = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                        c = 1.0 / sqrt(tt * tt + 1.0);
-                        sn = tt * c;
-                    }
-                }
-                pp[k] = p;
-                pq[k] = q;
-                pc[k] = c;
-                psn[k] = sn;
-            }
-            __syncthreads();
-            // columns: a <- a J
-            for (int t = tid; t < half * m; t += blockDim.x) {
-                const int k = t / m, r = t % m;
-                if (psn[k] == 0.0) continue;
-                const int p = pp[k], q = pq[k];
-                const double c = pc[k], sn = psn[k];
-                const double arp = a[r][p], arq = a[r][q];
-                a[r][p] = c * arp - sn * arq;
-                a[r][q] = sn * arp + c * arq;
-            }
-            __syncthreads();
-            // rows: a <- J^T a ; eigenvectors v <- v J
-            for (int t = tid; t < half * m; t += blockDim.x) {
-                const int k = t / m, r = t % m;
-                if (psn[k] == 0.0) continue;
-                const int p = pp[k], q = pq[k];
-                const double c = pc[k], sn = psn[k];
-                const double apr = a[p][r], aqr = a[q][r];
-                a[p][r] = c * apr - sn * aqr;
-                a[q][r] = sn * apr + c * aqr;
-                const double vrp = v[r][p], vrq = v[r][q];
-                v[r][p] = c * vrp - sn * vrq;
-                v[r][q] = sn * vrp + c * vrq;
-            }
-            __syncthreads();
-            // next round-robin pairing: player 0 stays, the others rotate
-            if (tid == 0) {
-                const int last = pos[me - 1];
-                for (int t = me - 1; t > 1; --t) pos[t] = pos[t - 1];
-                pos[1] = last;
-            }
-            __syncthreads();
-        }
-        if (!rotated) break;
-    }
-    if (tid == 0) {
-        for (int i = 0; i < m; ++i) order[i] = i;
-        for (int i = 1; i < m; ++i) {  // insertion sort, stable
-            int o = order[i];
-            int j = i - 1;
-            while (j >= 0 && a[order[j]][order[j]] > a[o][o]) {
-                order[j + 1] = order[j];
-                --j;
-            }
-            order[j + 1] = o;
-        }
-    }
-    __syncthreads();
-    for (int t = tid; t < m; t += blockDim.x) w[t] = a[order[t]][order[t]];
-    for (int t = tid; t < m * m; t += blockDim.x) {
-        int i = t / m, k = t % m;
-        V[i * m + k] = v[i][order[k]];
-    }
+    if (i == 31) host[16] = (double)*err;
 }
 
 // k smallest diagonal entries, ties broken by index: one pass per root over
@@ -694,10 +699,12 @@ struct Work {
     float *y32 = nullptr;                   // FP32 basis: [n] scratch
     double *A = nullptr;                    // [kMaxSub][kMaxSub] projected matrix
     double *w = nullptr, *V = nullptr;      // eigenvalues, eigenvectors
-    double *partial = nullptr;              // [kDotBlocks][32]
+    double *partial = nullptr;              // [2][kDotBlocks][32]
     double *scal = nullptr;                 // [64] scalars
     double *rn2 = nullptr;                  // [nroots] residual norms squared
     int *keep = nullptr;
+    int *counter = nullptr;                 // [4]: last-block counters (0, 1: dot sets; 2: others), 3: second-pass flag
+    double *host = nullptr;                 // pinned, the context's: [17] k_publish, [24] keep flag
     int64_t *idx = nullptr;                 // [nroots]
     int64_t *pidx = nullptr;                // [kDotBlocks + 1] reduction scratch (indices)
     int parity = 0;                         // fci_options.spin_parity (C^T = parity C), 0 = none
@@ -715,6 +722,13 @@ struct Work {
         allocs.back() = p;
         sizes.back() = p ? sizeof(P) * count : 0;
         return p;
+    }
+    // after the allocations: zero counters, the context's pinned words
+    int begin() {
+        if (!ctx->host_words) FCI_CUDA(cudaMallocHost((void **)&ctx->host_words, 32 * sizeof(double)));
+        host = ctx->host_words;
+        FCI_CUDA(cudaMemsetAsync(counter, 0, 4 * sizeof(int), s));
+        return FCI_OK;
     }
     ~Work() {
         for (size_t i = 0; i < allocs.size() && i < sizes.size(); ++i) dfree(ctx, allocs[i], sizes[i]);
@@ -752,19 +766,28 @@ void lincomb(cudaStream_t s, const double *X, int m, const double *coef, int coe
         k_lincomb<1><<<grid_for(n), 256, 0, s>>>(X, m, coef, coef_stride, beta, y, n);
 }
 
-// out[i*stride] = X_i . y for i < m (m <= 32)
-int dots(Work &W, const double *X, int m, const double *y, double *out, int stride) {
+// Dot products of the set s0 and, where s1.X is not null, of s1 (m <= 32).
+int dots2(Work &W, const DotSet &s0, const DotSet &s1, int m, const int *gate = nullptr) {
     if (m <= 0) return FCI_OK;
     if (m > 32) return fail(FCI_ERR_ARG, "subspace larger than 32 vectors");
     const int groups = (m + 7) / 8;
-    const bool vec = (W.n % 4 == 0) && ((uintptr_t)X % 32 == 0) && ((uintptr_t)y % 32 == 0);
+    auto al = [](const void *p) { return (uintptr_t)p % 32 == 0; };
+    const bool vec = W.n % 4 == 0 && al(s0.X) && al(s0.y) && (!s1.X || (al(s1.X) && al(s1.y)));
+    // four elements (or vectors of four) per thread at least
+    const int64_t units = vec ? W.n / 4 : W.n;
+    const int stripes = (int)std::min<int64_t>(kDotBlocks, std::max<int64_t>(1, (units + 1023) / 1024));
+    const dim3 grid((unsigned)(stripes * groups), s1.X ? 2 : 1);
     if (vec)
-        k_multidot<4><<<kDotBlocks * groups, 256, 0, W.s>>>(X, m, y, W.n, groups, W.partial);
+        k_multidot<4><<<grid, 256, 0, W.s>>>(s0, s1, m, W.n, groups, W.partial, W.counter, gate);
     else
-        k_multidot<1><<<kDotBlocks * groups, 256, 0, W.s>>>(X, m, y, W.n, groups, W.partial);
-    k_reduce_partials<32><<<1, 32, 0, W.s>>>(W.partial, kDotBlocks, m, out, stride);
+        k_multidot<1><<<grid, 256, 0, W.s>>>(s0, s1, m, W.n, groups, W.partial, W.counter, gate);
     FCI_CUDA(cudaGetLastError());
     return FCI_OK;
+}
+
+// out[i*stride] = X_i . y for i < m (m <= 32)
+int dots(Work &W, const double *X, int m, const double *y, double *out, int stride, const int *gate = nullptr) {
+    return dots2(W, DotSet{X, y, out, stride, m}, DotSet{nullptr, nullptr, nullptr, 0, 0}, m, gate);
 }
 
 // project y onto the spin parity (y <- (y + p y^T) / 2), if one is set
@@ -790,35 +813,31 @@ int orthonormalise(Work &W, const double *X, int m, double *y, int *kept) {
     if (m > 0) {
         const bool v2 = vec2(W.n, X, y);
         const unsigned grid = v2 ? grid_for(W.n / 2) : grid_for(W.n);
+        int *again = W.counter + 3;
         // classical Gram-Schmidt, repeated only when the first pass removed more
         // than half of ||y||^2 (DGKS criterion, ||y1|| < ||y0||/sqrt(2)); against
-        // an orthonormal basis ||y0||^2 = ||y1||^2 + sum_i c_i^2
+        // an orthonormal basis ||y0||^2 = ||y1||^2 + sum_i c_i^2.  The second pass
+        // is launched either way and looks at the first's verdict on the device:
+        // no round trip to the host
         for (int pass = 0; pass < 2; ++pass) {
-            if (int rc = dots(W, X, m, y, W.scal, 1)) return rc;
+            const int *gate = pass ? again : nullptr;
+            if (int rc = dots(W, X, m, y, W.scal, 1, gate)) return rc;
             if (v2)
-                k_sub_proj<2><<<grid, 256, 0, W.s>>>(X, m, W.scal, y, W.n, W.partial);
+                k_sub_proj<2><<<grid, 256, 0, W.s>>>(X, m, W.scal, y, W.n, W.partial, W.scal + 40, pass ? nullptr : again,
+                                                     W.counter + 2, gate);
             else
-                k_sub_proj<1><<<grid, 256, 0, W.s>>>(X, m, W.scal, y, W.n, W.partial);
-            k_reduce_partials<1><<<1, 32, 0, W.s>>>(W.partial, (int)grid, 1, W.scal + 40, 1);
+                k_sub_proj<1><<<grid, 256, 0, W.s>>>(X, m, W.scal, y, W.n, W.partial, W.scal + 40, pass ? nullptr : again,
+                                                     W.counter + 2, gate);
             FCI_CUDA(cudaGetLastError());
-            if (pass == 0) {
-                double h[41];
-                FCI_CUDA(cudaMemcpyAsync(h, W.scal, sizeof(double) * 41, cudaMemcpyDeviceToHost, W.s));
-                FCI_CUDA(cudaStreamSynchronize(W.s));
-                double c2 = 0.0;
-                for (int i = 0; i < m; ++i) c2 += h[i] * h[i];
-                if (h[40] >= c2) break;  // ||y1||^2 >= ||y0||^2 / 2: one pass suffices
-            }
         }
     } else if (int rc = dots(W, y, 1, y, W.scal + 40, 1)) {
         return rc;
     }
-    k_scale<<<grid_for(W.n), 256, 0, W.s>>>(y, W.scal + 40, 1e-10, W.keep, W.n);
+    int *keep = reinterpret_cast<int *>(W.host + 24);
+    k_scale<<<grid_for(W.n), 256, 0, W.s>>>(y, W.scal + 40, 1e-10, keep, W.n);
     FCI_CUDA(cudaGetLastError());
-    int h = 0;
-    FCI_CUDA(cudaMemcpyAsync(&h, W.keep, sizeof(int), cudaMemcpyDeviceToHost, W.s));
     FCI_CUDA(cudaStreamSynchronize(W.s));
-    *kept = h;
+    *kept = *keep;
     return FCI_OK;
 }
 
@@ -829,7 +848,7 @@ int dots_f32(Work &W, const float *X, int m, const float *y, double *out, int st
     if (m > 32) return fail(FCI_ERR_ARG, "subspace larger than 32 vectors");
     const int groups = (m + 7) / 8;
     k_multidot_f32<<<kDotBlocks * groups, 256, 0, W.s>>>(X, m, y, W.n, groups, W.partial);
-    k_reduce_partials<32><<<1, 32, 0, W.s>>>(W.partial, kDotBlocks, m, out, stride);
+    k_reduce_partials<32><<<1, 256, 0, W.s>>>(W.partial, kDotBlocks, m, out, stride);
     FCI_CUDA(cudaGetLastError());
     return FCI_OK;
 }
@@ -842,7 +861,7 @@ int orthonormalise_f32(Work &W, const float *X, int m, float *y, int *kept) {
         for (int pass = 0; pass < 2; ++pass) {
             if (int rc = dots_f32(W, X, m, y, W.scal, 1)) return rc;
             k_sub_proj_f32<<<grid, 256, 0, W.s>>>(X, m, W.scal, y, W.n, W.partial);
-            k_reduce_partials<1><<<1, 32, 0, W.s>>>(W.partial, (int)grid, 1, W.scal + 40, 1);
+            k_reduce_partials<1><<<1, 256, 0, W.s>>>(W.partial, (int)grid, 1, W.scal + 40, 1);
             FCI_CUDA(cudaGetLastError());
             if (pass == 0) {
                 double h[41];
@@ -900,13 +919,15 @@ static int run_davidson_f32basis(fci_ctx *ctx, int nroots, double tol, double *e
     W.A = W.get<double>(kMaxSub * kMaxSub);
     W.w = W.get<double>(kMaxSub);
     W.V = W.get<double>(kMaxSub * kMaxSub);
-    W.partial = W.get<double>(kDotBlocks * 32);
+    W.partial = W.get<double>(2 * kDotBlocks * 32);
     W.scal = W.get<double>(64);
     W.rn2 = W.get<double>(8);
     W.keep = W.get<int>(1);
+    W.counter = W.get<int>(4);
     W.idx = W.get<int64_t>(8);
     W.pidx = W.get<int64_t>(kDotBlocks + 1);
     if (W.rc) return W.rc;
+    if (int rc = W.begin()) return rc;
     ctx->log.clear();
     ctx->log_width = nroots + 3;
     ctx->iterations = 0;
@@ -982,7 +1003,7 @@ static int run_davidson_f32basis(fci_ctx *ctx, int nroots, double tol, double *e
     auto residuals = [&](int nr) -> int {
         for (int k = 0; k < nr; ++k) {
             k_resnorm<<<kDotBlocks, 256, 0, s>>>(W.X + (size_t)k * n, W.HX + (size_t)k * n, W.w, k, n, W.partial);
-            k_reduce_partials<1><<<1, 32, 0, s>>>(W.partial, kDotBlocks, 1, W.rn2 + k, 1);
+            k_reduce_partials<1><<<1, 256, 0, s>>>(W.partial, kDotBlocks, 1, W.rn2 + k, 1);
         }
         FCI_CUDA(cudaGetLastError());
         return FCI_OK;
@@ -1141,13 +1162,15 @@ int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *v
     W.A = W.get<double>(kMaxSub * kMaxSub);
     W.w = W.get<double>(kMaxSub);
     W.V = W.get<double>(kMaxSub * kMaxSub);
-    W.partial = W.get<double>(kDotBlocks * 32);
+    W.partial = W.get<double>(2 * kDotBlocks * 32);
     W.scal = W.get<double>(64);
     W.rn2 = W.get<double>(8);
     W.keep = W.get<int>(1);
+    W.counter = W.get<int>(4);
     W.idx = W.get<int64_t>(8);
     W.pidx = W.get<int64_t>(kDotBlocks + 1);
     if (W.rc) return W.rc;
+    if (int rc = W.begin()) return rc;
     const int64_t n = W.n;
     cudaStream_t s = W.s;
 
@@ -1204,18 +1227,23 @@ int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *v
         const int nr = nroots < m ? nroots : m;
         // Ritz vectors, their sigma, residuals and (2)-(3) preconditioned corrections
         for (int k = 0; k < nr; ++k) {
-            lincomb(s, W.Bv, m, W.V + k, m, 0.0, W.X + (size_t)k * n, n);
-            lincomb(s, W.Sv, m, W.V + k, m, 0.0, W.HX + (size_t)k * n, n);
-            k_residual_precond<<<kDotBlocks, 256, 0, s>>>(W.X + (size_t)k * n, W.HX + (size_t)k * n, ctx->hdiag, W.w,
-                                                          k, W.T + (size_t)k * n, n, W.partial);
-            k_reduce_partials<1><<<1, 32, 0, s>>>(W.partial, kDotBlocks, 1, W.rn2 + k, 1);
+            double *x = W.X + (size_t)k * n, *hx = W.HX + (size_t)k * n, *t = W.T + (size_t)k * n;
+            if (vec2(n, W.Bv, W.Sv) && vec2(n, x, hx) && vec2(n, t, ctx->hdiag))
+                k_ritz<2><<<grid_for(n / 2), 256, 0, s>>>(W.Bv, W.Sv, m, W.V, W.w, k, ctx->hdiag, x, hx, t, n, W.partial,
+                                                          W.rn2 + k, W.counter + 2);
+            else
+                k_ritz<1><<<grid_for(n), 256, 0, s>>>(W.Bv, W.Sv, m, W.V, W.w, k, ctx->hdiag, x, hx, t, n, W.partial,
+                                                      W.rn2 + k, W.counter + 2);
             FCI_CUDA(cudaGetLastError());
         }
-        FCI_CUDA(cudaMemcpyAsync(ev.data(), W.w, sizeof(double) * nr, cudaMemcpyDeviceToHost, s));
-        FCI_CUDA(cudaMemcpyAsync(rn.data(), W.rn2, sizeof(double) * nr, cudaMemcpyDeviceToHost, s));
-        int derr = 0;
-        FCI_CUDA(cudaMemcpyAsync(&derr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+        k_publish<<<1, 32, 0, s>>>(W.w, W.rn2, nr, ctx->d_err, W.host);
+        FCI_CUDA(cudaGetLastError());
         FCI_CUDA(cudaStreamSynchronize(s));
+        for (int k = 0; k < nr; ++k) {
+            ev[k] = W.host[k];
+            rn[k] = W.host[8 + k];
+        }
+        const int derr = (int)W.host[16];
         if (derr & 1) return fail(FCI_ERR_TIMEOUT, "a bounded device wait gave up inside sigma");
         if (derr) return fail(FCI_ERR_RANGE, "a level sum of the FP64 tensor-core sigma left its exact range");
         double rmax = 0.0, demax = 0.0;
@@ -1310,8 +1338,9 @@ int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *v
             // (4) new sigma (FP32 in mixed mode), new row/column of the projected matrix
             if (int rc = sigma_of(W, mixed && !fp64_tail, b, W.Sv + (size_t)m * n)) return rc;
             ++m;
-            if (int rc = dots(W, W.Bv, m, W.Sv + (size_t)(m - 1) * n, W.A + (m - 1), kMaxSub)) return rc;
-            if (int rc = dots(W, W.Sv, m, W.Bv + (size_t)(m - 1) * n, W.A + (size_t)(m - 1) * kMaxSub, 1)) return rc;
+            if (int rc = dots2(W, DotSet{W.Bv, W.Sv + (size_t)(m - 1) * n, W.A + (m - 1), kMaxSub, m},
+                               DotSet{W.Sv, W.Bv + (size_t)(m - 1) * n, W.A + (size_t)(m - 1) * kMaxSub, 1, m - 1}, m))
+                return rc;
             ++added;
         }
         if (added == 0) {

@@ -202,6 +202,7 @@ int fci_free(fci_ctx *ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     free_tables(ctx);
+    if (ctx->host_words) cudaFreeHost(ctx->host_words);
     for (auto &e : ctx->prof_ev) cudaEventDestroy(e);
     if (ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;

@@ -140,6 +140,7 @@ struct fci_ctx {
     int log_width = 0;
     int iterations = 0;
     int sigma_calls = 0;
+    double *host_words = nullptr;   // pinned host memory that the Davidson kernels report into (made on first use)
     // per-kernel timing ring (fci_profile_*)
     bool prof = false;
     std::vector<cudaEvent_t> prof_ev;    // kProfRing * (kProfMaxKernels + 1)
