@@ -70,11 +70,10 @@ RDM2_TC_TRAFFIC = ("paper_1707_04346_gb300/csrc/rdm2.cu", "k_rdm2_tc(", "dbb9c2a
 
 
 # Kernels one sigma call launches, by its profiled slots (the slots group kernels: "slice_c"
-# is the row-exponent and slicing pair, each dense same-spin product its exponent or plane
-# pass, the product and, once per call, the FP64 diagonal), counted from the ncu launch
-# lists under profiles/.  Pipelines not listed launch one kernel per slot.
+# is the row-exponent and slicing pair, the first dense same-spin product brings C's
+# exponent and plane passes), counted in the host code.  Pipelines not listed launch one kernel per slot.
 LAUNCHES_PER_SIGMA = {
-    ("slice_c", "sigma3_sliced", "sigma1_ss", "sigma2_ss"): 9,
+    ("slice_c", "sigma3_sliced", "sigma1_ss", "sigma2_ss"): 7,
     ("slice_c", "sigma3_sliced", "sigma1_rows", "sigma2_cols"): 5,
 }
 
@@ -223,16 +222,16 @@ def kernel_work(name, norb, na, nb, N, sa, sb, nsa, nsb, peaks, f32_splits=3):
         return ("alu", 12.0 * nsame * N, "Tops/s", fp32_pipe, fp32src,
                 f"FP32 operations: 12 per term x {nsame} terms per determinant")
     if name in ("sigma1_ss", "sigma2_ss"):  # FP64 same-spin terms as dense sliced products
-        # one GEMM of (strings of the summed spin) x (other spin) x (summed spin), 21 digit
-        # products, tiles of 128 x 48 rows (the plane rows padded to 384) and the FP64 diagonal
+        # one product of (strings of the summed spin) x (other spin) x (summed spin) in 21 digit
+        # products, zeros of the same-spin Hamiltonian included (K-steps that hold only zeros are
+        # not executed)
         ns_sum = nsb if name == "sigma1_ss" else nsa
-        mt, nt = -(-nsb // 128), -(-nsa // 48)  # output tiles: beta strings x alpha strings
-        f = 21 * 2.0 * 128 * 48 * (-(-ns_sum // 16) * 16) * mt * nt
-        return ("tensor", f, "TFLOP/s", *bf16,
-                f"bf16 MMA FLOP: 21 digit products x 2 x 128 x 48 x {-(-ns_sum // 16) * 16} x {mt * nt} tiles")
-    if name == "sigma12_f32":  # FP32 sigma_1 + sigma_2: one FMA per term
-        return ("alu", 2.0 * nsame * N, "Tops/s", fp32_pipe, fp32src,
-                f"FP32 FMAs: {nsame} terms per determinant, two spins")
+        return ("tensor", 21 * 2.0 * ns_sum * N, "TFLOP/s", *bf16,
+                f"bf16 FLOP: 21 digit products x 2 x {ns_sum} per determinant, zeros included")
+    if name in ("sigma12_ss32", "sigma2_ss32"):  # FP32 same-spin terms as dense products of 3 bf16 slices
+        ns_sum = nsa + nsb if name == "sigma12_ss32" else nsa
+        return ("tensor", 6 * 2.0 * ns_sum * N, "TFLOP/s", *bf16,
+                f"bf16 FLOP: 6 slice products x 2 x {ns_sum} per determinant, zeros included")
     if name == "sigma3_tc":
         return ("tensor", prods32 * 2.0 * 128 * npad * kpad * tiles, "TFLOP/s", *bf16,
                 f"bf16 MMA FLOP: {prods32} slice products x 2 x 128 x {npad} x {kpad} x {tiles} tiles")

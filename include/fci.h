@@ -412,7 +412,9 @@ int fci_tile_schedule(int64_t ns, int nsingle, int npair, const int32_t *tgt, co
  * oldest first (at most cap_records), then empties the ring.
  * fci_profile_kernel_name names kernel slot i of the current sigma pipeline
  * (NULL if out of range).  Enabling allocates the events (FCI_ERR_CUDA on
- * failure); disabling keeps them for reuse.
+ * failure); disabling keeps them for reuse.  Small spaces, whose sigma is one
+ * fused kernel, run the kernels of larger spaces (one per term, the same
+ * accuracy, other roundings) while profiling is enabled.
  */
 int fci_profile_enable(fci_ctx *ctx, int on);
 int fci_profile_read(fci_ctx *ctx, double *ms, int cap_records, int *nrecords, int *nkernels);

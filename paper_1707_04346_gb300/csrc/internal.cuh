@@ -82,7 +82,7 @@ struct SpinTables {
     bool owner = true;         // false when aliasing the alpha tables
 };
 
-// Digit planes of one spin's G_s (sigma_ss.cu): blocks of nb rows, each with the
+// Operand planes of one spin's G_s (sigma_ss.cu, sigma_ss32.cu): blocks of nb rows, each with the
 // K-steps that hold a nonzero.
 struct SsOperand {
     unsigned char *planes = nullptr;
@@ -91,6 +91,7 @@ struct SsOperand {
     size_t list_bytes = 0;
     int *e = nullptr;      // biased exponent of each row
     int nb = 0, nnb = 0;
+    size_t nsteps = 0;     // K-steps kept, all blocks
 };
 
 }  // namespace fci
@@ -131,6 +132,10 @@ struct fci_ctx {
     // their exponents
     fci::SsOperand ssGa, ssGb;
     unsigned char *ssCr = nullptr, *ssCc = nullptr;
+    size_t ssCr_bytes = 0, ssCc_bytes = 0;
+    // FP32 same-spin terms as dense products (sigma_ss32.cu): bf16 slices of G_s
+    fci::SsOperand ss32Ga, ss32Gb;
+    int ss32_rows = 0;
     int *ssEr = nullptr, *ssEc = nullptr;
     double *hdiag = nullptr;        // [ndet]
     int *d_err = nullptr;           // device error word (bounded waits that gave up)
@@ -225,6 +230,23 @@ int build_ss_tables(fci_ctx *ctx);
 void free_ss_tables(fci_ctx *ctx);
 // sigma += sigma_1 (which & 1) then sigma_2 (which & 2); profiling slots slot, slot + 1
 int launch_sigma_ss(fci_ctx *ctx, const double *C, double *sig, int which, cudaStream_t s, int rec, int slot);
+
+int ss_kstep_lists(fci_ctx *ctx, const SpinTables &T, int nb, SsOperand &O, int **slot, size_t *slot_bytes);
+int alloc_c_planes(fci_ctx *ctx, size_t row_bytes, size_t col_bytes);
+void free_ss_operand(fci_ctx *ctx, SsOperand &O, int64_t ns);
+
+// sigma_ss32.cu (FP32 sigma_1 / sigma_2 as dense tensor-core products)
+bool sigma_ss32_ok(const fci_ctx *ctx);
+int build_ss32_tables(fci_ctx *ctx);
+void free_ss32_tables(fci_ctx *ctx);
+// sigma = sigma_1 (which & 1) + sigma_2 (which & 2) with the diagonals of the
+// spins named; overwritten.  active: as for launch_sigma3_tc
+int launch_sigma_ss32(fci_ctx *ctx, const float *C, float *sig, int which, cudaStream_t s, const int *active = nullptr);
+
+// sigma_small.cu (all three terms in one kernel; opted in at fci_init)
+bool sigma_small_ok(const fci_ctx *ctx, int dtype);
+int prepare_sigma_small(const fci_ctx *ctx);
+int launch_sigma_small(fci_ctx *ctx, const void *C, void *sig, int dtype, cudaStream_t s, const int *active = nullptr);
 
 // davidson.cu
 int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *vecs, const void *guess);

@@ -23,20 +23,6 @@ namespace fci {
 
 constexpr int kEnt = 8;  // ELL entries whose table loads are issued together (FP32)
 
-// Table loads issued as volatile asm, so that a batch of them stays together in
-// program order ahead of its first use whatever the compiler's scheduling (the
-// fused FP32 kernel lost a third of its speed to a schedule change once).
-__device__ __forceinline__ int32_t ld_batch_s32(const int32_t *p) {
-    int32_t v;
-    asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float ld_batch_f32(const float *p) {
-    float v;
-    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
 template <typename T>
 __device__ __forceinline__ T gval_of(const SpinTables &S, int64_t idx);
 template <>
@@ -294,69 +280,6 @@ __global__ void __launch_bounds__(512, 1) k_sigma2_cols_df(const double *__restr
     }
 }
 
-// FP32 sigma_1 + sigma_2 in one pass when both spins share one string space
-// (n_alpha = n_beta, identical same-spin tables): a block stages R rows and
-// the same R columns of C, and every ELL entry it reads updates both,
-//   sigma(r0+r, x) += G[x][col] C(r0+r, col)      (sigma_1, row r0+r)
-//   sigma(x, r0+r) += G[x][col] C(col, r0+r)      (sigma_2, column r0+r)
-// which halves the table traffic that bounds the separate FP32 kernels.  Two
-// blocks meet on each element (its row block and its column block), so sigma
-// starts at zero and both adds are atomic; two addends onto zero give the
-// same sum in either order.
-template <int R>
-__global__ void __launch_bounds__(512) k_sigma12_f32(const float *__restrict__ C, float *__restrict__ sig,
-                                                     SpinTables S, const int *__restrict__ active) {
-    if (active != nullptr && *active == 0) return;  // gated launch (batched engine): instance not active
-    extern __shared__ float smf[];
-    const int64_t ns = S.ns;
-    float *rows = smf;           // [R][ns]
-    float *cols = smf + R * ns;  // [R][ns]
-    const int64_t r0 = (int64_t)blockIdx.x * R;
-    for (int64_t t = threadIdx.x; t < (int64_t)R * ns; t += blockDim.x) {
-        const int64_t r = t / ns, j = t % ns;
-        rows[t] = (r0 + r < ns) ? C[(r0 + r) * ns + j] : 0.f;
-    }
-    for (int64_t i = threadIdx.x; i < ns; i += blockDim.x) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) cols[(int64_t)r * ns + i] = (r0 + r < ns) ? C[i * ns + r0 + r] : 0.f;
-    }
-    __syncthreads();
-    for (int64_t x = threadIdx.x; x < ns; x += blockDim.x) {
-        float ar[R], ac[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) ar[r] = ac[r] = 0.f;
-        for (int e0 = 0; e0 < S.nsame; e0 += kEnt) {
-            int32_t col[kEnt];
-            float v[kEnt];
-#pragma unroll
-            for (int u = 0; u < kEnt; ++u) {  // in-range addresses; padding slots zeroed after the loads
-                const int64_t idx = (int64_t)(e0 + u < S.nsame ? e0 + u : 0) * ns + x;
-                col[u] = ld_batch_s32(S.gcol + idx);
-                v[u] = ld_batch_f32(S.gvalf + idx);
-            }
-#pragma unroll
-            for (int u = 0; u < kEnt; ++u)
-                if (e0 + u >= S.nsame) {
-                    col[u] = 0;
-                    v[u] = 0.f;
-                }
-#pragma unroll
-            for (int u = 0; u < kEnt; ++u)
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    ar[r] = fmaf(v[u], rows[(int64_t)r * ns + col[u]], ar[r]);
-                    ac[r] = fmaf(v[u], cols[(int64_t)r * ns + col[u]], ac[r]);
-                }
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (r0 + r < ns) {
-                atomicAdd(sig + (r0 + r) * ns + x, ar[r]);
-                atomicAdd(sig + x * ns + r0 + r, ac[r]);
-            }
-    }
-}
-
 // out[c][r] = in[r][c] (ADD: out[c][r] += in[r][c]) for a rows x cols matrix,
 // through 32 x 32 tiles in shared memory (block 32 x 8).
 template <bool ADD>
@@ -501,16 +424,16 @@ static size_t smem_limit() {
 }
 
 // Whether FP32 sigma_1/sigma_2 run through intermediate strings on the tensor
-// cores (asked for, or the staged same-spin kernels do not fit); that path
+// cores (asked for, or neither the dense products nor the staged same-spin
+// kernels fit); that path
 // needs the 2N-float workspace ws32, which fci_init allocates.
 bool f32_same_spin_tc(const fci_ctx *ctx) {
     const SpinTables &A = ctx->A, &B = ctx->B;
     const size_t lim = smem_limit();
     auto fits = [&](int r, int64_t len) { return (size_t)r * len * sizeof(float) <= lim; };
-    const bool fused = A.ne == B.ne && A.ns == B.ns && fits(8, A.ns);  // 2 x 4 rows of the fused kernel
     const bool tc_ok = A.nsingle > 0 && B.nsingle > 0 && ctx->npair + 1 <= 256 && A.nsingle <= 96 &&
                        B.nsingle <= 96;
-    return tc_ok && (ctx->opt.same_spin_tc == 1 || (!fused && (A.ne == B.ne || !fits(4, B.ns) || !fits(4, A.ns))));
+    return tc_ok && (ctx->opt.same_spin_tc == 1 || (!sigma_ss32_ok(ctx) && (!fits(4, B.ns) || !fits(4, A.ns))));
 }
 
 int alloc_sigma_workspace(fci_ctx *ctx) {
@@ -523,6 +446,10 @@ int alloc_sigma_workspace(fci_ctx *ctx) {
 template <typename T>
 static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int parity) {
     const SpinTables &A = ctx->A, &B = ctx->B;
+    // small spaces: one kernel for all terms (the kernels of larger spaces, one per
+    // term, while their times are being recorded)
+    if (!ctx->prof && sigma_small_ok(ctx, sizeof(T) == 8 ? FCI_F64 : FCI_F32))
+        return launch_sigma_small(ctx, C, sig, sizeof(T) == 8 ? FCI_F64 : FCI_F32, s);
     // a vector of known spin parity (C^T = parity C, one string space): sigma_1 from sigma_2
     if (A.ne != B.ne || A.ns != B.ns) parity = 0;
     if constexpr (sizeof(T) == 8)
@@ -535,18 +462,15 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
             if ((size_t)r * len * sizeof(T) <= lim) return r;
         return 0;
     };
-    // FP32 with one string space for both spins: fused sigma_1 + sigma_2
-    int fusedR = 0;
-    if (sizeof(T) == 4 && A.ne == B.ne && nsa == nsb)
-        for (int r : {8, 4})
-            if (!fusedR && (size_t)2 * r * nsa * sizeof(float) <= lim) fusedR = r;
     // FP32 same-spin terms through intermediate strings on the tensor cores: when
     // asked for, or when the staged kernels above do not fit (large string spaces)
     const bool same_tc = sizeof(T) == 4 && f32_same_spin_tc(ctx);
-    // profiled kernels (fci_profile_read): two slots when fused, else three
+    // both FP32 same-spin terms as dense tensor-core products in one launch
+    const bool ss32 = sizeof(T) == 4 && !same_tc && sigma_ss32_ok(ctx);
+    // profiled kernels (fci_profile_read)
     static const char *const names3[3] = {"sigma1_rows", "sigma2_cols", sizeof(T) == 4 ? "sigma3_tc" : "sigma3_exact"};
     static const char *const names3tc[3] = {"sigma2_tc", "sigma1_tc", "sigma3_tc"};
-    static const char *const names2[2] = {"sigma12_f32", "sigma3_tc"};
+    static const char *const names2ss[2] = {"sigma12_ss32", "sigma3_tc"};
     static const char *const names4[4] = {"slice_c", "sigma3_sliced", "sigma1_rows", "sigma2_cols"};
     // FP64 with the sliced tensor-core sigma_3: it runs first and overwrites sigma
     const bool sliced = sizeof(T) == 8 && A.nsingle > 0 && B.nsingle > 0 && ctx->opt.f64_kernels != FCI_F64_FMA &&
@@ -583,6 +507,16 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
                 prof_mark(ctx, rec, 1, s);
                 return launch_sigma3_sliced(ctx, C, sig, s, rec, 2, nullptr, 1);
             }
+        } else if (ss32) {
+            static const char *const namesp[3] = {"sigma2_ss32", "sigma1_sym", "sigma3_tc"};
+            const int rec = prof_begin(ctx, s, 3, namesp);
+            if (int rc = launch_sigma_ss32(ctx, (const float *)C, (float *)sig, 2, s)) return rc;
+            prof_mark(ctx, rec, 0, s);
+            if (int rc = sym_pairs(sig, nsa, 4, parity, 0, s)) return rc;
+            prof_mark(ctx, rec, 1, s);
+            if (int rc = launch_sigma3_tc(ctx, (const float *)C, (float *)sig, ctx->opt.f32_splits, s)) return rc;
+            prof_mark(ctx, rec, 2, s);
+            return FCI_OK;
         } else if (same_tc) {
             static const char *const namesp[3] = {"sigma2_tc", "sigma1_sym", "sigma3_tc"};
             const int rec = prof_begin(ctx, s, 3, namesp);
@@ -600,9 +534,10 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
     const bool ss = sliced && sigma_ss_ok(ctx);
     const int rec = ss ? prof_begin(ctx, s, 4, names4ss)
                     : sliced ? prof_begin(ctx, s, 4, names4)
+                    : ss32 ? prof_begin(ctx, s, 2, names2ss)
                     : same_tc ? prof_begin(ctx, s, 3, names3tc)
-                    : fusedR ? prof_begin(ctx, s, 2, names2) : prof_begin(ctx, s, 3, names3);
-    const int slot3 = (fusedR && !same_tc) ? 1 : 2;
+                             : prof_begin(ctx, s, 3, names3);
+    const int slot3 = ss32 ? 1 : 2;
     int slot = 0;  // next profiling slot of the staged same-spin kernels
     int add1 = 0;  // sigma_1 adds to what sigma_3 wrote
     if (sliced) {
@@ -613,7 +548,11 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
         slot = 2;
         add1 = 1;
     }
-    if (same_tc) {
+    if (ss32) {
+        if constexpr (sizeof(T) == 4)
+            if (int rc = launch_sigma_ss32(ctx, (const float *)C, (float *)sig, 3, s)) return rc;
+        prof_mark(ctx, rec, 0, s);
+    } else if (same_tc) {
         if constexpr (sizeof(T) == 4) {
             if (!ctx->ws32) return fail(FCI_ERR_STATE, "FP32 same-spin workspace missing (made at fci_init)");
             float *Ct = ctx->ws32, *Tt = ctx->ws32 + ctx->ndet;
@@ -630,16 +569,6 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
             FCI_CUDA(cudaGetLastError());
             prof_mark(ctx, rec, 1, s);
         }
-    } else if (fusedR) {
-        const size_t sm = (size_t)2 * fusedR * nsa * sizeof(float);
-        void *k = fusedR == 8 ? (void *)k_sigma12_f32<8> : (void *)k_sigma12_f32<4>;
-        FCI_CUDA(opt_in_max_smem(k, ctx->device));
-        FCI_CUDA(cudaMemsetAsync(sig, 0, sizeof(float) * (size_t)nsa * (size_t)nsb, s));
-        SpinTables St = A;
-        const int *no_gate = nullptr;
-        void *args[] = {(void *)&C, (void *)&sig, (void *)&St, (void *)&no_gate};
-        FCI_CUDA(cudaLaunchKernel(k, dim3(ceil_div(nsa, fusedR)), dim3(512), args, sm, s));
-        prof_mark(ctx, rec, 0, s);
     } else {
         {
             const int R = pick_r(nsb);
@@ -695,39 +624,21 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
 }
 
 // FP32 sigma of one instance of the batched engine, skipped on the device
-// when *active == 0 (so that a captured graph serves any active set).  Only
-// for one string space (fused sigma_1 + sigma_2) with the tensor-core sigma_3;
-// sigma is zeroed even when the instance is skipped.  The kernels' shared
-// memory limits are set once by prepare_sigma_f32_gated (outside any capture).
+// when *active == 0 (so that a captured graph serves any active set): the
+// one-kernel sigma of small spaces, else the dense same-spin products and the
+// tensor-core sigma_3 (sigma is then zeroed even when the instance is skipped).  The kernels' shared memory limits are set once by
+// prepare_sigma_f32_gated (outside any capture).
 bool sigma_f32_gated_ok(const fci_ctx *ctx) {
-    const SpinTables &A = ctx->A, &B = ctx->B;
-    if (A.ne != B.ne || A.ns != B.ns || A.nsingle == 0 || B.nsingle == 0) return false;
-    if ((size_t)2 * 4 * A.ns * sizeof(float) > smem_limit()) return false;
-    return sigma3_tc_smem(ctx, ctx->opt.f32_splits) > 0;
-}
-
-static void *gated_sigma12(int64_t ns, size_t *sm) {
-    const int R = (size_t)2 * 8 * ns * sizeof(float) <= smem_limit() ? 8 : 4;
-    *sm = (size_t)2 * R * ns * sizeof(float);
-    return R == 8 ? (void *)k_sigma12_f32<8> : (void *)k_sigma12_f32<4>;
+    return sigma_small_ok(ctx, FCI_F32) || (sigma_ss32_ok(ctx) && sigma3_tc_smem(ctx, ctx->opt.f32_splits) > 0);
 }
 
 int prepare_sigma_f32_gated(const fci_ctx *ctx) {
-    size_t sm = 0;
-    void *k = gated_sigma12(ctx->A.ns, &sm);
-    FCI_CUDA(opt_in_max_smem(k, ctx->device));
-    return prepare_sigma3_tc(ctx, ctx->opt.f32_splits);
+    return sigma_small_ok(ctx, FCI_F32) ? FCI_OK : prepare_sigma3_tc(ctx, ctx->opt.f32_splits);
 }
 
 int launch_sigma_f32_gated(fci_ctx *ctx, const float *C, float *sig, const int *active, cudaStream_t s) {
-    const int64_t ns = ctx->A.ns;
-    size_t sm = 0;
-    void *k = gated_sigma12(ns, &sm);
-    const int R = sm == (size_t)2 * 8 * ns * sizeof(float) ? 8 : 4;
-    FCI_CUDA(cudaMemsetAsync(sig, 0, sizeof(float) * (size_t)ns * (size_t)ns, s));
-    SpinTables St = ctx->A;
-    void *args[] = {(void *)&C, (void *)&sig, (void *)&St, (void *)&active};
-    FCI_CUDA(cudaLaunchKernel(k, dim3(ceil_div(ns, R)), dim3(512), args, sm, s));
+    if (sigma_small_ok(ctx, FCI_F32)) return launch_sigma_small(ctx, C, sig, FCI_F32, s, active);
+    if (int rc = launch_sigma_ss32(ctx, C, sig, 3, s, active)) return rc;
     return launch_sigma3_tc(ctx, C, sig, ctx->opt.f32_splits, s, active);
 }
 

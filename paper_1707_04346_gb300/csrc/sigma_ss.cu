@@ -173,8 +173,8 @@ __global__ void k_ss_cexp(const double *__restrict__ C, int64_t nrows, int64_t n
 // C's planes by rows (plane row = row of C, k = column; nullptr: not wanted) and
 // by columns (plane row = column of C, k = row), both from one read of a 64 x 64
 // tile of C through shared memory; 8 threads write the 128 bytes of 8 rows' core
-// matrix.  Rows past the matrix are written as zeros up to the end of a 64-row
-// tile (the planes' padding beyond starts at zero), columns past it as zeros.
+// matrix.  Plane rows and columns past the matrix are written as zeros up to the
+// ends of the 128-row tiles and K-steps (the grid covers them).
 __global__ void __launch_bounds__(256) k_ss_cplanes(const double *__restrict__ C, int64_t nrows, int64_t ncols,
                                                     const int *__restrict__ erow, const int *__restrict__ ecol,
                                                     unsigned char *__restrict__ prow, unsigned char *__restrict__ pcol) {
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256) k_ss_cplanes(const double *__restrict__ C
         const int x = it & 63, g = (it >> 6) & 7;  // plane row of the tile, group of 8 k
         const int64_t r = (cols ? c0 : r0) + x, k0 = (cols ? r0 : c0) + g * 8;
         const int64_t rows = cols ? ncols : nrows, klen = cols ? nrows : ncols;
-        if (k0 >= (klen + 15) / 16 * 16) continue;
+        if (k0 >= (klen + 15) / 16 * 16 || r >= (rows + kM - 1) / kM * kM) continue;
         const int e = r < rows ? (cols ? ecol[r] : erow[r]) : 0;
         uint32_t w[kSlices][4];
 #pragma unroll
@@ -515,6 +515,46 @@ bool sigma_ss_ok(const fci_ctx *ctx) { return ctx->ssGa.planes != nullptr; }
 // Rows of G per tile: 96 where its tiles fill half of the chip, else 16.
 static int tile_rows(int64_t M, int64_t N, int nsm) { return ss::nblocks(M, ss::kM) * ss::nblocks(N, 96) * 2 >= nsm ? 96 : 16; }
 
+// The K-steps of every block of nb rows of G_s that hold a nonzero (every block
+// keeps at least one), into O.lists, and on the device for each (block, K-step)
+// its place in the planes, *slot (to be freed by the caller).
+int ss_kstep_lists(fci_ctx *ctx, const SpinTables &T, int nb, SsOperand &O, int **slot, size_t *slot_bytes) {
+    int rc = FCI_OK;
+    cudaStream_t s = ctx->stream;
+    const int64_t nks = ss::ksteps(T.ns), nnb = ss::nblocks(T.ns, nb);
+    std::vector<unsigned char> used((size_t)(nnb * nks));
+    std::vector<int> place(used.size(), 0), tab;
+    O.nb = nb;
+    O.nnb = (int)nnb;
+    O.list_bytes = sizeof(int) * (size_t)(nnb + 1 + nnb * nks);
+    O.lists = (int *)dalloc(ctx, O.list_bytes, &rc);  // koff [nnb + 1], kidx
+    *slot_bytes = sizeof(int) * place.size();
+    *slot = (int *)dalloc(ctx, *slot_bytes, &rc);
+    if (rc) return rc;
+    unsigned char *dused = reinterpret_cast<unsigned char *>(*slot);  // read back before the places go there
+    FCI_CUDA(cudaMemsetAsync(dused, 0, used.size(), s));
+    ss::k_ss_used<<<ceil_div(T.ns * (int64_t)T.nsame, 256), 256, 0, s>>>(T.gcol, T.gval, T.ns, T.nsame, nb, nks, dused);
+    FCI_CUDA(cudaGetLastError());
+    FCI_CUDA(cudaMemcpyAsync(used.data(), dused, used.size(), cudaMemcpyDeviceToHost, s));
+    FCI_CUDA(cudaStreamSynchronize(s));
+    std::vector<int> kidx;
+    tab.push_back(0);
+    for (int64_t b = 0; b < nnb; ++b) {
+        for (int64_t k = 0; k < nks; ++k)
+            if (used[b * nks + k] || (k == nks - 1 && (int)kidx.size() == tab.back())) {
+                place[b * nks + k] = (int)kidx.size();
+                kidx.push_back((int)k);
+            }
+        tab.push_back((int)kidx.size());
+    }
+    O.nsteps = kidx.size();
+    tab.insert(tab.end(), kidx.begin(), kidx.end());
+    FCI_CUDA(cudaMemcpyAsync(O.lists, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, s));
+    FCI_CUDA(cudaMemcpyAsync(*slot, place.data(), *slot_bytes, cudaMemcpyHostToDevice, s));
+    FCI_CUDA(cudaStreamSynchronize(s));
+    return FCI_OK;
+}
+
 int build_ss_tables(fci_ctx *ctx) {
     const SpinTables &A = ctx->A, &B = ctx->B;
     if (ctx->opt.f64_same_spin == FCI_SS_FAMILY) return FCI_OK;
@@ -524,56 +564,26 @@ int build_ss_tables(fci_ctx *ctx) {
     FCI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     const bool shared = (&A == &B) || (A.gval == B.gval);
     auto build = [&](const SpinTables &T, int64_t M, SsOperand &O) -> int {
-        const int nb = O.nb = tile_rows(M, T.ns, nsm);
-        const int64_t nks = ss::ksteps(T.ns), nnb = ss::nblocks(T.ns, nb);
-        const unsigned ell = ceil_div(T.ns * (int64_t)T.nsame, 256);
-        // the K-steps of each row block that hold a nonzero (every block keeps at
-        // least one)
-        std::vector<unsigned char> used((size_t)(nnb * nks));
-        std::vector<int> slot(used.size(), 0), tab;
-        O.list_bytes = sizeof(int) * (size_t)(nnb + 1 + nnb * nks);
-        O.lists = (int *)dalloc(ctx, O.list_bytes, &rc);  // koff [nnb + 1], kidx
-        O.e = (int *)dalloc(ctx, sizeof(int) * (size_t)T.ns, &rc);
-        int *dslot = (int *)dalloc(ctx, sizeof(int) * slot.size(), &rc);
-        unsigned char *dused = reinterpret_cast<unsigned char *>(dslot);  // read back before the slots go there
-        auto done = [&](int code) {
-            dfree(ctx, dslot, sizeof(int) * slot.size());
-            return code;
-        };
-        if (rc) return done(rc);
-        cudaError_t e = cudaMemsetAsync(dused, 0, used.size(), s);
-        if (e == cudaSuccess) {
-            ss::k_ss_used<<<ell, 256, 0, s>>>(T.gcol, T.gval, T.ns, T.nsame, nb, nks, dused);
+        const int nb = tile_rows(M, T.ns, nsm);
+        int *slot = nullptr;
+        size_t slot_bytes = 0;
+        auto fill = [&]() -> int {
+            if (int r = ss_kstep_lists(ctx, T, nb, O, &slot, &slot_bytes)) return r;
+            O.plane_bytes = O.nsteps * (size_t)(6 * nb * 32);
+            O.planes = (unsigned char *)dalloc(ctx, O.plane_bytes, &rc);
+            O.e = (int *)dalloc(ctx, sizeof(int) * (size_t)T.ns, &rc);
+            if (rc) return rc;
+            FCI_CUDA(cudaMemsetAsync(O.planes, 0, O.plane_bytes, s));
             ss::k_ss_rowexp<<<ceil_div(T.ns, 256), 256, 0, s>>>(T.gval, T.ns, T.nsame, O.e);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(used.data(), dused, used.size(), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return done(cuda_fail(e, "same-spin K-step lists"));
-        std::vector<int> koff(1, 0), kidx;
-        for (int64_t b = 0; b < nnb; ++b) {
-            for (int64_t k = 0; k < nks; ++k)
-                if (used[b * nks + k] || (k == nks - 1 && (int)kidx.size() == koff.back())) {
-                    slot[b * nks + k] = (int)kidx.size();
-                    kidx.push_back((int)k);
-                }
-            koff.push_back((int)kidx.size());
-        }
-        tab = koff;
-        tab.insert(tab.end(), kidx.begin(), kidx.end());
-        O.nnb = (int)nnb;
-        O.plane_bytes = kidx.size() * (size_t)(6 * nb * 32);
-        O.planes = (unsigned char *)dalloc(ctx, O.plane_bytes, &rc);
-        if (rc) return done(rc);
-        e = cudaMemcpyAsync(O.lists, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dslot, slot.data(), sizeof(int) * slot.size(), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(O.planes, 0, O.plane_bytes, s);
-        if (e == cudaSuccess) {
-            ss::k_ss_gplanes<<<ell, 256, 0, s>>>(T.gcol, T.gval, T.ns, T.nsame, O.e, nb, nks, dslot, O.planes);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        return done(e == cudaSuccess ? FCI_OK : cuda_fail(e, "same-spin planes"));
+            ss::k_ss_gplanes<<<ceil_div(T.ns * (int64_t)T.nsame, 256), 256, 0, s>>>(
+                T.gcol, T.gval, T.ns, T.nsame, O.e, nb, ss::ksteps(T.ns), slot, O.planes);
+            FCI_CUDA(cudaGetLastError());
+            FCI_CUDA(cudaStreamSynchronize(s));
+            return FCI_OK;
+        };
+        const int r = fill();
+        dfree(ctx, slot, slot_bytes);
+        return r;
     };
     if ((rc = build(A, B.ns, ctx->ssGa))) return rc;
     if (shared)
@@ -581,33 +591,47 @@ int build_ss_tables(fci_ctx *ctx) {
     else if ((rc = build(B, A.ns, ctx->ssGb)))
         return rc;
     // per-call workspace: C by rows (K = J_b) and by columns (K = J_a), and their exponents
-    ctx->ssCr = (unsigned char *)dalloc(ctx, ss::c_bytes(A.ns, B.ns), &rc);
-    ctx->ssCc = (unsigned char *)dalloc(ctx, ss::c_bytes(B.ns, A.ns), &rc);
+    if ((rc = alloc_c_planes(ctx, ss::c_bytes(A.ns, B.ns), ss::c_bytes(B.ns, A.ns)))) return rc;
     ctx->ssEr = (int *)dalloc(ctx, sizeof(int) * (size_t)(A.ns + B.ns + 1), &rc);
     if (rc) return rc;
     ctx->ssEc = ctx->ssEr + A.ns;
-    // plane padding (rows past the strings, K past the last string) stays zero
-    FCI_CUDA(cudaMemsetAsync(ctx->ssCr, 0, ss::c_bytes(A.ns, B.ns), s));
-    FCI_CUDA(cudaMemsetAsync(ctx->ssCc, 0, ss::c_bytes(B.ns, A.ns), s));
     FCI_CUDA(opt_in_max_smem((const void *)ss::k_ss_tc<96>, ctx->device));
     FCI_CUDA(opt_in_max_smem((const void *)ss::k_ss_tc<16>, ctx->device));
-    FCI_CUDA(cudaStreamSynchronize(s));
     return FCI_OK;
+}
+
+// The operand planes of C by rows and by columns, shared by the FP64 and the FP32
+// products (each call writes all of what it reads): made, or made larger.
+int alloc_c_planes(fci_ctx *ctx, size_t row_bytes, size_t col_bytes) {
+    int rc = FCI_OK;
+    if (row_bytes > ctx->ssCr_bytes) {
+        dfree(ctx, ctx->ssCr, ctx->ssCr_bytes);
+        ctx->ssCr = (unsigned char *)dalloc(ctx, row_bytes, &rc);
+        ctx->ssCr_bytes = rc ? 0 : row_bytes;
+    }
+    if (!rc && col_bytes > ctx->ssCc_bytes) {
+        dfree(ctx, ctx->ssCc, ctx->ssCc_bytes);
+        ctx->ssCc = (unsigned char *)dalloc(ctx, col_bytes, &rc);
+        ctx->ssCc_bytes = rc ? 0 : col_bytes;
+    }
+    return rc;
+}
+
+void free_ss_operand(fci_ctx *ctx, SsOperand &O, int64_t ns) {
+    dfree(ctx, O.planes, O.plane_bytes);
+    dfree(ctx, O.lists, O.list_bytes);
+    dfree(ctx, O.e, sizeof(int) * (size_t)ns);
+    O = SsOperand{};
 }
 
 void free_ss_tables(fci_ctx *ctx) {
     const SpinTables &A = ctx->A, &B = ctx->B;
-    auto drop = [&](SsOperand &O, int64_t ns) {
-        dfree(ctx, O.planes, O.plane_bytes);
-        dfree(ctx, O.lists, O.list_bytes);
-        dfree(ctx, O.e, sizeof(int) * (size_t)ns);
-        O = SsOperand{};
-    };
-    if (ctx->ssGb.e != ctx->ssGa.e) drop(ctx->ssGb, B.ns);
+    if (ctx->ssGb.lists != ctx->ssGa.lists) free_ss_operand(ctx, ctx->ssGb, B.ns);
     ctx->ssGb = SsOperand{};
-    drop(ctx->ssGa, A.ns);
-    dfree(ctx, ctx->ssCr, ss::c_bytes(A.ns, B.ns));
-    dfree(ctx, ctx->ssCc, ss::c_bytes(B.ns, A.ns));
+    free_ss_operand(ctx, ctx->ssGa, A.ns);
+    dfree(ctx, ctx->ssCr, ctx->ssCr_bytes);
+    dfree(ctx, ctx->ssCc, ctx->ssCc_bytes);
+    ctx->ssCr_bytes = ctx->ssCc_bytes = 0;
     dfree(ctx, ctx->ssEr, sizeof(int) * (size_t)(A.ns + B.ns + 1));
     ctx->ssCr = ctx->ssCc = nullptr;
     ctx->ssEr = ctx->ssEc = nullptr;
@@ -651,7 +675,7 @@ int launch_sigma_ss(fci_ctx *ctx, const double *C, double *sig, int which, cudaS
     FCI_CUDA(cudaMemsetAsync(ctx->ssEr, 0, sizeof(int) * (size_t)(nsa + nsb), s));
     ss::k_ss_cexp<<<dim3(ceil_div(nsb, 32), ceil_div(nsa, 32)), dim3(32, 8), 0, s>>>(C, nsa, nsb, ctx->ssEr, ctx->ssEc);
     FCI_CUDA(cudaGetLastError());
-    ss::k_ss_cplanes<<<dim3(ceil_div(nsb, 64), ceil_div(nsa, 64)), 256, 0, s>>>(
+    ss::k_ss_cplanes<<<dim3(2 * ceil_div(nsb, ss::kM), 2 * ceil_div(nsa, ss::kM)), 256, 0, s>>>(
         C, nsa, nsb, ctx->ssEr, ctx->ssEc, which & 1 ? ctx->ssCr : nullptr, which & 2 ? ctx->ssCc : nullptr);
     FCI_CUDA(cudaGetLastError());
     if (which & 1) {  // sigma_1: A = C by rows (m = I_a), B = G_b (n = I_b), K = J_b
