@@ -725,7 +725,7 @@ struct Work {
     }
     // after the allocations: zero counters, the context's pinned words
     int begin() {
-        if (!ctx->host_words) FCI_CUDA(cudaMallocHost((void **)&ctx->host_words, 32 * sizeof(double)));
+        if (int r = host_words(ctx)) return r;
         host = ctx->host_words;
         FCI_CUDA(cudaMemsetAsync(counter, 0, 4 * sizeof(int), s));
         return FCI_OK;

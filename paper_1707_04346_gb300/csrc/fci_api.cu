@@ -57,6 +57,11 @@ void dfree(fci_ctx *ctx, void *p, size_t bytes) {
     ctx->bytes -= bytes;
 }
 
+int host_words(fci_ctx *ctx) {
+    if (!ctx->host_words) FCI_CUDA(cudaMallocHost((void **)&ctx->host_words, kHostWords * sizeof(double)));
+    return FCI_OK;
+}
+
 int unpack_table(fci_ctx *ctx, int spin, int32_t *tgt, int8_t *k, int8_t *l, int8_t *sg);
 
 int prof_begin(fci_ctx *ctx, cudaStream_t s, int nkernels, const char *const *names) {

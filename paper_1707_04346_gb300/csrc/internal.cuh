@@ -145,7 +145,7 @@ struct fci_ctx {
     int log_width = 0;
     int iterations = 0;
     int sigma_calls = 0;
-    double *host_words = nullptr;   // pinned host memory that the Davidson kernels report into (made on first use)
+    double *host_words = nullptr;   // pinned host memory that kernels report into (kHostWords, made on first use)
     // per-kernel timing ring (fci_profile_*)
     bool prof = false;
     std::vector<cudaEvent_t> prof_ev;    // kProfRing * (kProfMaxKernels + 1)
@@ -164,6 +164,8 @@ constexpr int kProfMaxKernels = 8;
 int prof_begin(fci_ctx *ctx, cudaStream_t s, int nkernels, const char *const *names);
 void prof_mark(fci_ctx *ctx, int rec, int i, cudaStream_t s);
 
+constexpr int kHostWords = 1024;  // >= 30 x 30
+int host_words(fci_ctx *ctx);     // make ctx->host_words
 void *dalloc(fci_ctx *ctx, size_t bytes, int *rc);
 void dfree(fci_ctx *ctx, void *p, size_t bytes);
 
