@@ -118,6 +118,10 @@ struct fci_ctx {
     int *rowexp = nullptr;          // [N_alpha]
     uint16_t *planes = nullptr;
     size_t planes_bytes = 0;
+    // FP32 sigma_3 of spaces whose row fits in shared memory (sigma3_f32.cu; its
+    // slices share `planes`)
+    int *rowexp32 = nullptr;        // [N_alpha]
+    int eW32 = 0;
     // FP64 sigma for large spaces (sigma_wide.cu): the fixed-point integral
     // table, the exponent of the call's C, and the 64-bit accumulator
     // (aliases ws32 when the context has it)
@@ -217,6 +221,14 @@ bool sigma3_sliced_ok(const fci_ctx *ctx);
 int launch_sigma3_sliced(fci_ctx *ctx, const double *C, double *sig, cudaStream_t s, int rec, int prof_slot,
                          const int *active = nullptr, int add = 0);
 int prepare_sigma3_sliced(const fci_ctx *ctx);
+
+int build_pair_table16(fci_ctx *ctx);  // SpinTables::tabp of the beta spin
+
+// sigma3_f32.cu (FP32 sigma_3 with the sigma row in shared memory)
+bool sigma3_f32_ok(const fci_ctx *ctx);
+int build_sigma3_f32(fci_ctx *ctx, const double *eri_host);
+void free_sigma3_f32(fci_ctx *ctx);
+int launch_sigma3_f32(fci_ctx *ctx, const float *C, float *sig, cudaStream_t s, const int *active = nullptr);
 
 // sigma_wide.cu (FP64-accurate sigma for large spaces: all three terms on the
 // tensor cores, one integer accumulator)

@@ -115,15 +115,24 @@ int build_sliced_tables(fci_ctx *ctx, const double *h1_host, const double *eri_h
     ctx->rowexp = (int *)dalloc(ctx, sizeof(int) * (size_t)ctx->A.ns, &rc);
     ctx->planes_bytes = sizeof(uint16_t) * sl::kSlices * (size_t)ctx->A.ns * plane_pitch(ctx->B.ns);
     ctx->planes = (uint16_t *)dalloc(ctx, ctx->planes_bytes, &rc);
-    SpinTables &B = ctx->B;
-    B.tabp = (uint16_t *)dalloc(ctx, sizeof(uint16_t) * (size_t)npad * B.ns, &rc);
+    if (!rc) rc = build_pair_table16(ctx);
     if (rc) return rc;
     ctx->eW = eW;
     FCI_CUDA(cudaMemcpyAsync(ctx->XW, xw.data(), sizeof(long long) * xw.size(), cudaMemcpyHostToDevice, ctx->stream));
+    FCI_CUDA(cudaStreamSynchronize(ctx->stream));
+    return FCI_OK;
+}
+
+// The beta spin's replacement lists by orbital pair (at most 32767 strings).
+int build_pair_table16(fci_ctx *ctx) {
+    SpinTables &B = ctx->B;
+    const int npad = round_up16(ctx->npair);
+    int rc = FCI_OK;
+    B.tabp = (uint16_t *)dalloc(ctx, sizeof(uint16_t) * (size_t)npad * B.ns, &rc);
+    if (rc) return rc;
     FCI_CUDA(cudaMemsetAsync(B.tabp, 0xFF, sizeof(uint16_t) * (size_t)npad * B.ns, ctx->stream));
     k_pair_table<<<ceil_div(B.ns * B.nsingle, 256), 256, 0, ctx->stream>>>(B.tab, B.ns, B.nsingle, npad, B.tabp);
     FCI_CUDA(cudaGetLastError());
-    FCI_CUDA(cudaStreamSynchronize(ctx->stream));
     return FCI_OK;
 }
 
@@ -134,6 +143,7 @@ void free_sliced_tables(fci_ctx *ctx) {
     dfree(ctx, ctx->XW, sizeof(long long) * (size_t)np * np);
     dfree(ctx, ctx->rowexp, sizeof(int) * (size_t)ctx->A.ns);
     dfree(ctx, ctx->planes, ctx->planes_bytes);
+    ctx->planes_bytes = 0;
     ctx->XW = nullptr;
     ctx->rowexp = nullptr;
     ctx->planes = nullptr;

@@ -74,13 +74,16 @@ static int tc_plan(const fci_ctx *ctx, int nsplit, TcPlan *P) {
 // Opt the chosen kernel into its shared memory (not done while a stream is
 // being captured: the batched engine prepares its instances beforehand).
 int prepare_sigma3_tc(const fci_ctx *ctx, int nsplit) {
+    if (sigma3_f32_ok(ctx)) return FCI_OK;  // opted in at fci_init
     TcPlan P;
     if (int rc = tc_plan(ctx, nsplit, &P)) return rc;
     FCI_CUDA(opt_in_max_smem(P.kern, ctx->device));
     return FCI_OK;
 }
 
+// (spaces whose sigma row fits in shared memory: sigma3_f32.cu)
 int launch_sigma3_tc(fci_ctx *ctx, const float *C, float *sig, int nsplit, cudaStream_t s, const int *active) {
+    if (sigma3_f32_ok(ctx)) return launch_sigma3_f32(ctx, C, sig, s, active);
     TcPlan P;
     if (int rc = tc_plan(ctx, nsplit, &P)) return rc;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

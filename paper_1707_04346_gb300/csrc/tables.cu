@@ -420,6 +420,7 @@ int build_tables(fci_ctx *ctx, const double *h1_host, const double *eri_host) {
     if ((rc = build_sliced_tables(ctx, h1_host, eri_host))) return rc;
     if ((sigma3_sliced_ok(ctx) || sigma_wide_ok(ctx)) && (rc = build_ss_tables(ctx))) return rc;
     if ((rc = build_ss32_tables(ctx))) return rc;
+    if ((rc = build_sigma3_f32(ctx, eri_host))) return rc;
     if ((rc = prepare_sigma_small(ctx))) return rc;
     if ((rc = alloc_sigma_workspace(ctx))) return rc;
     ctx->hdiag = (double *)dalloc(ctx, sizeof(double) * ctx->ndet, &rc);
@@ -456,6 +457,7 @@ void free_tables(fci_ctx *ctx) {
     const int n = ctx->norb;
     free_wide_tables(ctx);
     free_ss32_tables(ctx);
+    free_sigma3_f32(ctx);
     free_ss_tables(ctx);
     free_sliced_tables(ctx);
     free_spin(ctx, ctx->B);
