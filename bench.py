@@ -613,10 +613,11 @@ def density_leg(pkg, norb, na, nb, h1, eri, c_dev, sigma_ms, peaks):
         t2.append(time.perf_counter() - t)
     pkg.fci_free(ctx)
     n = norb
-    R = n * n + 1
-    Rd = (R + 7) // 8 * 8
+    blocks = [n * (n + 1) // 2 + 1, n * (n - 1) // 2]  # rows of the two Gram matrices
+    Rd = [(R + 15) // 16 * 16 for R in blocks]
     nks = (c_dev.numel() + 15) // 16
-    ctx1 = pkg.fci_init(norb, na, nb, h1, eri, pkg.default_options(rdm2_chunk_bytes=float(6 * Rd * 32 * nks + 1)))
+    planes = 7.0 * sum(Rd) * 32 * nks  # digit-plane bytes, read once
+    ctx1 = pkg.fci_init(norb, na, nb, h1, eri, pkg.default_options(rdm2_chunk_bytes=planes + 1))
     pkg.fci_profile_enable(ctx1, True)
     for _ in range(3):
         pkg.fci_rdm2(ctx1, c_dev)
@@ -624,15 +625,17 @@ def density_leg(pkg, norb, na, nb, h1, eri, c_dev, sigma_ms, peaks):
     pkg.fci_profile_enable(ctx1, False)
     pkg.fci_free(ctx1)
     km = np.median(prof[-2:], axis=0)  # ms per kernel
-    bn = 48  # B rows per tile of the Gram kernel
-    nrb, ncb = (Rd + 127) // 128, (Rd + bn - 1) // bn
-    ntile = sum(ncb - (-(-(rb * 128 - (bn - 1)) // bn) if rb * 128 > bn - 1 else 0) for rb in range(nrb))
-    executed = 2.0 * 128 * bn * 16 * 21 * ntile * nks  # MMA FLOP: 21 digit products per tile and K-step
-    useful = float(R) * R * 16 * nks  # one triangle of the FP64 Gram matrix, 2 FLOP per product
+    mmas = 0  # executed MMA elements per K-step: tiles of 128 rows x bn columns
+    for rd in Rd:
+        if rd:
+            nct = (rd + 79) // 80
+            bn = (-(-rd // nct) + 15) // 16 * 16
+            mmas += 128 * bn * nct * ((rd + 127) // 128)
+    executed = 2.0 * mmas * 16 * 12 * nks  # 12 digit products per tile and K-step
+    useful = sum(float(R) * R for R in blocks) * 16 * nks  # one triangle of each FP64 Gram matrix, 2 FLOP per product
     itc = list(names).index("rdm2_tc")
     tc_s = km[itc] / 1e3
     peak = peaks.get("bf16_tflops")
-    planes = 6.0 * Rd * 32 * nks  # digit-plane bytes, read once
     path, marker, digest, ratio = RDM2_TC_TRAFFIC
     try:
         traffic = planes * ratio if kernel_digest(path, marker) == digest else None
@@ -649,7 +652,7 @@ def density_leg(pkg, norb, na, nb, h1, eri, c_dev, sigma_ms, peaks):
                              "traffic": traffic, "digit_plane_bytes": planes,
                              "traffic_note": "DRAM bytes per digit-plane byte of a CAS(12e,12o) ncu capture "
                                              "(profiles/rdm2_tc_cas12.md), scaled to this workload's planes",
-                             "note": "executed bf16 MMA FLOP (6 digits, 21 products, 128 x 48 tiles) per launch / "
+                             "note": "executed bf16 MMA FLOP (6 digits, 12 products of the symmetric half, 128 x at most 80 tiles) per launch / "
                                      "CUDA-event time; peak = measured burst bf16"},
         "timing": "whole blocking calls (allocation, statistics round trip, host copies included), median of 3",
     }

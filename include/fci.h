@@ -115,8 +115,8 @@ typedef struct fci_options {
                             (double-float next to the per-row sigma_3, intermediate strings
                             next to the wide kernels) */
     double rdm2_chunk_bytes; /* fci_rdm2: device memory for the digit planes of one chunk of
-                            determinants (about 192 (norb^2 + 1) bytes per 16 determinants
-                            per chunk); 0 = 1 GiB (default).  (Resource control; no
+                            determinants (about 224 (norb^2 + 1) bytes per 16 determinants
+                            per chunk); 0 = about 256 MiB (default).  (Resource control; no
                             counterpart in the paper.) */
 } fci_options;
 
@@ -308,9 +308,9 @@ int fci_rdm1(fci_ctx *ctx, const void *c, int dtype, double *gamma);
  * "1e/2e Density Matrices").  With gamma = fci_rdm1's density,
  *   <c|H|c> = sum h_pq gamma_pq + 1/2 sum (pq|rs) (Gamma_pqrs - delta_qr gamma_ps).
  * Gamma_pqrs = sum_K <K|E_qp|c> <K|E_rs|c> over the determinants K, computed
- * as one Gram matrix on the tensor cores with FP64 accuracy (c in 45-bit fixed
- * point relative to its largest element, six 8-bit digits, exact 64-bit
- * integer accumulation): about 1e-14 of ||c||^2, bit-reproducible.  c need
+ * as the Gram matrices of (E_rs + E_sr)|c> and (E_rs - E_sr)|c>, and gamma, on
+ * the tensor cores with FP64 accuracy (c in 45-bit fixed point relative to its largest element, six 8-bit digits, exact integer
+ * accumulation): about 1e-14 of ||c||^2, bit-reproducible.  c need
  * not be normalised (both densities scale with ||c||^2).
  *
  *  c       device vector (dtype FCI_F64 or FCI_F32) of N elements; the call
@@ -318,7 +318,8 @@ int fci_rdm1(fci_ctx *ctx, const void *c, int dtype, double *gamma);
  *  gamma1  HOST array norb x norb (gamma_pq, from the same pass), or NULL
  *  gamma2  HOST array norb^4, row-major [p][q][r][s], filled on return
  * Allocates its scratch (the digit planes of one chunk of determinants, see
- * fci_options.rdm2_chunk_bytes, and (norb^2 + 1)^2 64-bit integers) per call.
+ * fci_options.rdm2_chunk_bytes, 8 bytes per determinant and about norb^4 64-bit
+ * integers) per call.
  * A non-finite c gives NaN densities.  Blocking.  FCI_ERR_TIMEOUT when a
  * bounded wait inside the tensor-core kernel gave up, FCI_ERR_RANGE if an
  * exact accumulator left its range (neither is expected).
