@@ -43,7 +43,8 @@ constexpr int kBlock = 256;
 constexpr int kMaxSub = 32;
 constexpr int kMaxRoots = 8;
 constexpr int kChunk = 256;    // elementwise kernels: one CTA per chunk of <= kChunk elements
-constexpr int kDChunk = 8192;  // dot products: 32 elements per thread before the block reduction
+constexpr int kDPer = 4;       // dot products: elements per thread, all loads in flight
+constexpr int kDChunk = 1024;  // kDPer x kBlock
 constexpr double kPad = 1e30;
 constexpr int64_t kHybridMinDets = 32768;  // FP32 sigma of instances this large: single-instance kernels
 constexpr int kRefinePeriod = 4;           // mixed precision: refinements on every 4th non-restart iteration
@@ -280,14 +281,26 @@ __global__ void __launch_bounds__(kBlock) k_bdots(const Chunk *__restrict__ ch, 
     double acc[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[j] = 0.0;
-    if (on[c.inst])
-        for (int t = threadIdx.x; t < c.len; t += kBlock) {
-            const int64_t idx = c.start + t;
-            const double yv = y[idx];
+    if (on[c.inst]) {
+        double yv[kDPer];
+        int64_t idx[kDPer];
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j < mg) acc[j] = fma(X[(int64_t)(i0 + j) * ntot + idx], yv, acc[j]);
+        for (int u = 0; u < kDPer; ++u) {
+            const int t = threadIdx.x + u * kBlock;
+            idx[u] = c.start + (t < c.len ? t : 0);
+            yv[u] = t < c.len ? y[idx[u]] : 0.0;
         }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (j < mg) {
+                double xv[kDPer];
+#pragma unroll
+                for (int u = 0; u < kDPer; ++u)
+                    xv[u] = threadIdx.x + u * kBlock < c.len ? X[(int64_t)(i0 + j) * ntot + idx[u]] : 0.0;
+#pragma unroll
+                for (int u = 0; u < kDPer; ++u) acc[j] = fma(xv[u], yv[u], acc[j]);
+            }
+    }
     __shared__ double red[8][kBlock / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double v = sd::warp_reduce8(acc, lane);
