@@ -228,6 +228,9 @@ def kernel_work(name, norb, na, nb, N, sa, sb, nsa, nsb, peaks, f32_splits=3):
         ns_sum = nsb if name == "sigma1_ss" else nsa
         return ("tensor", 21 * 2.0 * ns_sum * N, "TFLOP/s", *bf16,
                 f"bf16 FLOP: 21 digit products x 2 x {ns_sum} per determinant, zeros included")
+    if name == "sigma12_f32":  # FP32 sigma_1 + sigma_2 by the tables: one FMA per term
+        return ("alu", 2.0 * nsame * N, "Tops/s", fp32_pipe, fp32src,
+                f"FP32 FMAs: {nsame} terms per determinant, two spins")
     if name in ("sigma12_ss32", "sigma2_ss32"):  # FP32 same-spin terms as dense products of 3 bf16 slices
         ns_sum = nsa + nsb if name == "sigma12_ss32" else nsa
         return ("tensor", 6 * 2.0 * ns_sum * N, "TFLOP/s", *bf16,

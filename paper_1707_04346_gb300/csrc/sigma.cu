@@ -23,6 +23,20 @@ namespace fci {
 
 constexpr int kEnt = 8;  // ELL entries whose table loads are issued together (FP32)
 
+// Table loads issued as volatile asm, so that a batch of them stays together in
+// program order ahead of its first use whatever the compiler's scheduling (the
+// fused FP32 kernel lost a third of its speed to a schedule change once).
+__device__ __forceinline__ int32_t ld_batch_s32(const int32_t *p) {
+    int32_t v;
+    asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_batch_f32(const float *p) {
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 template <typename T>
 __device__ __forceinline__ T gval_of(const SpinTables &S, int64_t idx);
 template <>
@@ -280,6 +294,72 @@ __global__ void __launch_bounds__(512, 1) k_sigma2_cols_df(const double *__restr
     }
 }
 
+// FP32 sigma_1 + sigma_2 in one pass when both spins share one string space
+// (n_alpha = n_beta, identical same-spin tables): a block stages R rows and
+// the same R columns of C, and every ELL entry it reads updates both,
+//   sigma(r0+r, x) += G[x][col] C(r0+r, col)      (sigma_1, row r0+r)
+//   sigma(x, r0+r) += G[x][col] C(col, r0+r)      (sigma_2, column r0+r)
+// which halves the table traffic that bounds the separate FP32 kernels.  Two
+// blocks meet on each element (its row block and its column block), so sigma
+// starts at zero and both adds are atomic; two addends onto zero give the
+// same sum in either order.  Up to kFusedStrings strings, where the dense products'
+// pipeline (sigma_ss32.cu) costs more than the table walk: 252 strings (CAS(10,10))
+// 28 us against 38, 330 strings 34 against 38, 462 strings 47 against 43.
+constexpr int64_t kFusedStrings = 400;
+template <int R>
+__global__ void __launch_bounds__(512) k_sigma12_f32(const float *__restrict__ C, float *__restrict__ sig,
+                                                     SpinTables S, const int *__restrict__ active) {
+    if (active != nullptr && *active == 0) return;  // gated launch (batched engine): instance not active
+    extern __shared__ float smf[];
+    const int64_t ns = S.ns;
+    float *rows = smf;           // [R][ns]
+    float *cols = smf + R * ns;  // [R][ns]
+    const int64_t r0 = (int64_t)blockIdx.x * R;
+    for (int64_t t = threadIdx.x; t < (int64_t)R * ns; t += blockDim.x) {
+        const int64_t r = t / ns, j = t % ns;
+        rows[t] = (r0 + r < ns) ? C[(r0 + r) * ns + j] : 0.f;
+    }
+    for (int64_t i = threadIdx.x; i < ns; i += blockDim.x) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) cols[(int64_t)r * ns + i] = (r0 + r < ns) ? C[i * ns + r0 + r] : 0.f;
+    }
+    __syncthreads();
+    for (int64_t x = threadIdx.x; x < ns; x += blockDim.x) {
+        float ar[R], ac[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) ar[r] = ac[r] = 0.f;
+        for (int e0 = 0; e0 < S.nsame; e0 += kEnt) {
+            int32_t col[kEnt];
+            float v[kEnt];
+#pragma unroll
+            for (int u = 0; u < kEnt; ++u) {  // in-range addresses; padding slots zeroed after the loads
+                const int64_t idx = (int64_t)(e0 + u < S.nsame ? e0 + u : 0) * ns + x;
+                col[u] = ld_batch_s32(S.gcol + idx);
+                v[u] = ld_batch_f32(S.gvalf + idx);
+            }
+#pragma unroll
+            for (int u = 0; u < kEnt; ++u)
+                if (e0 + u >= S.nsame) {
+                    col[u] = 0;
+                    v[u] = 0.f;
+                }
+#pragma unroll
+            for (int u = 0; u < kEnt; ++u)
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    ar[r] = fmaf(v[u], rows[(int64_t)r * ns + col[u]], ar[r]);
+                    ac[r] = fmaf(v[u], cols[(int64_t)r * ns + col[u]], ac[r]);
+                }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (r0 + r < ns) {
+                atomicAdd(sig + (r0 + r) * ns + x, ar[r]);
+                atomicAdd(sig + x * ns + r0 + r, ac[r]);
+            }
+    }
+}
+
 // out[c][r] = in[r][c] (ADD: out[c][r] += in[r][c]) for a rows x cols matrix,
 // through 32 x 32 tiles in shared memory (block 32 x 8).
 template <bool ADD>
@@ -436,6 +516,22 @@ bool f32_same_spin_tc(const fci_ctx *ctx) {
     return tc_ok && (ctx->opt.same_spin_tc == 1 || (!sigma_ss32_ok(ctx) && (!fits(4, B.ns) || !fits(4, A.ns))));
 }
 
+static bool sigma12_fused_ok(const fci_ctx *ctx) {
+    return ctx->A.ne == ctx->B.ne && ctx->A.ns == ctx->B.ns && ctx->A.nsingle > 0 && ctx->A.ns <= kFusedStrings &&
+           !f32_same_spin_tc(ctx);
+}
+
+static int launch_sigma12_f32(const fci_ctx *ctx, const float *C, float *sig, cudaStream_t s,
+                              const int *active = nullptr) {
+    constexpr int R = 8;
+    const int64_t ns = ctx->A.ns;
+    static_assert(2 * R * kFusedStrings * sizeof(float) <= 48 * 1024, "shared memory without an opt-in");
+    FCI_CUDA(cudaMemsetAsync(sig, 0, sizeof(float) * (size_t)ns * (size_t)ns, s));
+    k_sigma12_f32<R><<<ceil_div(ns, R), 512, (size_t)2 * R * ns * sizeof(float), s>>>(C, sig, ctx->A, active);
+    FCI_CUDA(cudaGetLastError());
+    return FCI_OK;
+}
+
 int alloc_sigma_workspace(fci_ctx *ctx) {
     if (!f32_same_spin_tc(ctx) || ctx->ws32) return FCI_OK;
     int rc = FCI_OK;
@@ -467,10 +563,13 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
     const bool same_tc = sizeof(T) == 4 && f32_same_spin_tc(ctx);
     // both FP32 same-spin terms as dense tensor-core products in one launch
     const bool ss32 = sizeof(T) == 4 && !same_tc && sigma_ss32_ok(ctx);
+    // or, for few strings of one space, by the fused table walk (no parity)
+    const bool fused = sizeof(T) == 4 && sigma12_fused_ok(ctx);
     // profiled kernels (fci_profile_read)
     static const char *const names3[3] = {"sigma1_rows", "sigma2_cols", sizeof(T) == 4 ? "sigma3_tc" : "sigma3_exact"};
     static const char *const names3tc[3] = {"sigma2_tc", "sigma1_tc", "sigma3_tc"};
     static const char *const names2ss[2] = {"sigma12_ss32", "sigma3_tc"};
+    static const char *const names2[2] = {"sigma12_f32", "sigma3_tc"};
     static const char *const names4[4] = {"slice_c", "sigma3_sliced", "sigma1_rows", "sigma2_cols"};
     // FP64 with the sliced tensor-core sigma_3: it runs first and overwrites sigma
     const bool sliced = sizeof(T) == 8 && A.nsingle > 0 && B.nsingle > 0 && ctx->opt.f64_kernels != FCI_F64_FMA &&
@@ -534,10 +633,11 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
     const bool ss = sliced && sigma_ss_ok(ctx);
     const int rec = ss ? prof_begin(ctx, s, 4, names4ss)
                     : sliced ? prof_begin(ctx, s, 4, names4)
+                    : fused ? prof_begin(ctx, s, 2, names2)
                     : ss32 ? prof_begin(ctx, s, 2, names2ss)
                     : same_tc ? prof_begin(ctx, s, 3, names3tc)
                              : prof_begin(ctx, s, 3, names3);
-    const int slot3 = ss32 ? 1 : 2;
+    const int slot3 = fused || ss32 ? 1 : 2;
     int slot = 0;  // next profiling slot of the staged same-spin kernels
     int add1 = 0;  // sigma_1 adds to what sigma_3 wrote
     if (sliced) {
@@ -548,7 +648,11 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
         slot = 2;
         add1 = 1;
     }
-    if (ss32) {
+    if (fused) {
+        if constexpr (sizeof(T) == 4)
+            if (int rc = launch_sigma12_f32(ctx, (const float *)C, (float *)sig, s)) return rc;
+        prof_mark(ctx, rec, 0, s);
+    } else if (ss32) {
         if constexpr (sizeof(T) == 4)
             if (int rc = launch_sigma_ss32(ctx, (const float *)C, (float *)sig, 3, s)) return rc;
         prof_mark(ctx, rec, 0, s);
@@ -625,9 +729,9 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
 
 // FP32 sigma of one instance of the batched engine, skipped on the device
 // when *active == 0 (so that a captured graph serves any active set): the
-// one-kernel sigma of small spaces, else the dense same-spin products and the
-// tensor-core sigma_3 (sigma is then zeroed even when the instance is skipped).  The kernels' shared memory limits are set once by
-// prepare_sigma_f32_gated (outside any capture).
+// one-kernel sigma of small spaces, else the same-spin products and the tensor-core
+// sigma_3 (sigma is then zeroed even when the instance is skipped).  The kernels'
+// shared memory limits are set once by prepare_sigma_f32_gated (outside any capture).
 bool sigma_f32_gated_ok(const fci_ctx *ctx) {
     return sigma_small_ok(ctx, FCI_F32) || (sigma_ss32_ok(ctx) && sigma3_tc_smem(ctx, ctx->opt.f32_splits) > 0);
 }
@@ -638,7 +742,9 @@ int prepare_sigma_f32_gated(const fci_ctx *ctx) {
 
 int launch_sigma_f32_gated(fci_ctx *ctx, const float *C, float *sig, const int *active, cudaStream_t s) {
     if (sigma_small_ok(ctx, FCI_F32)) return launch_sigma_small(ctx, C, sig, FCI_F32, s, active);
-    if (int rc = launch_sigma_ss32(ctx, C, sig, 3, s, active)) return rc;
+    if (int rc = sigma12_fused_ok(ctx) ? launch_sigma12_f32(ctx, C, sig, s, active)
+                                       : launch_sigma_ss32(ctx, C, sig, 3, s, active))
+        return rc;
     return launch_sigma3_tc(ctx, C, sig, ctx->opt.f32_splits, s, active);
 }
 

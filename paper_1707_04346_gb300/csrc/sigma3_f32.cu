@@ -14,11 +14,11 @@
 // slot of the sigma row in shared memory (|h| < 2^22 and |l| <= 2^21, at most 96
 // adds: neither overflows; exact, in any order: the result is bit-reproducible).
 //
-// The kernel before this one (sigma_tc_kernel.cuh, which still covers the spaces
-// whose row does not fit) split C into slices once per replacement, 56 times a
+// The kernel before this one (sigma_tc_kernel.cuh, which still takes smaller spaces
+// and rows that do not fit) split C into slices once per replacement, 56 times a
 // value at CAS(14,14), in the producers' registers, and gathered each target's
 // contributions on four warps.  sigma_3 of one call, slices included, before and
-// now: 2.97 and 2.23 ms at CAS(14,14), 55.7 and 36.3 ms at CAS(16,16).
+// now: 2.97 and 2.24 ms at CAS(14,14), 55.7 and 36.4 ms at CAS(16,16).
 //
 // What bounds it at CAS(14,14): the copies of C's rows (0.75 GB of cp.async through
 // L2 for 56 replacements x 3 slices, with their hand-over to the MMAs) and the shared
@@ -397,6 +397,13 @@ struct Plan {
     void *kern = nullptr;
 };
 
+// A row's set-up (exponents, integral slices) and the slicing pass pay off over
+// seven tiles of beta strings and four rows per SM: 792 x 792 strings 156 us against
+// 159 with the kernel of sigma_tc_kernel.cuh, 924 x 924 201 against 209, 1287 x 1287
+// 359 against 385; below, 715 x 715 strings 137 against 121, 364 x 1001 114 against
+// 105, 252 x 252 32 against 22.
+constexpr int64_t kMinRows = 600, kMinStrings = 769;
+
 // Sizes for this context (the ring as deep as fits, at least four K-steps);
 // false when the kernel does not cover it.
 static bool plan(const fci_ctx *ctx, Plan *P) {
@@ -404,7 +411,8 @@ static bool plan(const fci_ctx *ctx, Plan *P) {
     const int ns = ctx->opt.f32_splits;
     P->kpad = (A.nsingle + 15) / 16 * 16;
     P->npad = (ctx->npair + 15) / 16 * 16;
-    if (A.nsingle == 0 || B.nsingle == 0 || P->kpad > 96 || P->npad > 256 || B.ns > 0x7FFF || B.nsingle > 96)
+    if (A.nsingle == 0 || B.nsingle == 0 || P->kpad > 96 || P->npad > 256 || B.ns > 0x7FFF || B.nsingle > 96 ||
+        A.ns < kMinRows || B.ns < kMinStrings)
         return false;
     int lim = 0;
     if (cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device) != cudaSuccess) return false;

@@ -179,13 +179,15 @@ static double macs(const fci_ctx *ctx) {  // multiply-adds of the call
 
 }  // namespace sml
 
-// FP64 up to kSmall64 multiply-adds (CAS(9; 5,4), 1.1e7: 37 us against 80 us with
-// the sliced products; CAS(10; 4,4) and CAS(10; 5,5), 4 and 7e7, would take as long
-// on the FP64 pipe as the 100 us of the products); FP32 up to kSmall32 (CAS(10;
-// 5,5), 7e7: 57 us against 60 us on the tensor cores; CAS(11; 6,5), 3e8: 270
-// against 115 us); both spins with replacements (the single-spin terms alone stay with
-// the staged kernels), default kernel choices.
-constexpr double kSmall64 = 1.5e7, kSmall32 = 8e7;
+// FP64 up to kSmall64 multiply-adds (CAS(9; 5,4), 1.1e7: 37 us against 81 us with
+// the sliced products; CAS(10; 5,3), 2.4e7: 89 with them).  FP32 up to kSmall32 for
+// unequal spins (CAS(10; 5,4): 51 us against 68 with the dense products; CAS(11;
+// 6,5), 3e8: 270 against 115) and kSmall32Same for one string space, whose same-spin
+// terms the fused table walk of sigma.cu takes next (15876 determinants of CAS(9; 4,4):
+// 19 us against 28; CAS(11; 3,3), 2e7: 44 both; CAS(10; 4,4), 4e7: 50 against 44).
+// Both spins with replacements (the single-spin terms alone stay with the staged
+// kernels), default kernel choices.
+constexpr double kSmall64 = 1.5e7, kSmall32 = 8e7, kSmall32Same = 2.5e7;
 
 bool sigma_small_ok(const fci_ctx *ctx, int dtype) {
     const fci_options &o = ctx->opt;
@@ -193,7 +195,8 @@ bool sigma_small_ok(const fci_ctx *ctx, int dtype) {
     if (dtype == FCI_F64)
         return o.f64_kernels == FCI_F64_AUTO && o.f64_same_spin == FCI_SS_AUTO && sml::macs<double>(ctx) <= kSmall64 &&
                sml::smem_bytes<double>(ctx) <= 100 * 1024;
-    return o.same_spin_tc == 0 && o.f32_row_global == 0 && sml::macs<float>(ctx) <= kSmall32 &&
+    return o.same_spin_tc == 0 && o.f32_row_global == 0 &&
+           sml::macs<float>(ctx) <= (ctx->A.ne == ctx->B.ne ? kSmall32Same : kSmall32) &&
            sml::smem_bytes<float>(ctx) <= 100 * 1024;
 }
 

@@ -25,7 +25,9 @@
 // on each element: sigma starts at zero and takes two atomic adds, whose order
 // does not change the sum of two addends onto zero.
 //
-// CAS(14,14): SS32.
+// Both terms with their passes over C, against the fused table-driven FP32 kernel
+// before (unequal spins: one kernel per term): CAS(14,14) 2.24 -> 0.75 ms,
+// CAS(16,16) 80.3 -> 25.7 ms.
 #include <algorithm>
 
 #include "sliced_mma.cuh"

@@ -25,6 +25,9 @@ def pkg():
 # rows of 1365, 462, 165, 1716, 715 and 715 strings
 @pytest.mark.parametrize("norb,na,nb,splits", [
     (15, 1, 4, 3), (11, 2, 5, 3), (11, 3, 8, 2), (13, 3, 7, 3), (13, 6, 4, 3), (13, 9, 4, 2),
+    # at least 600 x 769 strings: 715 x 1287 (K = 40, 45), 792 x 792 (K = 40), 1001 x 1001 (K = 44
+    # and 50 targets a string), 816 x 816 (K = 48, 171 pairs)
+    (13, 4, 5, 3), (13, 9, 8, 2), (12, 5, 5, 3), (14, 4, 10, 2), (18, 3, 3, 3),
 ])
 def test_rows_match_oracle(pkg, oracle_mod, norb, na, nb, splits):
     h1, eri = fi.make_integrals(norb, 60)
