@@ -319,7 +319,7 @@ int fci_rdm1(fci_ctx *ctx, const void *c, int dtype, double *gamma);
  *  gamma2  HOST array norb^4, row-major [p][q][r][s], filled on return
  * Allocates its scratch (the digit planes of one chunk of determinants, see
  * fci_options.rdm2_chunk_bytes, 8 bytes per determinant and about norb^4 64-bit
- * integers) per call.
+ * integers) per call; up to 64 MiB in all stays with the context until fci_free.
  * A non-finite c gives NaN densities.  Blocking.  FCI_ERR_TIMEOUT when a
  * bounded wait inside the tensor-core kernel gave up, FCI_ERR_RANGE if an
  * exact accumulator left its range (neither is expected).

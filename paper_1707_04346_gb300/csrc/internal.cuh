@@ -121,6 +121,9 @@ struct fci_ctx {
     // FP32 sigma_3 of spaces whose row fits in shared memory (sigma3_f32.cu; its
     // slices share `planes`)
     int *rowexp32 = nullptr;        // [N_alpha]
+    // fci_rdm2's scratch when small (rdm2.cu)
+    unsigned char *rdm2_ws = nullptr;
+    size_t rdm2_ws_bytes = 0;
     int eW32 = 0;
     // FP64 sigma for large spaces (sigma_wide.cu): the fixed-point integral
     // table, the exponent of the call's C, and the 64-bit accumulator
