@@ -50,23 +50,22 @@ FP32_LANES_PER_SM = 128  # FP32 operations issued per SM per clock
 # only while that source is unchanged.
 NCU_TRAFFIC = {
     "sigma3_exact": ("paper_1707_04346_gb300/csrc/sigma.cu", "k_sigma3_exact(", "d3fba1cadf6cd31c", 610262016.0),
-    "sigma3_tc": ("paper_1707_04346_gb300/csrc/sigma_tc_kernel.cuh", "k_sigma3_tc(", "878aabf229629b81", 124323328.0),
-    "sigma3_sliced": ("paper_1707_04346_gb300/csrc/sigma3_sliced_kernel.cuh", "k_sigma3_sliced(", "2f62dcb8acf96f61",
-                      978847232.0),
+    "sigma3_tc": ("paper_1707_04346_gb300/csrc/sigma3_f32.cu", "k_sigma3_f32(", "f894b1c00eede3f4", 221401344.0),
+    "sigma3_sliced": ("paper_1707_04346_gb300/csrc/sigma3_sliced_kernel.cuh", "k_sigma3_sliced(", "0d1f7828b6d7bb70", 1077408768.0),
     # sigma_1 as a dense sliced product (k_ss_tc; sigma_2 runs the same kernel with the operands swapped)
-    "sigma1_ss": ("paper_1707_04346_gb300/csrc/sigma_ss.cu", "k_ss_tc(", "9c370e9bb4171175", 2206744880.0),
+    "sigma1_ss": ("paper_1707_04346_gb300/csrc/sigma_ss.cu", "k_ss_tc(", "9edff8592af53966", 1402157568.0),
     # the wide kernels at CAS(14,14) (bench.py --f64-kernels wide)
-    "sigma3_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "3b63c3cbe309e741", 1016815808.0),
-    "sigma1_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "3b63c3cbe309e741", 2433141328.0),
-    "sigma2_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "3b63c3cbe309e741", 2452579616.0),
+    "sigma3_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "81d454a69f812b05", 1064472320.0),
+    "sigma1_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "81d454a69f812b05", 2521320704.0),
+    "sigma2_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "81d454a69f812b05", 2508126640.0),
 }
 
 
-# The 2-RDM's Gram kernel, captured on CAS(12e,12o) (the CAS(14,14) launch holds 28 GB of digit
+# The 2-RDM's Gram kernel, captured on CAS(12e,12o) (the CAS(14,14) launch holds 34 GB of digit
 # planes, above the capture size rule): DRAM bytes per byte of digit planes read once, scaled to
 # the workload's planes while the kernel's source is unchanged.
-RDM2_TC_TRAFFIC = ("paper_1707_04346_gb300/csrc/rdm2.cu", "k_rdm2_tc(", "dbb9c2a6acd29160",
-                   (2413767000.0 + 3238656.0) / (53361 * 6 * 152 * 32))
+RDM2_TC_TRAFFIC = ("paper_1707_04346_gb300/csrc/rdm2.cu", "k_rdm2_tc(", "5c4fa46bf3e768e4",
+                   (1912671744.0 + 1474304.0) / (53361 * 7 * 160 * 32))
 
 
 # Kernels one sigma call launches, by its profiled slots (the slots group kernels: "slice_c"
@@ -654,7 +653,7 @@ def density_leg(pkg, norb, na, nb, h1, eri, c_dev, sigma_ms, peaks):
                              "executed_flop": executed, "fp64_equivalent_tflops": useful / tc_s / 1e12,
                              "traffic": traffic, "digit_plane_bytes": planes,
                              "traffic_note": "DRAM bytes per digit-plane byte of a CAS(12e,12o) ncu capture "
-                                             "(profiles/rdm2_tc_cas12.md), scaled to this workload's planes",
+                                             "(profiles/kernel_traffic_cas14.md), scaled to this workload's planes",
                              "note": "executed bf16 MMA FLOP (6 digits, 12 products of the symmetric half, 128 x at most 80 tiles) per launch / "
                                      "CUDA-event time; peak = measured burst bf16"},
         "timing": "whole blocking calls (allocation, statistics round trip, host copies included), median of 3",
