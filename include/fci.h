@@ -298,6 +298,10 @@ int fci_davidson_log(fci_ctx *ctx, double *out, int cap, int *count);
  *  c      device vector (dtype FCI_F64 or FCI_F32) of N elements; the call
  *         first waits for all work on the device, so c may come from any stream
  *  gamma  HOST array norb x norb, row-major, filled on return (blocking)
+ *
+ * Scratch as fci_rdm2's: of this call alone, so that fci_rdm1 and fci_rdm2 may run
+ * in several host threads and beside fci_sigma on one context; up to 64 MiB stay
+ * with the context until fci_free.
  */
 int fci_rdm1(fci_ctx *ctx, const void *c, int dtype, double *gamma);
 
@@ -319,7 +323,9 @@ int fci_rdm1(fci_ctx *ctx, const void *c, int dtype, double *gamma);
  *  gamma2  HOST array norb^4, row-major [p][q][r][s], filled on return
  * Allocates its scratch (the digit planes of one chunk of determinants, see
  * fci_options.rdm2_chunk_bytes, 8 bytes per determinant and about norb^4 64-bit
- * integers) per call; up to 64 MiB in all stays with the context until fci_free.
+ * integers); the context keeps up to 64 MiB of scratch from density call to density
+ * call until fci_free (calls that run at the same time, and larger ones, allocate
+ * their own and give it back).
  * A non-finite c gives NaN densities.  Blocking.  FCI_ERR_TIMEOUT when a
  * bounded wait inside the tensor-core kernel gave up, FCI_ERR_RANGE if an
  * exact accumulator left its range (neither is expected).

@@ -726,7 +726,7 @@ struct Work {
     // after the allocations: zero counters, the context's pinned words
     int begin() {
         if (int r = host_words(ctx)) return r;
-        host = ctx->host_words;
+        host = ctx->host_words + kDensityWords;
         FCI_CUDA(cudaMemsetAsync(counter, 0, 4 * sizeof(int), s));
         return FCI_OK;
     }

@@ -32,7 +32,7 @@ void *dalloc(fci_ctx *ctx, size_t bytes, int *rc) {
     if (ctx->opt.max_device_bytes > 0 && (double)ctx->bytes + (double)bytes > ctx->opt.max_device_bytes) {
         char buf[200];
         snprintf(buf, sizeof(buf), "allocation of %zu bytes would exceed fci_options.max_device_bytes (%.0f; %zu held)",
-                 bytes, ctx->opt.max_device_bytes, ctx->bytes);
+                 bytes, ctx->opt.max_device_bytes, ctx->bytes.load());
         set_error(buf);
         *rc = FCI_ERR_OOM;
         return nullptr;
@@ -58,8 +58,44 @@ void dfree(fci_ctx *ctx, void *p, size_t bytes) {
 }
 
 int host_words(fci_ctx *ctx) {
-    if (!ctx->host_words) FCI_CUDA(cudaMallocHost((void **)&ctx->host_words, kHostWords * sizeof(double)));
+    std::lock_guard<std::mutex> lock(ctx->scratch_mu);
+    if (!ctx->host_words)
+        FCI_CUDA(cudaMallocHost((void **)&ctx->host_words, (kDensityWords + kDavidsonWords) * sizeof(double)));
     return FCI_OK;
+}
+
+int DensityScratch::take(size_t bytes) {
+    int rc = FCI_OK;
+    if (bytes <= kKeptScratch) {
+        std::lock_guard<std::mutex> lock(ctx->scratch_mu);
+        kept_ = !ctx->scratch_taken;
+        if (kept_) ctx->scratch_taken = true;
+    }
+    if (!kept_) {
+        dev = (unsigned char *)dalloc(ctx, bytes, &rc);
+        bytes_ = rc ? 0 : bytes;
+        return rc;
+    }
+    if ((rc = host_words(ctx))) return rc;
+    if (ctx->scratch_bytes < bytes) {
+        dfree(ctx, ctx->scratch, ctx->scratch_bytes);
+        ctx->scratch_bytes = 0;
+        ctx->scratch = (unsigned char *)dalloc(ctx, bytes, &rc);
+        if (rc) return rc;
+        ctx->scratch_bytes = bytes;
+    }
+    dev = ctx->scratch;
+    host = ctx->host_words;
+    return FCI_OK;
+}
+
+DensityScratch::~DensityScratch() {
+    if (!kept_) {
+        dfree(ctx, dev, bytes_);
+        return;
+    }
+    std::lock_guard<std::mutex> lock(ctx->scratch_mu);
+    ctx->scratch_taken = false;
 }
 
 int unpack_table(fci_ctx *ctx, int spin, int32_t *tgt, int8_t *k, int8_t *l, int8_t *sg);
@@ -427,7 +463,7 @@ int64_t fci_query(fci_ctx *ctx, int what) {
         case FCI_Q_NSINGLE_ALPHA: return ctx->A.nsingle;
         case FCI_Q_NSINGLE_BETA: return ctx->B.nsingle;
         case FCI_Q_NPAIR: return ctx->npair;
-        case FCI_Q_DEVICE_BYTES: return (int64_t)ctx->bytes;
+        case FCI_Q_DEVICE_BYTES: return (int64_t)ctx->bytes.load();
         case FCI_Q_ITERATIONS: return ctx->iterations;
         case FCI_Q_SIGMA_CALLS: return ctx->sigma_calls;
         case FCI_Q_DEVICE_ERROR: {

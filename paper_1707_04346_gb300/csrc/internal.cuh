@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -121,9 +123,12 @@ struct fci_ctx {
     // FP32 sigma_3 of spaces whose row fits in shared memory (sigma3_f32.cu; its
     // slices share `planes`)
     int *rowexp32 = nullptr;        // [N_alpha]
-    // fci_rdm2's scratch when small (rdm2.cu)
-    unsigned char *rdm2_ws = nullptr;
-    size_t rdm2_ws_bytes = 0;
+    // scratch of the density calls (DensityScratch): one call at a time has it
+    std::mutex scratch_mu;          // guards the four members below
+    bool scratch_taken = false;
+    unsigned char *scratch = nullptr;
+    size_t scratch_bytes = 0;
+    double *host_words = nullptr;   // pinned host memory that kernels report into (made on first use)
     int eW32 = 0;
     // FP64 sigma for large spaces (sigma_wide.cu): the fixed-point integral
     // table, the exponent of the call's C, and the 64-bit accumulator
@@ -146,13 +151,12 @@ struct fci_ctx {
     int *ssEr = nullptr, *ssEc = nullptr;
     double *hdiag = nullptr;        // [ndet]
     int *d_err = nullptr;           // device error word (bounded waits that gave up)
-    size_t bytes = 0;
+    std::atomic<size_t> bytes{0};   // calls of several threads allocate
     // Davidson bookkeeping
     std::vector<double> log;        // records of (nroots + 3) doubles
     int log_width = 0;
     int iterations = 0;
     int sigma_calls = 0;
-    double *host_words = nullptr;   // pinned host memory that kernels report into (kHostWords, made on first use)
     // per-kernel timing ring (fci_profile_*)
     bool prof = false;
     std::vector<cudaEvent_t> prof_ev;    // kProfRing * (kProfMaxKernels + 1)
@@ -171,10 +175,33 @@ constexpr int kProfMaxKernels = 8;
 int prof_begin(fci_ctx *ctx, cudaStream_t s, int nkernels, const char *const *names);
 void prof_mark(fci_ctx *ctx, int rec, int i, cudaStream_t s);
 
-constexpr int kHostWords = 1024;  // >= 30 x 30
+// Pinned host words: a density's kDensityWords (>= 30 x 30), then the Davidson driver's.
+constexpr int kDensityWords = 1024, kDavidsonWords = 32;
 int host_words(fci_ctx *ctx);     // make ctx->host_words
 void *dalloc(fci_ctx *ctx, size_t bytes, int *rc);
 void dfree(fci_ctx *ctx, void *p, size_t bytes);
+
+// Device scratch of one density call (fci_rdm1, fci_rdm2).  Densities may run beside
+// each other and beside fci_sigma on one context (other host threads), so a call's
+// scratch is its own: the context's, kept from call to call up to kKeptScratch
+// bytes (a call of a small space takes about as long as allocating and freeing:
+// fci_rdm2 at CAS(8,8) 255 us with, the kernels 70), or, while another call has that
+// or for more bytes, an allocation of this call.
+constexpr size_t kKeptScratch = (size_t)64 << 20;
+struct DensityScratch {
+    fci_ctx *ctx;
+    unsigned char *dev = nullptr;
+    double *host = nullptr;  // the context's pinned density words, or null: copy from the device
+    explicit DensityScratch(fci_ctx *c) : ctx(c) {}
+    DensityScratch(const DensityScratch &) = delete;
+    DensityScratch &operator=(const DensityScratch &) = delete;
+    ~DensityScratch();
+    int take(size_t bytes);
+
+  private:
+    bool kept_ = false;
+    size_t bytes_ = 0;
+};
 
 // tables.cu
 int build_tables(fci_ctx *ctx, const double *h1_host, const double *eri_host);

@@ -297,7 +297,7 @@ struct RdmPlan {
 
     RdmPlan(const fci_ctx *ctx, int max_chunks) {
         const SpinTables &A = ctx->A, &B = ctx->B;
-        if (ctx->ndet <= kSmallDets) {  // no scratch
+        if (ctx->ndet <= kSmallDets) {  // gamma alone
             doubles = (size_t)ctx->norb * ctx->norb;
             return;
         }
@@ -376,22 +376,19 @@ int launch_rdm1(fci_ctx *ctx, const T *C, const RdmPlan &P, cudaStream_t s) {
 template <typename T>
 int rdm_impl(fci_ctx *ctx, const T *C, double *gamma_host) {
     RdmPlan P(ctx, 1 << 20);
-    if (int rc = host_words(ctx)) return rc;
-    const bool scratch = ctx->ndet > kSmallDets;
-    int rc = FCI_OK;
-    // the operand planes of C that sigma's dense products use are free during the call
-    const size_t bytes = sizeof(double) * P.doubles;
-    const bool own = scratch && bytes > ctx->ssCr_bytes;
-    double *base = own ? (double *)dalloc(ctx, bytes, &rc) : (double *)ctx->ssCr;
-    if (rc) return rc;
-    if (scratch) P.place(ctx, base);
-    P.gamma = ctx->host_words;  // the last kernel writes the density into pinned host memory
+    DensityScratch mem(ctx);
+    if (int rc = mem.take(sizeof(double) * P.doubles)) return rc;
+    P.place(ctx, reinterpret_cast<double *>(mem.dev));
+    const size_t bytes = sizeof(double) * ctx->norb * ctx->norb;
+    if (mem.host) P.gamma = mem.host;  // the last kernel writes the density into pinned host memory
     cudaStream_t s = ctx->stream;
-    rc = launch_rdm1<T>(ctx, C, P, s);
-    const cudaError_t e = cudaStreamSynchronize(s);
+    int rc = launch_rdm1<T>(ctx, C, P, s);
+    cudaError_t e = cudaSuccess;
+    if (rc == FCI_OK && !mem.host) e = cudaMemcpyAsync(gamma_host, P.gamma, bytes, cudaMemcpyDeviceToHost, s);
+    const cudaError_t done = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = done;
     if (rc == FCI_OK && e != cudaSuccess) rc = cuda_fail(e, "rdm1");
-    if (rc == FCI_OK) memcpy(gamma_host, ctx->host_words, sizeof(double) * ctx->norb * ctx->norb);
-    if (own) dfree(ctx, base, bytes);
+    if (rc == FCI_OK && mem.host) memcpy(gamma_host, mem.host, bytes);
     return rc;
 }
 

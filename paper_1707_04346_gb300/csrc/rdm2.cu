@@ -668,8 +668,6 @@ __global__ void k_rdm2_finish(const unsigned long long *__restrict__ G, int RdS,
 
 // Digit planes of one chunk when the caller names no size.
 constexpr size_t kDefaultChunk = (size_t)256 << 20;
-// Scratch that a context keeps from call to call.
-constexpr size_t kKept = (size_t)64 << 20;
 
 inline unsigned grid_blocks(int64_t n) { return (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 16); }
 
@@ -708,28 +706,9 @@ int rdm2_impl(fci_ctx *ctx, const T *C, double *g1_host, double *g2_host) {
     const size_t o_dg = part(step_bytes * (size_t)chunk), o_stat = part(sizeof(int) * 2), o_G = part(gbytes),
                  o_out = part(sizeof(double) * (size_t)(n4 + n2)), o_x = part(sizeof(long long) * (size_t)N),
                  o_rows = part(sizeof(uint16_t) * ((size_t)ctx->A.ns * ctx->A.nsingle + (size_t)ctx->B.ns * ctx->B.nsingle));
-    // up to kKept bytes stay with the context (a call of a small space takes about as
-    // long as allocating and freeing them: CAS(8,8) 255 us with, the kernels 70); more
-    // is given back at the end of the call
-    int rc = FCI_OK;
-    const bool keep = total <= kKept;
-    unsigned char *mem = keep ? ctx->rdm2_ws : nullptr;
-    if (!mem || total > ctx->rdm2_ws_bytes) {
-        if (keep) {
-            dfree(ctx, ctx->rdm2_ws, ctx->rdm2_ws_bytes);
-            ctx->rdm2_ws = nullptr;
-            ctx->rdm2_ws_bytes = 0;
-        }
-        mem = (unsigned char *)dalloc(ctx, total, &rc);
-        if (rc) return rc;
-        if (keep) {
-            ctx->rdm2_ws = mem;
-            ctx->rdm2_ws_bytes = total;
-        }
-    }
-    auto release = [&]() {
-        if (!keep) dfree(ctx, mem, total);
-    };
+    DensityScratch scratch(ctx);
+    if (int rc = scratch.take(total)) return rc;
+    unsigned char *mem = scratch.dev;
     unsigned char *dg = mem + o_dg;
     unsigned long long *G = reinterpret_cast<unsigned long long *>(mem + o_G);
     double *out = reinterpret_cast<double *>(mem + o_out);
@@ -791,7 +770,6 @@ int rdm2_impl(fci_ctx *ctx, const T *C, double *g1_host, double *g2_host) {
     if (e == cudaSuccess && g1_host) e = cudaMemcpyAsync(g1_host, out + n4, sizeof(double) * n2, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    release();
     if (e != cudaSuccess) return cuda_fail(e, "rdm2");
     if (herr & 1) return fail(FCI_ERR_TIMEOUT, "rdm2: a bounded wait in the tensor-core kernel gave up");
     if (herr) return fail(FCI_ERR_RANGE, "rdm2: an exact accumulator left its range");

@@ -458,8 +458,8 @@ void free_tables(fci_ctx *ctx) {
     free_wide_tables(ctx);
     free_ss32_tables(ctx);
     free_sigma3_f32(ctx);
-    dfree(ctx, ctx->rdm2_ws, ctx->rdm2_ws_bytes);
-    ctx->rdm2_ws = nullptr;
+    dfree(ctx, ctx->scratch, ctx->scratch_bytes);
+    ctx->scratch = nullptr;
     free_ss_tables(ctx);
     free_sliced_tables(ctx);
     free_spin(ctx, ctx->B);
