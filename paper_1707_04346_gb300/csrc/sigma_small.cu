@@ -157,9 +157,11 @@ __global__ void __launch_bounds__(kThreads) k_sigma_small(const T *__restrict__ 
         }
         __syncthreads();
         if (on && p == 0) {
-            T v = sRed[tid];
-            for (int k = 1; k < parts; ++k) v += sRed[tid + k * width];
-            sig[(size_t)row * nsb + ib] = v;
+            // as above: up to 256 parts, one of which holds the diagonal (a plain FP32 sum of
+            // them left 4e-7 of the result at CAS(12; 6,12), this one 7e-8)
+            Sum<T> v;
+            for (int k = 0; k < parts; ++k) v.add(sRed[tid + k * width]);
+            sig[(size_t)row * nsb + ib] = v.get();
         }
         __syncthreads();
     }
