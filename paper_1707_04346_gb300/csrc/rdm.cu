@@ -17,7 +17,7 @@
 //  * one CTA per pair of orbitals sums its partials in a fixed order: the result
 //    is bitwise reproducible.
 // CAS(14,14), the whole blocking call: 3.5 ms with one dot per replacement (a
-// thread's column dots gathered from global memory), 1.5 ms this way (6e8
+// thread's column dots gathered from global memory), 1.45 ms this way (6e8
 // multiply-adds: 1.0 ms of the FP64 pipe).
 #include <algorithm>
 #include <cstdio>
@@ -31,6 +31,8 @@ namespace {
 constexpr int kPairsPerThread = 8;
 constexpr int kBetaThreads = 512;
 constexpr int kPairsPerBlock = kPairsPerThread * kBetaThreads;
+constexpr int kMinRows = 8;       // of a beta row chunk
+constexpr int kListStrings = 512;
 
 struct RdmSpin {
     int32_t *off = nullptr;
@@ -40,51 +42,51 @@ struct RdmSpin {
     int nr = 0;  // 0: the spin has no electrons
 };
 
-// The pair lists, one CTA per spin: for string x first x itself (pair index
+// The pair lists, a CTA per 512 strings: for string x first x itself (pair index
 // kPairMask), then its replacements to higher addresses (packed entries), from
-// off[x] on; off[ns] is the length.
-__global__ void __launch_bounds__(1024) k_rdm_lists(SpinTables A, SpinTables B, RdmSpin a, RdmSpin b) {
-    const SpinTables &S = blockIdx.x ? B : A;
-    const RdmSpin &R = blockIdx.x ? b : a;
-    if (R.nr == 0) return;
-    const int noff = S.nsingle - S.ne;
-    __shared__ int warp_sum[32];
+// off[x] on; off[ns] is the length.  Strings are in ascending order, so a+_k a_l goes
+// to a higher address where k > l, and the entries of the strings before a CTA's own
+// are counted from the bitmasks alone (one CTA per spin that carried the count along
+// took 33 us for 1716 strings, 350 for 12870).
+__global__ void __launch_bounds__(kListStrings) k_rdm_lists(SpinTables A, SpinTables B, int norb, RdmSpin a, RdmSpin b) {
+    const SpinTables &S = blockIdx.y ? B : A;
+    const RdmSpin &R = blockIdx.y ? b : a;
+    const int64_t x0 = (int64_t)blockIdx.x * kListStrings, x = x0 + threadIdx.x;
+    if (R.nr == 0 || x0 >= S.ns) return;
+    const uint32_t all = (1u << norb) - 1u;
+    auto count = [&](int64_t y) {
+        const uint32_t occ = S.str[y], empty = all & ~occ;
+        int n = 1;
+        for (uint32_t m = occ; m; m &= m - 1u) n += __popc(empty & ~(m ^ (m - 1u)));
+        return n;
+    };
+    int before = 0;
+    for (int64_t y = threadIdx.x; y < x0; y += kListStrings) before += count(y);
+    const int n = x < S.ns ? count(x) : 0;
+    __shared__ int warp_sum[kListStrings / 32], warp_before[kListStrings / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int carry = 0;
-    if (threadIdx.x == 0) R.off[0] = 0;
-    for (int64_t x0 = 0; x0 < S.ns; x0 += 1024) {
-        const int64_t x = x0 + threadIdx.x;
-        int n = 0;
-        if (x < S.ns) {
-            n = 1;
+    before = __reduce_add_sync(0xFFFFFFFFu, before);
+    int v = n;  // inclusive sum over the warp
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xFFFFFFFFu, v, o);
+        if (lane >= o) v += u;
+    }
+    if (lane == 31) {
+        warp_sum[warp] = v;
+        warp_before[warp] = before;
+    }
+    __syncthreads();
+    for (int w = 0; w < kListStrings / 32; ++w) v += warp_before[w] + (w < warp ? warp_sum[w] : 0);
+    if (x >= S.ns) return;
+    if (x == 0) R.off[0] = 0;
+    R.off[x + 1] = v;
+    uint32_t *out = R.ent + (v - n);
+    *out++ = (uint32_t)x | (kPairMask << kPairShift);
+    const int noff = S.nsingle - S.ne;
 #pragma unroll 8
-            for (int e = 0; e < noff; ++e) n += (int64_t)ent_target(S.tabo[(int64_t)e * S.ns + x]) > x;
-        }
-        int v = n;  // inclusive sum over the block
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xFFFFFFFFu, v, o);
-            if (lane >= o) v += u;
-        }
-        if (lane == 31) warp_sum[warp] = v;
-        __syncthreads();
-        int before = 0, all = 0;
-        for (int w = 0; w < 32; ++w) {
-            if (w < warp) before += warp_sum[w];
-            all += warp_sum[w];
-        }
-        v += before + carry;
-        if (x < S.ns) {
-            R.off[x + 1] = v;
-            uint32_t *out = R.ent + (v - n);
-            *out++ = (uint32_t)x | (kPairMask << kPairShift);
-#pragma unroll 8
-            for (int e = 0; e < noff; ++e) {
-                const uint32_t t = S.tabo[(int64_t)e * S.ns + x];
-                if ((int64_t)ent_target(t) > x) *out++ = t;
-            }
-        }
-        carry += all;
-        __syncthreads();
+    for (int e = 0; e < noff; ++e) {
+        const uint32_t t = S.tabo[(int64_t)e * S.ns + x];
+        if ((int64_t)ent_target(t) > x) *out++ = t;
     }
 }
 
@@ -232,6 +234,7 @@ __global__ void __launch_bounds__(1024) k_rdm_bins(SpinTables A, SpinTables B, R
 // Small spaces, one launch: a CTA per pair of orbitals {k, l} finds the strings'
 // entries of that pair in the tables (to higher addresses, or E_kk), and its
 // warps add their dots lane by lane; one reduction at the end.
+constexpr int kScan = 4;  // table entries per thread in flight
 template <typename T>
 __global__ void __launch_bounds__(256) k_rdm_small(const T *__restrict__ C, SpinTables A, SpinTables B, int norb,
                                                    double *__restrict__ gamma) {
@@ -246,24 +249,31 @@ __global__ void __launch_bounds__(256) k_rdm_small(const T *__restrict__ C, Spin
         const int ns = spin ? nsb : nsa, len = spin ? nsa : nsb;         // strings, length of a dot
         const int ld = spin ? 1 : nsb, step = spin ? nsb : 1;            // between strings, along a dot
         const int total = ns * S.nsingle;
-        for (int t0 = threadIdx.x - lane; t0 < total; t0 += 256) {
-            const int t = t0 + lane;
-            uint32_t e = 0;
-            int x = 0;
-            bool match = false;
-            if (t < total) {
-                e = S.tab[t];
-                x = t % ns;
-                match = (int)ent_pair(e) == P && (k == l || (int)ent_target(e) > x);
+        for (int t0 = threadIdx.x - lane; t0 < total; t0 += 256 * kScan) {
+            uint32_t es[kScan];
+#pragma unroll
+            for (int u = 0; u < kScan; ++u) {
+                const int t = t0 + u * 256 + lane;
+                es[u] = t < total ? S.tab[t] : kPairMask << kPairShift;  // no pair has that index
             }
-            for (uint32_t m = __ballot_sync(0xFFFFFFFFu, match); m; m &= m - 1u) {
-                const int from = __ffs(m) - 1;
-                const uint32_t ee = __shfl_sync(0xFFFFFFFFu, e, from);
-                const int xx = __shfl_sync(0xFFFFFFFFu, x, from);
-                const T *u = C + (size_t)xx * ld, *v = C + (size_t)ent_target(ee) * ld;
-                double d = 0.0;
-                for (int i = lane; i < len; i += 32) d = fma((double)u[(size_t)i * step], (double)v[(size_t)i * step], d);
-                acc += ent_negative(ee) ? -d : d;
+#pragma unroll
+            for (int u = 0; u < kScan; ++u) {
+                const uint32_t e = es[u];
+                int x = 0;
+                bool match = false;
+                if ((int)ent_pair(e) == P) {
+                    x = (t0 + u * 256 + lane) % ns;
+                    match = k == l || (int)ent_target(e) > x;
+                }
+                for (uint32_t m = __ballot_sync(0xFFFFFFFFu, match); m; m &= m - 1u) {
+                    const int from = __ffs(m) - 1;
+                    const uint32_t ee = __shfl_sync(0xFFFFFFFFu, e, from);
+                    const int xx = __shfl_sync(0xFFFFFFFFu, x, from);
+                    const T *a = C + (size_t)xx * ld, *b = C + (size_t)ent_target(ee) * ld;
+                    double d = 0.0;
+                    for (int i = lane; i < len; i += 32) d = fma((double)a[(size_t)i * step], (double)b[(size_t)i * step], d);
+                    acc += ent_negative(ee) ? -d : d;
+                }
             }
         }
     }
@@ -279,9 +289,18 @@ __global__ void __launch_bounds__(256) k_rdm_small(const T *__restrict__ C, Spin
     }
 }
 
-// Up to this many determinants the one launch is the faster way (CAS(9; 5,4), 15876:
-// 65 us; CAS(10,10), 63504: 175 us against 100 us).
-constexpr int64_t kSmallDets = 20000;
+// Where the one launch is the faster way: few elements in the dots of a pair of orbitals
+// (CAS(9; 5,4), 8800: 53 us against 72; (11; 3,3), 11000: 79 against 70; CAS(10,10), 32000:
+// 143 against 74), some more where one spin has few strings, which leave the other kernels
+// few CTAs ((11; 2,5), 10600; (18; 1,4), 12600).  With one alpha string the other kernels'
+// only work is the beta spin's, whose columns lie together, and the search through the
+// tables costs more from about 30000 entries on ((11; 11,5), 16000: 40 against 50; (12;
+// 12,6), 39000: 72 against 60; (16; 16,8), 927000: 636 against 485).
+bool one_launch(const fci_ctx *ctx) {
+    const SpinTables &A = ctx->A, &B = ctx->B;
+    const int64_t limit = std::min(A.ns, B.ns) < 64 ? 13000 : 10000;
+    return ctx->ndet * (A.nsingle + B.nsingle) <= 2 * limit * ctx->npair && (A.ns > 1 || B.ns * B.nsingle <= 30000);
+}
 
 // Entries of a spin's pair list: a string each and half of the off-diagonal replacements.
 int64_t pair_count(const SpinTables &S) { return S.ns + S.ns * (int64_t)(S.nsingle - S.ne) / 2; }
@@ -297,7 +316,7 @@ struct RdmPlan {
 
     RdmPlan(const fci_ctx *ctx, int max_chunks) {
         const SpinTables &A = ctx->A, &B = ctx->B;
-        if (ctx->ndet <= kSmallDets) {  // gamma alone
+        if (one_launch(ctx)) {  // gamma alone
             doubles = (size_t)ctx->norb * ctx->norb;
             return;
         }
@@ -310,11 +329,11 @@ struct RdmPlan {
             at += (size_t)((S.ns + 2) / 2 + (R.np + 1) / 2 + R.np * nr);
         };
         spin(A, a, 1, ga);
-        // enough row chunks to give every SM two blocks, at least 16 rows each
+        // enough row chunks to give every SM two blocks, at least kMinRows rows each
         int chunks = 1;
         if (B.nsingle) {
             const int64_t blocks = (pair_count(B) + kPairsPerBlock - 1) / kPairsPerBlock;
-            chunks = (int)std::min<int64_t>(std::max<int64_t>(1, 304 / blocks), std::max<int64_t>(1, A.ns / 16));
+            chunks = (int)std::min<int64_t>(std::max<int64_t>(1, 304 / blocks), std::max<int64_t>(1, A.ns / kMinRows));
             chunks = std::min(chunks, max_chunks);
             rows = (A.ns + chunks - 1) / chunks;
             chunks = (int)((A.ns + rows - 1) / rows);
@@ -339,7 +358,7 @@ struct RdmPlan {
 template <typename T>
 int launch_rdm1(fci_ctx *ctx, const T *C, const RdmPlan &P, cudaStream_t s) {
     const SpinTables &A = ctx->A, &B = ctx->B;
-    if (ctx->ndet <= kSmallDets) {
+    if (one_launch(ctx)) {
         k_rdm_small<T><<<ctx->npair, 256, 0, s>>>(C, A, B, ctx->norb, P.gamma);
         FCI_CUDA(cudaGetLastError());
         return FCI_OK;
@@ -351,7 +370,8 @@ int launch_rdm1(fci_ctx *ctx, const T *C, const RdmPlan &P, cudaStream_t s) {
         b.ent = a.ent;
     }
     if (a.nr || b.nr) {
-        k_rdm_lists<<<shared ? 1 : 2, 1024, 0, s>>>(A, B, a, b);
+        k_rdm_lists<<<dim3(ceil_div(std::max(A.ns, B.ns), kListStrings), shared ? 1 : 2), kListStrings, 0, s>>>(
+            A, B, ctx->norb, a, b);
         FCI_CUDA(cudaGetLastError());
     }
     if (a.nr) {
