@@ -1117,15 +1117,18 @@ int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *v
         if (maxsub > ctx->ndet) maxsub = (int)ctx->ndet;
         const int keepn = std::max(nroots, std::min(8, maxsub / 2));
         const bool mixed = ctx->opt.precision == FCI_PREC_MIXED;
-        size_t fr = 0, tot = 0;
-        FCI_CUDA(cudaMemGetInfo(&fr, &tot));
-        size_t avail = fr > ((size_t)2 << 30) ? fr - ((size_t)2 << 30) : 0;  // 2 GiB left for the runtime
-        if (ctx->opt.max_device_bytes > 0) {
-            const double cap = ctx->opt.max_device_bytes - (double)ctx->bytes;
-            avail = std::min(avail, cap > 0 ? (size_t)cap : (size_t)0);
-        }
-        const bool f32b = mixed && (ctx->opt.basis_f32 == 1 ||
-                                    (ctx->opt.basis_f32 == 0 && f64_basis_bytes(ctx->ndet, maxsub, keepn, nroots, mixed) > avail));
+        const size_t need = f64_basis_bytes(ctx->ndet, maxsub, keepn, nroots, mixed);
+        size_t avail = 0;
+        do {  // once more without the scratch kept for the density calls
+            size_t fr = 0, tot = 0;
+            FCI_CUDA(cudaMemGetInfo(&fr, &tot));
+            avail = fr > ((size_t)2 << 30) ? fr - ((size_t)2 << 30) : 0;  // 2 GiB left for the runtime
+            if (ctx->opt.max_device_bytes > 0) {
+                const double cap = ctx->opt.max_device_bytes - (double)ctx->bytes;
+                avail = std::min(avail, cap > 0 ? (size_t)cap : (size_t)0);
+            }
+        } while (need > avail && drop_idle_scratch(ctx));
+        const bool f32b = mixed && (ctx->opt.basis_f32 == 1 || (ctx->opt.basis_f32 == 0 && need > avail));
         if (f32b) {
             FCI_CUDA(cudaDeviceSynchronize());  // caller's guess buffer is complete
             const int m = ctx->opt.basis_f32 == 1 ? maxsub : f32_basis_fit(ctx->ndet, nroots, std::min(maxsub, 8), avail);

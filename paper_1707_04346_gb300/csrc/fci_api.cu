@@ -27,18 +27,39 @@ int cuda_fail(cudaError_t e, const char *what) {
     return e == cudaErrorMemoryAllocation ? FCI_ERR_OOM : FCI_ERR_CUDA;
 }
 
+// Give back the density calls' scratch unless one of them has it; false when there
+// was none to give back.
+bool drop_idle_scratch(fci_ctx *ctx) {
+    std::lock_guard<std::mutex> lock(ctx->scratch_mu);
+    if (ctx->scratch_taken || !ctx->scratch) return false;
+    dfree(ctx, ctx->scratch, ctx->scratch_bytes);
+    ctx->scratch = nullptr;
+    ctx->scratch_bytes = 0;
+    return true;
+}
+
+// An allocation of the context: nullptr and FCI_ERR_OOM in *rc beyond
+// fci_options.max_device_bytes or where the device has no more memory, after the
+// scratch kept for the density calls has been given back.
 void *dalloc(fci_ctx *ctx, size_t bytes, int *rc) {
     if (*rc != FCI_OK || bytes == 0) return nullptr;
-    if (ctx->opt.max_device_bytes > 0 && (double)ctx->bytes + (double)bytes > ctx->opt.max_device_bytes) {
+    const double cap = ctx->opt.max_device_bytes;
+    auto beyond = [&]() { return cap > 0 && (double)ctx->bytes + (double)bytes > cap; };
+    if (beyond()) drop_idle_scratch(ctx);
+    if (beyond()) {
         char buf[200];
         snprintf(buf, sizeof(buf), "allocation of %zu bytes would exceed fci_options.max_device_bytes (%.0f; %zu held)",
-                 bytes, ctx->opt.max_device_bytes, ctx->bytes.load());
+                 bytes, cap, ctx->bytes.load());
         set_error(buf);
         *rc = FCI_ERR_OOM;
         return nullptr;
     }
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && drop_idle_scratch(ctx)) {
+        cudaGetLastError();
+        e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         char buf[160];

@@ -178,6 +178,7 @@ void prof_mark(fci_ctx *ctx, int rec, int i, cudaStream_t s);
 // Pinned host words: a density's kDensityWords (>= 30 x 30), then the Davidson driver's.
 constexpr int kDensityWords = 1024, kDavidsonWords = 32;
 int host_words(fci_ctx *ctx);     // make ctx->host_words
+bool drop_idle_scratch(fci_ctx *ctx);
 void *dalloc(fci_ctx *ctx, size_t bytes, int *rc);
 void dfree(fci_ctx *ctx, void *p, size_t bytes);
 
