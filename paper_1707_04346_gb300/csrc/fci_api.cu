@@ -87,7 +87,7 @@ int host_words(fci_ctx *ctx) {
 
 int DensityScratch::take(size_t bytes) {
     int rc = FCI_OK;
-    if (bytes <= kKeptScratch) {
+    if (!kept_ && bytes <= kKeptScratch) {
         std::lock_guard<std::mutex> lock(ctx->scratch_mu);
         kept_ = !ctx->scratch_taken;
         if (kept_) ctx->scratch_taken = true;

@@ -197,7 +197,7 @@ struct DensityScratch {
     DensityScratch(const DensityScratch &) = delete;
     DensityScratch &operator=(const DensityScratch &) = delete;
     ~DensityScratch();
-    int take(size_t bytes);
+    int take(size_t bytes);  // again, for less, where it failed
 
   private:
     bool kept_ = false;

@@ -397,12 +397,17 @@ template <typename T>
 int rdm_impl(fci_ctx *ctx, const T *C, double *gamma_host) {
     RdmPlan P(ctx, 1 << 20);
     DensityScratch mem(ctx);
-    if (int rc = mem.take(sizeof(double) * P.doubles)) return rc;
+    int rc = mem.take(sizeof(double) * P.doubles);
+    if (rc == FCI_ERR_OOM && P.b.nr > 1) {  // one row chunk needs a partial per pair only
+        P = RdmPlan(ctx, 1);
+        rc = mem.take(sizeof(double) * P.doubles);
+    }
+    if (rc) return rc;
     P.place(ctx, reinterpret_cast<double *>(mem.dev));
     const size_t bytes = sizeof(double) * ctx->norb * ctx->norb;
     if (mem.host) P.gamma = mem.host;  // the last kernel writes the density into pinned host memory
     cudaStream_t s = ctx->stream;
-    int rc = launch_rdm1<T>(ctx, C, P, s);
+    rc = launch_rdm1<T>(ctx, C, P, s);
     cudaError_t e = cudaSuccess;
     if (rc == FCI_OK && !mem.host) e = cudaMemcpyAsync(gamma_host, P.gamma, bytes, cudaMemcpyDeviceToHost, s);
     const cudaError_t done = cudaStreamSynchronize(s);

@@ -695,19 +695,26 @@ int rdm2_impl(fci_ctx *ctx, const T *C, double *g1_host, double *g2_host) {
     else
         chunk = (chunk + round - 1) / round * round;
     if (chunk > nks) chunk = nks;
-    // one allocation: planes, Gram integers, results, statistics, c's integers, rows
-    size_t total = 0;
-    auto part = [&](size_t bytes) {
-        const size_t at = total;
-        total += (bytes + 255) / 256 * 256;
-        return at;
-    };
+    // one allocation: planes, Gram integers, results, statistics, c's integers, rows; with
+    // smaller chunks (down to one flush group) where it does not fit
+    size_t total = 0, o_dg = 0, o_stat = 0, o_G = 0, o_out = 0, o_x = 0, o_rows = 0;
     const size_t gbytes = sizeof(long long) * 2 * ((size_t)bs.Rd * bs.Rd + (size_t)ba.Rd * ba.Rd);
-    const size_t o_dg = part(step_bytes * (size_t)chunk), o_stat = part(sizeof(int) * 2), o_G = part(gbytes),
-                 o_out = part(sizeof(double) * (size_t)(n4 + n2)), o_x = part(sizeof(long long) * (size_t)N),
-                 o_rows = part(sizeof(uint16_t) * ((size_t)ctx->A.ns * ctx->A.nsingle + (size_t)ctx->B.ns * ctx->B.nsingle));
     DensityScratch scratch(ctx);
-    if (int rc = scratch.take(total)) return rc;
+    for (;;) {
+        total = 0;
+        auto part = [&](size_t bytes) {
+            const size_t at = total;
+            total += (bytes + 255) / 256 * 256;
+            return at;
+        };
+        o_dg = part(step_bytes * (size_t)chunk), o_stat = part(sizeof(int) * 2), o_G = part(gbytes);
+        o_out = part(sizeof(double) * (size_t)(n4 + n2)), o_x = part(sizeof(long long) * (size_t)N);
+        o_rows = part(sizeof(uint16_t) * ((size_t)ctx->A.ns * ctx->A.nsingle + (size_t)ctx->B.ns * ctx->B.nsingle));
+        const int rc = scratch.take(total);
+        if (rc == FCI_OK) break;
+        if (rc != FCI_ERR_OOM || chunk <= kKTile) return rc;
+        chunk = std::max<int64_t>(kKTile, chunk / 2 / kKTile * kKTile);
+    }
     unsigned char *mem = scratch.dev;
     unsigned char *dg = mem + o_dg;
     unsigned long long *G = reinterpret_cast<unsigned long long *>(mem + o_G);
