@@ -91,6 +91,15 @@ typedef struct fci_options {
     double max_device_bytes; /* cap on the device memory one context (with its Davidson
                             workspace) may hold; an allocation beyond it fails with
                             FCI_ERR_OOM before cudaMalloc is called.  0 = no cap (default).
+                            What only makes calls faster gives way: the scratch kept for
+                            the densities, and the planes of the FP32 products (about 6
+                            bytes per element of each G_s that is not in an all-zero
+                            16-column step, and 18 per determinant where the FP64 kernels
+                            have no planes), which fci_init leaves out where they do not
+                            fit and fci_davidson gives back where its workspace or a
+                            larger basis needs the room (not after an FP32 fci_sigma
+                            was captured in a graph); FP32 sigma then uses the kernels
+                            that need none.
                             (Resource control; no counterpart in the paper.) */
     int f32_row_global;  /* FCI_F32 tensor-core sigma_3: 1 = keep the sigma row in global
                             memory (the epilogue large spaces such as CAS(18,18) need) even

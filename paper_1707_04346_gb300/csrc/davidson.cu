@@ -1102,43 +1102,56 @@ static int run_davidson_f32basis(fci_ctx *ctx, int nroots, double tol, double *e
 
 // Device bytes of the FP64-basis workspace, and the largest FP32-basis
 // subspace (<= want) that fits in `avail` bytes (0 when none does).
+constexpr size_t kSolveSmall = (size_t)256 << 10;  // matrices, partial sums and scalars
 static size_t f64_basis_bytes(int64_t n, int maxsub, int keepn, int nroots, bool mixed) {
     return (size_t)n * 8 * (size_t)(2 * maxsub + 2 * keepn + nroots) + (mixed ? (size_t)n * 8 : 0);
 }
+static size_t f32_basis_bytes(int64_t n, int m, int nroots) {
+    return (size_t)n * 4 * (size_t)(2 * m + 1) + (size_t)n * 8 * 2 * nroots;
+}
 static int f32_basis_fit(int64_t n, int nroots, int want, size_t avail) {
     for (int m = want; m >= 2 * nroots && m >= 2; --m)
-        if ((size_t)n * 4 * (size_t)(2 * m + 1) + (size_t)n * 8 * 2 * nroots <= avail) return m;
+        if (f32_basis_bytes(n, m, nroots) <= avail) return m;
     return 0;
 }
 
 int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *vecs, const void *guess) {
+    using clk = std::chrono::steady_clock;
+    const auto t0 = clk::now();
+    FCI_CUDA(cudaDeviceSynchronize());  // the caller's guess buffer is complete, no sigma is in flight
     {  // basis storage: FP64, or FP32 (mixed precision) where asked for or where FP64 does not fit
         int maxsub = std::min(32, std::max(ctx->opt.max_subspace, 2 * nroots));
         if (maxsub > ctx->ndet) maxsub = (int)ctx->ndet;
         const int keepn = std::max(nroots, std::min(8, maxsub / 2));
         const bool mixed = ctx->opt.precision == FCI_PREC_MIXED;
         const size_t need = f64_basis_bytes(ctx->ndet, maxsub, keepn, nroots, mixed);
+        const int want32 = ctx->opt.basis_f32 == 1 ? maxsub : std::min(maxsub, 8);
+        const size_t all = kSolveSmall + (mixed && ctx->opt.basis_f32 == 1 ? f32_basis_bytes(ctx->ndet, maxsub, nroots) : need);
+        const size_t spare = mixed ? (size_t)2 << 30 : 0;  // left for the runtime
         size_t avail = 0;
-        do {  // once more without the scratch kept for the density calls
+        // whether the FP32 tables' memory lets the basis fit, or an FP32 basis be larger
+        auto tables_help = [&]() {
+            const size_t gain = f32_table_bytes(ctx);
+            return all <= avail + gain || (mixed && ctx->opt.basis_f32 == 0 &&
+                                           f32_basis_fit(ctx->ndet, nroots, want32, avail) <
+                                               f32_basis_fit(ctx->ndet, nroots, want32, avail + gain));
+        };
+        do {  // once more without the scratch kept for the density calls, then without the FP32 tables
             size_t fr = 0, tot = 0;
             FCI_CUDA(cudaMemGetInfo(&fr, &tot));
-            avail = fr > ((size_t)2 << 30) ? fr - ((size_t)2 << 30) : 0;  // 2 GiB left for the runtime
+            avail = fr > spare ? fr - spare : 0;
             if (ctx->opt.max_device_bytes > 0) {
                 const double cap = ctx->opt.max_device_bytes - (double)ctx->bytes;
                 avail = std::min(avail, cap > 0 ? (size_t)cap : (size_t)0);
             }
-        } while (need > avail && drop_idle_scratch(ctx));
+        } while (all > avail && (drop_idle_scratch(ctx) || (tables_help() && drop_f32_tables(ctx))));
         const bool f32b = mixed && (ctx->opt.basis_f32 == 1 || (ctx->opt.basis_f32 == 0 && need > avail));
         if (f32b) {
-            FCI_CUDA(cudaDeviceSynchronize());  // caller's guess buffer is complete
-            const int m = ctx->opt.basis_f32 == 1 ? maxsub : f32_basis_fit(ctx->ndet, nroots, std::min(maxsub, 8), avail);
+            const int m = ctx->opt.basis_f32 == 1 ? maxsub : f32_basis_fit(ctx->ndet, nroots, want32, avail);
             if (m == 0) return fail(FCI_ERR_OOM, "Davidson: not even an FP32 basis of 2 vectors per root fits");
             return run_davidson_f32basis(ctx, nroots, tol, energies, vecs, guess, m);
         }
     }
-    using clk = std::chrono::steady_clock;
-    const auto t0 = clk::now();
-    FCI_CUDA(cudaDeviceSynchronize());  // caller's guess buffer is complete
     Work W;
     W.ctx = ctx;
     W.s = ctx->stream;

@@ -78,6 +78,17 @@ void dfree(fci_ctx *ctx, void *p, size_t bytes) {
     ctx->bytes -= bytes;
 }
 
+int grow_buffer(fci_ctx *ctx, void **p, size_t *held, size_t bytes) {
+    if (bytes <= *held) return FCI_OK;
+    int rc = FCI_OK;
+    void *q = dalloc(ctx, bytes, &rc);
+    if (rc) return rc;  // the old one stays
+    dfree(ctx, *p, *held);
+    *p = q;
+    *held = bytes;
+    return FCI_OK;
+}
+
 int host_words(fci_ctx *ctx) {
     std::lock_guard<std::mutex> lock(ctx->scratch_mu);
     if (!ctx->host_words)

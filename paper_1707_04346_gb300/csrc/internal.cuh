@@ -148,6 +148,10 @@ struct fci_ctx {
     // FP32 same-spin terms as dense products (sigma_ss32.cu): bf16 slices of G_s
     fci::SsOperand ss32Ga, ss32Gb;
     int ss32_rows = 0;
+    // the FP32 tables (ss32G*, rowexp32) may be given back: what was made for them alone,
+    // and whether a graph may hold their addresses
+    bool f32_own_planes = false, f32_own_c = false, f32_own_tabp = false;
+    bool f32_captured = false;
     int *ssEr = nullptr, *ssEc = nullptr;
     double *hdiag = nullptr;        // [ndet]
     int *d_err = nullptr;           // device error word (bounded waits that gave up)
@@ -179,6 +183,8 @@ void prof_mark(fci_ctx *ctx, int rec, int i, cudaStream_t s);
 constexpr int kDensityWords = 1024, kDavidsonWords = 32;
 int host_words(fci_ctx *ctx);     // make ctx->host_words
 bool drop_idle_scratch(fci_ctx *ctx);
+bool drop_f32_tables(fci_ctx *ctx);  // tables.cu
+size_t f32_table_bytes(const fci_ctx *ctx);
 void *dalloc(fci_ctx *ctx, size_t bytes, int *rc);
 void dfree(fci_ctx *ctx, void *p, size_t bytes);
 
@@ -221,7 +227,7 @@ int launch_sigma(fci_ctx *ctx, const void *c, void *sigma, int dtype, cudaStream
 // square n x n matrix of floats (elem 4), doubles (elem 8) or 64-bit integers
 // (elem -8; half must be 0)
 int sym_pairs(void *y, int64_t n, int elem, int sgn, int half, cudaStream_t s);
-bool f32_same_spin_tc(const fci_ctx *ctx);
+bool f32_same_spin_tc(const fci_ctx *ctx, bool planes = true);
 int alloc_sigma_workspace(fci_ctx *ctx);  // at fci_init: ws32 when the FP32 same-spin tensor-core path is used
 
 // FP64 sigma of one batched instance (sliced sigma_3, double-float same-spin
@@ -254,6 +260,8 @@ int launch_sigma3_sliced(fci_ctx *ctx, const double *C, double *sig, cudaStream_
 int prepare_sigma3_sliced(const fci_ctx *ctx);
 
 int build_pair_table16(fci_ctx *ctx);  // SpinTables::tabp of the beta spin
+void free_pair_table16(fci_ctx *ctx);
+int grow_buffer(fci_ctx *ctx, void **p, size_t *held, size_t bytes);  // made, or made larger
 
 // sigma3_f32.cu (FP32 sigma_3 with the sigma row in shared memory)
 bool sigma3_f32_ok(const fci_ctx *ctx);
@@ -278,6 +286,7 @@ int launch_sigma_ss(fci_ctx *ctx, const double *C, double *sig, int which, cudaS
 
 int ss_kstep_lists(fci_ctx *ctx, const SpinTables &T, int nb, SsOperand &O, int **slot, size_t *slot_bytes);
 int alloc_c_planes(fci_ctx *ctx, size_t row_bytes, size_t col_bytes);
+void free_c_planes(fci_ctx *ctx);
 void free_ss_operand(fci_ctx *ctx, SsOperand &O, int64_t ns);
 
 // sigma_ss32.cu (FP32 sigma_1 / sigma_2 as dense tensor-core products)

@@ -304,7 +304,8 @@ __global__ void __launch_bounds__(512, 1) k_sigma2_cols_df(const double *__restr
 // starts at zero and both adds are atomic; two addends onto zero give the
 // same sum in either order.  Up to kFusedStrings strings, where the dense products'
 // pipeline (sigma_ss32.cu) costs more than the table walk: 252 strings (CAS(10,10))
-// 28 us against 38, 330 strings 34 against 38, 462 strings 47 against 43.
+// 28 us against 38, 330 strings 34 against 38, 462 strings 47 against 43; above, where
+// the context has no planes for the products (see build_f32_tables).
 constexpr int64_t kFusedStrings = 400;
 template <int R>
 __global__ void __launch_bounds__(512) k_sigma12_f32(const float *__restrict__ C, float *__restrict__ sig,
@@ -503,31 +504,51 @@ static size_t smem_limit() {
     return (size_t)lim;
 }
 
+// Rows per block of the fused FP32 sigma_1 + sigma_2 (0: not one string space, or
+// four rows and columns do not fit in shared memory).
+static int fused_rows(const fci_ctx *ctx) {
+    const SpinTables &A = ctx->A, &B = ctx->B;
+    if (A.ne != B.ne || A.ns != B.ns || A.nsingle == 0) return 0;
+    for (int r : {8, 4})
+        if ((size_t)2 * r * A.ns * sizeof(float) <= smem_limit()) return r;
+    return 0;
+}
+
 // Whether FP32 sigma_1/sigma_2 run through intermediate strings on the tensor
-// cores (asked for, or neither the dense products nor the staged same-spin
-// kernels fit); that path
+// cores (asked for, or neither the dense products, unless planes is false, nor the
+// fused or staged same-spin kernels fit); that path
 // needs the 2N-float workspace ws32, which fci_init allocates.
-bool f32_same_spin_tc(const fci_ctx *ctx) {
+bool f32_same_spin_tc(const fci_ctx *ctx, bool planes) {
     const SpinTables &A = ctx->A, &B = ctx->B;
     const size_t lim = smem_limit();
     auto fits = [&](int r, int64_t len) { return (size_t)r * len * sizeof(float) <= lim; };
     const bool tc_ok = A.nsingle > 0 && B.nsingle > 0 && ctx->npair + 1 <= 256 && A.nsingle <= 96 &&
                        B.nsingle <= 96;
-    return tc_ok && (ctx->opt.same_spin_tc == 1 || (!sigma_ss32_ok(ctx) && (!fits(4, B.ns) || !fits(4, A.ns))));
+    return tc_ok && (ctx->opt.same_spin_tc == 1 || (!(planes && sigma_ss32_ok(ctx)) && fused_rows(ctx) == 0 &&
+                                                   (A.ne == B.ne || !fits(4, B.ns) || !fits(4, A.ns))));
 }
 
 static bool sigma12_fused_ok(const fci_ctx *ctx) {
-    return ctx->A.ne == ctx->B.ne && ctx->A.ns == ctx->B.ns && ctx->A.nsingle > 0 && ctx->A.ns <= kFusedStrings &&
-           !f32_same_spin_tc(ctx);
+    return fused_rows(ctx) > 0 && (ctx->A.ns <= kFusedStrings || !sigma_ss32_ok(ctx));
+}
+
+static int prepare_sigma12_f32(const fci_ctx *ctx) {
+    const int R = fused_rows(ctx);
+    if ((size_t)2 * R * ctx->A.ns * sizeof(float) > 48 * 1024)
+        FCI_CUDA(opt_in_max_smem(R == 8 ? (const void *)k_sigma12_f32<8> : (const void *)k_sigma12_f32<4>, ctx->device));
+    return FCI_OK;
 }
 
 static int launch_sigma12_f32(const fci_ctx *ctx, const float *C, float *sig, cudaStream_t s,
                               const int *active = nullptr) {
-    constexpr int R = 8;
     const int64_t ns = ctx->A.ns;
-    static_assert(2 * R * kFusedStrings * sizeof(float) <= 48 * 1024, "shared memory without an opt-in");
+    const int R = fused_rows(ctx);
+    const size_t sm = (size_t)2 * R * ns * sizeof(float);
     FCI_CUDA(cudaMemsetAsync(sig, 0, sizeof(float) * (size_t)ns * (size_t)ns, s));
-    k_sigma12_f32<R><<<ceil_div(ns, R), 512, (size_t)2 * R * ns * sizeof(float), s>>>(C, sig, ctx->A, active);
+    if (R == 8)
+        k_sigma12_f32<8><<<ceil_div(ns, R), 512, sm, s>>>(C, sig, ctx->A, active);
+    else
+        k_sigma12_f32<4><<<ceil_div(ns, R), 512, sm, s>>>(C, sig, ctx->A, active);
     FCI_CUDA(cudaGetLastError());
     return FCI_OK;
 }
@@ -564,7 +585,7 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
     // both FP32 same-spin terms as dense tensor-core products in one launch
     const bool ss32 = sizeof(T) == 4 && !same_tc && sigma_ss32_ok(ctx);
     // or, for few strings of one space, by the fused table walk (no parity)
-    const bool fused = sizeof(T) == 4 && sigma12_fused_ok(ctx);
+    const bool fused = sizeof(T) == 4 && !same_tc && sigma12_fused_ok(ctx);
     // profiled kernels (fci_profile_read)
     static const char *const names3[3] = {"sigma1_rows", "sigma2_cols", sizeof(T) == 4 ? "sigma3_tc" : "sigma3_exact"};
     static const char *const names3tc[3] = {"sigma2_tc", "sigma1_tc", "sigma3_tc"};
@@ -649,8 +670,10 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
         add1 = 1;
     }
     if (fused) {
-        if constexpr (sizeof(T) == 4)
+        if constexpr (sizeof(T) == 4) {
+            if (int rc = prepare_sigma12_f32(ctx)) return rc;
             if (int rc = launch_sigma12_f32(ctx, (const float *)C, (float *)sig, s)) return rc;
+        }
         prof_mark(ctx, rec, 0, s);
     } else if (ss32) {
         if constexpr (sizeof(T) == 4)
@@ -733,11 +756,15 @@ static int sigma_impl(fci_ctx *ctx, const T *C, T *sig, cudaStream_t s, int pari
 // sigma_3 (sigma is then zeroed even when the instance is skipped).  The kernels'
 // shared memory limits are set once by prepare_sigma_f32_gated (outside any capture).
 bool sigma_f32_gated_ok(const fci_ctx *ctx) {
-    return sigma_small_ok(ctx, FCI_F32) || (sigma_ss32_ok(ctx) && sigma3_tc_smem(ctx, ctx->opt.f32_splits) > 0);
+    return sigma_small_ok(ctx, FCI_F32) ||
+           ((sigma_ss32_ok(ctx) || sigma12_fused_ok(ctx)) && sigma3_tc_smem(ctx, ctx->opt.f32_splits) > 0);
 }
 
 int prepare_sigma_f32_gated(const fci_ctx *ctx) {
-    return sigma_small_ok(ctx, FCI_F32) ? FCI_OK : prepare_sigma3_tc(ctx, ctx->opt.f32_splits);
+    if (sigma_small_ok(ctx, FCI_F32)) return FCI_OK;
+    if (sigma12_fused_ok(ctx))
+        if (int rc = prepare_sigma12_f32(ctx)) return rc;
+    return prepare_sigma3_tc(ctx, ctx->opt.f32_splits);
 }
 
 int launch_sigma_f32_gated(fci_ctx *ctx, const float *C, float *sig, const int *active, cudaStream_t s) {
@@ -794,6 +821,12 @@ int launch_sigma_f64_gated(fci_ctx *ctx, const double *C, double *sig, const int
 
 int launch_sigma(fci_ctx *ctx, const void *c, void *sigma, int dtype, cudaStream_t s, int parity) {
     if (dtype == FCI_F64) return sigma_impl<double>(ctx, (const double *)c, (double *)sigma, s, parity);
+    if (dtype == FCI_F32 && (sigma_ss32_ok(ctx) || sigma3_f32_ok(ctx)) && !ctx->f32_captured) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+        if (e != cudaSuccess) cudaGetLastError();
+        ctx->f32_captured = e != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    }
     if (dtype == FCI_F32) return sigma_impl<float>(ctx, (const float *)c, (float *)sigma, s, parity);
     return fail(FCI_ERR_ARG, "dtype must be FCI_F64 or FCI_F32");
 }

@@ -440,13 +440,8 @@ int build_sigma3_f32(fci_ctx *ctx, const double *eri_host) {
     double wmax = 0.0;
     for (int64_t i = 0; i < (int64_t)n * n * n * n; ++i) wmax = std::fmax(wmax, std::fabs(eri_host[i]));
     if (wmax > 0) std::frexp(wmax, &ctx->eW32);  // |W| < 2^eW32
-    int rc = FCI_OK;
     const size_t bytes = sizeof(uint16_t) * ctx->opt.f32_splits * (size_t)ctx->A.ns * plane_pitch(ctx->B.ns);
-    if (bytes > ctx->planes_bytes) {
-        dfree(ctx, ctx->planes, ctx->planes_bytes);
-        ctx->planes = (uint16_t *)dalloc(ctx, bytes, &rc);
-        ctx->planes_bytes = rc ? 0 : bytes;
-    }
+    int rc = grow_buffer(ctx, (void **)&ctx->planes, &ctx->planes_bytes, bytes);
     if (!rc && !ctx->B.tabp) rc = build_pair_table16(ctx);
     ctx->rowexp32 = rc ? nullptr : (int *)dalloc(ctx, sizeof(int) * (size_t)ctx->A.ns, &rc);
     if (rc) return rc;

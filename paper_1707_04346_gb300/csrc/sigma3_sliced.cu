@@ -136,10 +136,14 @@ int build_pair_table16(fci_ctx *ctx) {
     return FCI_OK;
 }
 
+void free_pair_table16(fci_ctx *ctx) {
+    dfree(ctx, ctx->B.tabp, sizeof(uint16_t) * (size_t)round_up16(ctx->npair) * ctx->B.ns);
+    ctx->B.tabp = nullptr;
+}
+
 void free_sliced_tables(fci_ctx *ctx) {
     const int np = ctx->npair;
-    if (ctx->B.tabp) dfree(ctx, ctx->B.tabp, sizeof(uint16_t) * (size_t)((np + 15) / 16 * 16) * ctx->B.ns);
-    ctx->B.tabp = nullptr;
+    free_pair_table16(ctx);
     dfree(ctx, ctx->XW, sizeof(long long) * (size_t)np * np);
     dfree(ctx, ctx->rowexp, sizeof(int) * (size_t)ctx->A.ns);
     dfree(ctx, ctx->planes, ctx->planes_bytes);

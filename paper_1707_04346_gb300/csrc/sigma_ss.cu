@@ -604,18 +604,15 @@ int build_ss_tables(fci_ctx *ctx) {
 // The operand planes of C by rows and by columns, shared by the FP64 and the FP32
 // products (each call writes all of what it reads): made, or made larger.
 int alloc_c_planes(fci_ctx *ctx, size_t row_bytes, size_t col_bytes) {
-    int rc = FCI_OK;
-    if (row_bytes > ctx->ssCr_bytes) {
-        dfree(ctx, ctx->ssCr, ctx->ssCr_bytes);
-        ctx->ssCr = (unsigned char *)dalloc(ctx, row_bytes, &rc);
-        ctx->ssCr_bytes = rc ? 0 : row_bytes;
-    }
-    if (!rc && col_bytes > ctx->ssCc_bytes) {
-        dfree(ctx, ctx->ssCc, ctx->ssCc_bytes);
-        ctx->ssCc = (unsigned char *)dalloc(ctx, col_bytes, &rc);
-        ctx->ssCc_bytes = rc ? 0 : col_bytes;
-    }
-    return rc;
+    if (int rc = grow_buffer(ctx, (void **)&ctx->ssCr, &ctx->ssCr_bytes, row_bytes)) return rc;
+    return grow_buffer(ctx, (void **)&ctx->ssCc, &ctx->ssCc_bytes, col_bytes);
+}
+
+void free_c_planes(fci_ctx *ctx) {
+    dfree(ctx, ctx->ssCr, ctx->ssCr_bytes);
+    dfree(ctx, ctx->ssCc, ctx->ssCc_bytes);
+    ctx->ssCr = ctx->ssCc = nullptr;
+    ctx->ssCr_bytes = ctx->ssCc_bytes = 0;
 }
 
 void free_ss_operand(fci_ctx *ctx, SsOperand &O, int64_t ns) {
@@ -630,11 +627,8 @@ void free_ss_tables(fci_ctx *ctx) {
     if (ctx->ssGb.lists != ctx->ssGa.lists) free_ss_operand(ctx, ctx->ssGb, B.ns);
     ctx->ssGb = SsOperand{};
     free_ss_operand(ctx, ctx->ssGa, A.ns);
-    dfree(ctx, ctx->ssCr, ctx->ssCr_bytes);
-    dfree(ctx, ctx->ssCc, ctx->ssCc_bytes);
-    ctx->ssCr_bytes = ctx->ssCc_bytes = 0;
+    free_c_planes(ctx);
     dfree(ctx, ctx->ssEr, sizeof(int) * (size_t)(A.ns + B.ns + 1));
-    ctx->ssCr = ctx->ssCc = nullptr;
     ctx->ssEr = ctx->ssEc = nullptr;
 }
 

@@ -349,11 +349,12 @@ bool sigma_ss32_ok(const fci_ctx *ctx) { return ctx->ss32Ga.planes != nullptr; }
 
 // Built where FCI_F32 covers the space at all (replacements of both spins on the
 // tensor cores, see sigma_tc.cu), neither string space exceeds 16384 strings (as
-// for the FP64 products) and the one-kernel sigma does not take the space anyway.
+// for the FP64 products) and neither the one-kernel sigma nor the caller's choice of
+// the intermediate-string kernels takes the space anyway.
 int build_ss32_tables(fci_ctx *ctx) {
     const SpinTables &A = ctx->A, &B = ctx->B;
     if (A.nsingle == 0 || B.nsingle == 0 || A.nsingle > 96 || ctx->npair > 256 || A.ns > 16384 || B.ns > 16384) return FCI_OK;
-    if (sigma_small_ok(ctx, FCI_F32)) return FCI_OK;
+    if (sigma_small_ok(ctx, FCI_F32) || ctx->opt.same_spin_tc == 1) return FCI_OK;
     int rc = FCI_OK, nsm = 0;
     cudaStream_t s = ctx->stream;
     FCI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));

@@ -375,6 +375,57 @@ static int build_spin(fci_ctx *ctx, SpinTables &T, int ne) {
     return build_tile_schedule(ctx, T);
 }
 
+static void free_f32_tables(fci_ctx *ctx) {
+    free_ss32_tables(ctx);
+    free_sigma3_f32(ctx);
+    if (ctx->f32_own_planes) {
+        dfree(ctx, ctx->planes, ctx->planes_bytes);
+        ctx->planes = nullptr;
+        ctx->planes_bytes = 0;
+    }
+    if (ctx->f32_own_c) free_c_planes(ctx);
+    if (ctx->f32_own_tabp) free_pair_table16(ctx);
+    ctx->f32_own_planes = ctx->f32_own_c = ctx->f32_own_tabp = false;
+}
+
+// The planes and tables of the faster FP32 kernels (sigma_ss32.cu, sigma3_f32.cu).
+// FP32 can do without (the fused, staged or intermediate-string kernels and the sigma_3
+// of sigma_tc.cu), so a context for which they leave no room is made without them.
+static int build_f32_tables(fci_ctx *ctx, const double *eri_host) {
+    ctx->f32_own_planes = !ctx->planes;
+    ctx->f32_own_c = !ctx->ssCr;
+    ctx->f32_own_tabp = !ctx->B.tabp;
+    int rc = build_ss32_tables(ctx);
+    if (!rc) rc = build_sigma3_f32(ctx, eri_host);
+    const double cap = ctx->opt.max_device_bytes;
+    if (!rc && cap > 0 && (double)ctx->bytes + 8.0 * (double)ctx->ndet + 4.0 > cap) rc = FCI_ERR_OOM;  // hdiag, d_err
+    if (rc == FCI_ERR_OOM) {
+        free_f32_tables(ctx);
+        set_error("");
+        rc = FCI_OK;
+    }
+    return rc;
+}
+
+size_t f32_table_bytes(const fci_ctx *ctx) {
+    const SsOperand &a = ctx->ss32Ga, &b = ctx->ss32Gb;
+    size_t n = a.plane_bytes + a.list_bytes + (b.lists != a.lists ? b.plane_bytes + b.list_bytes : 0);
+    if (ctx->f32_own_planes) n += ctx->planes_bytes;
+    if (ctx->f32_own_c) n += ctx->ssCr_bytes + ctx->ssCc_bytes;
+    return n;
+}
+
+// Give the FP32 tables back for another use of their memory: not once a captured
+// graph may hold their addresses, nor where FP32 would need them (a space that
+// sigma_tc.cu does not take, or a workspace that was not made).  The caller has
+// waited for the device.
+bool drop_f32_tables(fci_ctx *ctx) {
+    if ((!sigma_ss32_ok(ctx) && !sigma3_f32_ok(ctx)) || ctx->f32_captured) return false;
+    if (sigma3_tc_smem(ctx, ctx->opt.f32_splits) == 0 || (f32_same_spin_tc(ctx, false) && !ctx->ws32)) return false;
+    free_f32_tables(ctx);
+    return true;
+}
+
 int build_tables(fci_ctx *ctx, const double *h1_host, const double *eri_host) {
     const int n = ctx->norb;
     int rc = FCI_OK;
@@ -419,8 +470,7 @@ int build_tables(fci_ctx *ctx, const double *h1_host, const double *eri_host) {
     ctx->ndet = ctx->A.ns * ctx->B.ns;
     if ((rc = build_sliced_tables(ctx, h1_host, eri_host))) return rc;
     if ((sigma3_sliced_ok(ctx) || sigma_wide_ok(ctx)) && (rc = build_ss_tables(ctx))) return rc;
-    if ((rc = build_ss32_tables(ctx))) return rc;
-    if ((rc = build_sigma3_f32(ctx, eri_host))) return rc;
+    if ((rc = build_f32_tables(ctx, eri_host))) return rc;
     if ((rc = prepare_sigma_small(ctx))) return rc;
     if ((rc = alloc_sigma_workspace(ctx))) return rc;
     ctx->hdiag = (double *)dalloc(ctx, sizeof(double) * ctx->ndet, &rc);

@@ -73,3 +73,67 @@ def test_densities_take_less_scratch_where_room_is_short(pkg):
     ctx = pkg.fci_init(norb, na, nb, h1, eri, pkg.default_options(max_device_bytes=tables + room))
     assert np.abs(pkg.fci_rdm1(ctx, c) - g).max() < 1e-13 * (na + nb)
     pkg.fci_free(ctx)
+
+
+def f32_error(pkg, oracle_mod, ctx, space, h1, eri):
+    """Largest error of an FP32 sigma on sampled rows, in units of its largest element."""
+    c = fi.make_vector(ctx.ndet).astype(np.float32)
+    out = torch.empty(ctx.ndet, dtype=torch.float32, device="cuda")
+    pkg.fci_sigma(ctx, torch.from_numpy(c).cuda(), out)
+    rows = np.unique(np.random.default_rng(5).integers(0, ctx.ndet, 500)).astype(np.int64)
+    ref = oracle_mod.sigma_rows(*space, h1, eri, c.astype(np.float64), rows)
+    return np.abs(out.double().cpu().numpy()[rows] - ref).max() / np.abs(ref).max()
+
+
+# one string space (the fused kernel without planes: 8 rows, and 4 at 6435 strings), two spaces (staged)
+@pytest.mark.parametrize("space", [(12, 6, 6), (13, 6, 5), (15, 7, 7)])
+@pytest.mark.parametrize("f64_kernels", [0, 1])
+def test_contexts_without_room_for_the_fp32_planes(pkg, oracle_mod, space, f64_kernels):
+    """fci_init leaves the planes of the FP32 same-spin products out where they do not fit, and
+    FP32 sigma uses the kernels that need none."""
+    if space == (15, 7, 7) and f64_kernels == 0:
+        pytest.skip("the same FP32 kernels; 41 million determinants once are enough")
+    h1, eri = fi.make_integrals(space[0], 40)
+    ctx = pkg.fci_init(*space, h1, eri, pkg.default_options(f64_kernels=f64_kernels))
+    full = held(pkg, ctx)
+    pkg.fci_free(ctx)
+    ctx = pkg.fci_init(*space, h1, eri, pkg.default_options(f64_kernels=f64_kernels, max_device_bytes=float(full - 1)))
+    assert held(pkg, ctx) < full
+    assert f32_error(pkg, oracle_mod, ctx, space, h1, eri) <= 2e-6  # the bar of the FP32 kernels
+    pkg.fci_free(ctx)
+
+
+@pytest.mark.parametrize("space", [(12, 6, 6), (13, 6, 5)])
+def test_fp32_planes_give_way_to_a_solve(pkg, oracle_mod, space):
+    """A workspace that does not fit beside the planes of the FP32 products takes their place,
+    unless a captured graph may still read them."""
+    h1, eri = fi.make_integrals(space[0], 40)
+    opts = dict(f64_kernels=1, max_subspace=4, max_iter=2)  # FP64 kernels without planes of their own
+    ctx = pkg.fci_init(*space, h1, eri, pkg.default_options(**opts))
+    full, n = held(pkg, ctx), ctx.ndet
+    pkg.fci_free(ctx)
+    solve = 8 * n * (2 * 4 + 2 * 2 + 1)  # the vectors alone
+    for captured in (False, True):
+        ctx = pkg.fci_init(*space, h1, eri, pkg.default_options(max_device_bytes=float(full + solve - 4096), **opts))
+        assert held(pkg, ctx) == full
+        if captured:
+            c = torch.from_numpy(fi.make_vector(n).astype(np.float32)).cuda()
+            out = torch.empty_like(c)
+            pkg.fci_sigma(ctx, c, out)
+            want = out.clone()
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                pkg.fci_sigma(ctx, c, out)
+        with pytest.raises(pkg.FciError) as err:
+            pkg.fci_davidson(ctx, 1, 1e-12)
+        if captured:
+            assert err.value.code == pkg.fci.FCI_ERR_OOM and held(pkg, ctx) == full
+            out.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            assert float((out - want).abs().max()) <= 2e-6 * float(want.abs().max())
+        else:
+            assert err.value.code == pkg.fci.FCI_ERR_NOCONV and held(pkg, ctx) < full
+            assert f32_error(pkg, oracle_mod, ctx, space, h1, eri) <= 2e-6
+        pkg.fci_free(ctx)
