@@ -439,17 +439,9 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) k_ss_tc(SsArgs P) {
                     }
             }
             if (!ok) break;
-            // dm: the lane's share of the diagonal; P.C decides whether there is one, not
-            // the strides (with one beta string sigma_2's sn is 1 as well)
-            auto put = [&](int row, int n, long long V, int ea, int eb, double dm) {
-                const int64_t at = row * P.sm + n * P.sn;
-                const double v = element(V, ea, eb);
-                if (P.C)
-                    P.out[at] = fma(P.dn[n] + dm, P.C[at], P.out[at]) + v;
-                else
-                    P.out[at] += v;
-            };
-            if (kCols == 32 && P.sn == 1) {
+            // sigma_1's strides only (it carries no diagonal): with one beta string sigma_2
+            // has sm = sn = 1 (asking for P.C == nullptr here costs 6 us a product at CAS(14,14))
+            if (kCols == 32 && P.sn < P.sm) {
                 // a thread holds consecutive columns of one row: transpose the warp's
                 // 32 x 32 block so that its stores run along the row
 #pragma unroll
@@ -467,8 +459,10 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) k_ss_tc(SsArgs P) {
                     const int ebn = P.eB[n];
 #pragma unroll
                     for (int j = 0; j < kCols; ++j)
-                        if (m0 + j < P.M)
-                            put(m0 + j, n, acc[j], P.eA[m0 + j], ebn, P.C && P.dm ? P.dm[m0 + j] : 0.0);
+                        if (m0 + j < P.M) {
+                            const int eam = P.eA[m0 + j];
+                            P.out[(m0 + j) * P.sm + n] += element(acc[j], eam, ebn);
+                        }
                 }
             } else if (m < P.M) {
                 const int eam = P.eA[m];
@@ -476,7 +470,14 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) k_ss_tc(SsArgs P) {
 #pragma unroll
                 for (int j = 0; j < kCols; ++j) {
                     const int n = nb * NB + sub * kCols + j;
-                    if (n < P.N) put(m, n, acc[j], eam, P.eB[n], dm);
+                    if (n < P.N) {
+                        const double v = element(acc[j], eam, P.eB[n]);
+                        double *o = P.out + m * P.sm + n * P.sn;
+                        if (P.C)
+                            *o = fma(P.dn[n] + dm, P.C[m * P.sm + n * P.sn], *o) + v;
+                        else
+                            *o += v;
+                    }
                 }
             }
         }
