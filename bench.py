@@ -19,7 +19,9 @@ work has: a plain FP64 CPU implementation written from the paper).
 from __future__ import annotations
 
 import argparse
+import functools
 import hashlib
+import itertools
 import json
 import math
 import os
@@ -197,6 +199,23 @@ def cpu_baseline(norb, na, nb, h1, eri, c, target_s=15.0, seed=0):
                       f"{dt:.1f} s"}
 
 
+@functools.lru_cache(maxsize=None)
+def kept_elements(norb, ne, rows):
+    """Elements of one spin's same-spin Hamiltonian that the dense products multiply: per block of
+    `rows` strings, the 16-column steps that hold an off-diagonal nonzero (strings one or two
+    replacements apart; a block without any keeps one step)."""
+    s = np.array(sorted(sum(1 << p for p in occ) for occ in itertools.combinations(range(norb), ne)), dtype=np.uint32)
+    steps = -(-s.size // 16)
+    total = 0
+    for r in range(0, s.size, rows):
+        block = s[r:r + rows]
+        apart = np.bitwise_count(block[:, None] ^ s[None, :])
+        used = np.zeros(steps * 16, dtype=bool)
+        used[:s.size] = ((apart > 0) & (apart <= 4)).any(0)
+        total += block.size * 16 * max(1, int(used.reshape(steps, 16).any(1).sum()))
+    return total
+
+
 def kernel_work(name, norb, na, nb, N, sa, sb, nsa, nsb, peaks, f32_splits=3):
     """(bound, amount per launch, unit, peak, peak source, description) of one
     sigma kernel: the algorithmic work each kernel's roofline is taken on."""
@@ -222,18 +241,21 @@ def kernel_work(name, norb, na, nb, N, sa, sb, nsa, nsb, peaks, f32_splits=3):
                 f"FP32 operations: 12 per term x {nsame} terms per determinant")
     if name in ("sigma1_ss", "sigma2_ss"):  # FP64 same-spin terms as dense sliced products
         # one product of (strings of the summed spin) x (other spin) x (summed spin) in 21 digit
-        # products, zeros of the same-spin Hamiltonian included (K-steps that hold only zeros are
-        # not executed)
-        ns_sum = nsb if name == "sigma1_ss" else nsa
-        return ("tensor", 21 * 2.0 * ns_sum * N, "TFLOP/s", *bf16,
-                f"bf16 FLOP: 21 digit products x 2 x {ns_sum} per determinant, zeros included")
+        # products: the 16-column steps of the same-spin Hamiltonian that are not all zero
+        ns_sum, ne_sum, other = (nsb, nb, nsa) if name == "sigma1_ss" else (nsa, na, nsb)
+        rows = 96 if -(-other // 128) * -(-ns_sum // 96) * 2 >= GB300_SMS else 16
+        kept = kept_elements(norb, ne_sum, rows)
+        return ("tensor", 21 * 2.0 * kept * other, "TFLOP/s", *bf16,
+                f"bf16 FLOP: 21 digit products x 2 x {kept / ns_sum:.0f} of {ns_sum} columns per determinant")
     if name == "sigma12_f32":  # FP32 sigma_1 + sigma_2 by the tables: one FMA per term
         return ("alu", 2.0 * nsame * N, "Tops/s", fp32_pipe, fp32src,
                 f"FP32 FMAs: {nsame} terms per determinant, two spins")
     if name in ("sigma12_ss32", "sigma2_ss32"):  # FP32 same-spin terms as dense products of 3 bf16 slices
-        ns_sum = nsa + nsb if name == "sigma12_ss32" else nsa
-        return ("tensor", 6 * 2.0 * ns_sum * N, "TFLOP/s", *bf16,
-                f"bf16 FLOP: 6 slice products x 2 x {ns_sum} per determinant, zeros included")
+        macs = kept_elements(norb, na, 128) * nsb  # sigma_2; then sigma_1
+        if name == "sigma12_ss32":
+            macs += kept_elements(norb, nb, 128) * nsa
+        return ("tensor", 6 * 2.0 * macs, "TFLOP/s", *bf16,
+                f"bf16 FLOP: 6 slice products x 2 x {macs / N:.0f} per determinant (steps that are not all zero)")
     if name == "sigma3_tc":
         return ("tensor", prods32 * 2.0 * 128 * npad * kpad * tiles, "TFLOP/s", *bf16,
                 f"bf16 MMA FLOP: {prods32} slice products x 2 x 128 x {npad} x {kpad} x {tiles} tiles")
