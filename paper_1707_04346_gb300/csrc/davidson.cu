@@ -702,7 +702,7 @@ struct Work {
     double *partial = nullptr;              // [2][kDotBlocks][32]
     double *scal = nullptr;                 // [64] scalars
     double *rn2 = nullptr;                  // [nroots] residual norms squared
-    int *keep = nullptr;
+    int *keep = nullptr;                    // FP32 basis: kept flag of the last orthonormalisation
     int *counter = nullptr;                 // [4]: last-block counters (0, 1: dot sets; 2: others), 3: second-pass flag
     double *host = nullptr;                 // pinned, the context's: [17] k_publish, [24] keep flag
     int64_t *idx = nullptr;                 // [nroots]
@@ -1181,7 +1181,6 @@ int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *v
     W.partial = W.get<double>(2 * kDotBlocks * 32);
     W.scal = W.get<double>(64);
     W.rn2 = W.get<double>(8);
-    W.keep = W.get<int>(1);
     W.counter = W.get<int>(4);
     W.idx = W.get<int64_t>(8);
     W.pidx = W.get<int64_t>(kDotBlocks + 1);

@@ -70,7 +70,6 @@ namespace r2 {
 using sl::kSlices;
 using tc::kM;
 using sm::bulk_g2s;
-using sm::levels_to_int_f;
 using sm::mbar_expect_tx;
 
 constexpr int kThreads = 448;        // warp 0 copies, warp 1 issues the MMAs, warps 2-13 epilogue

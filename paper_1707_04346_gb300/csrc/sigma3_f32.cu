@@ -378,11 +378,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
 }
 
+// (no space of norb <= 30 with kMinRows strings has 32 replacements or fewer)
 template <int NS>
 static void *kernel(int kpad) {
     switch (kpad) {
-        case 16: return (void *)k_sigma3_f32<16, NS>;
-        case 32: return (void *)k_sigma3_f32<32, NS>;
         case 48: return (void *)k_sigma3_f32<48, NS>;
         case 64: return (void *)k_sigma3_f32<64, NS>;
         case 80: return (void *)k_sigma3_f32<80, NS>;
@@ -411,7 +410,7 @@ static bool plan(const fci_ctx *ctx, Plan *P) {
     const int ns = ctx->opt.f32_splits;
     P->kpad = (A.nsingle + 15) / 16 * 16;
     P->npad = (ctx->npair + 15) / 16 * 16;
-    if (A.nsingle == 0 || B.nsingle == 0 || P->kpad > 96 || P->npad > 256 || B.ns > 0x7FFF || B.nsingle > 96 ||
+    if (A.nsingle == 0 || B.nsingle == 0 || P->kpad < 48 || P->kpad > 96 || P->npad > 256 || B.ns > 0x7FFF || B.nsingle > 96 ||
         A.ns < kMinRows || B.ns < kMinStrings)
         return false;
     int lim = 0;
