@@ -55,11 +55,11 @@ NCU_TRAFFIC = {
     "sigma3_tc": ("paper_1707_04346_gb300/csrc/sigma3_f32.cu", "k_sigma3_f32(", "f894b1c00eede3f4", 221401344.0),
     "sigma3_sliced": ("paper_1707_04346_gb300/csrc/sigma3_sliced_kernel.cuh", "k_sigma3_sliced(", "0d1f7828b6d7bb70", 1077408768.0),
     # sigma_1 as a dense sliced product (k_ss_tc; sigma_2 runs the same kernel with the operands swapped)
-    "sigma1_ss": ("paper_1707_04346_gb300/csrc/sigma_ss.cu", "k_ss_tc(", "9edff8592af53966", 1402157568.0),
+    "sigma1_ss": ("paper_1707_04346_gb300/csrc/sigma_ss.cu", "k_ss_tc(", "0d8b373e2b3169e5", 1381889792.0),
     # the wide kernels at CAS(14,14) (bench.py --f64-kernels wide)
-    "sigma3_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "81d454a69f812b05", 1064472320.0),
-    "sigma1_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "81d454a69f812b05", 2521320704.0),
-    "sigma2_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "81d454a69f812b05", 2508126640.0),
+    "sigma3_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "1d4c993d3fc8435f", 1064472320.0),
+    "sigma1_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "1d4c993d3fc8435f", 2521320704.0),
+    "sigma2_wide": ("paper_1707_04346_gb300/csrc/sigma_wide_kernel.cuh", "k_sigma_wide(", "1d4c993d3fc8435f", 2508126640.0),
 }
 
 
@@ -678,7 +678,7 @@ def density_leg(pkg, norb, na, nb, h1, eri, c_dev, sigma_ms, peaks):
                                              "(profiles/kernel_traffic_cas14.md), scaled to this workload's planes",
                              "note": "executed bf16 MMA FLOP (6 digits, 12 products of the symmetric half, 128 x at most 80 tiles) per launch / "
                                      "CUDA-event time; peak = measured burst bf16"},
-        "timing": "whole blocking calls (allocation, statistics round trip, host copies included), median of 3",
+        "timing": "whole blocking calls (allocation and host copies included), median of 3",
     }
 
 

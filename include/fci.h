@@ -79,13 +79,16 @@ typedef struct fci_options {
     int precision;       /* FCI_PREC_FP64 (default) or FCI_PREC_MIXED */
     double mixed_switch; /* MIXED: residual reduction between FP64 refinements (default 1e-2) */
     double symmetry_tol; /* absolute tolerance of the h1/eri symmetry check (default 1e-12) */
-    int f32_splits;      /* FCI_F32 sigma_3 on the tensor cores: FP32 operands split into 2
-                            (split-BF16x3, ~1e-5 relative) or 3 (split-BF16x6, ~FP32) bf16
-                            slices; default 3 */
+    int f32_splits;      /* FCI_F32 sigma_3 on the tensor cores, and the same-spin terms with
+                            it where they go through intermediate strings: FP32 operands
+                            split into 2 (split-BF16x3, ~1e-5 relative) or 3 (split-BF16x6,
+                            ~FP32) bf16 slices; default 3.  The dense same-spin products
+                            always use 3 slices, the one-kernel sigma of small spaces none */
     int same_spin_tc;    /* FCI_F32 sigma_1 and sigma_2 through intermediate strings on the
                             tensor cores (Eq. 8's E_ij E_kl as a pair-matrix contraction):
-                            0 = only when the staged same-spin kernels do not fit in shared
-                            memory (default), 1 = always */
+                            0 = only where neither the dense products (up to 16384 strings
+                            per spin) nor the fused or staged same-spin kernels fit
+                            (default), 1 = always */
     int f64_kernels;     /* FCI_F64 sigma kernels: FCI_F64_AUTO (default), FCI_F64_FMA,
                             FCI_F64_SLICED or FCI_F64_WIDE, below */
     double max_device_bytes; /* cap on the device memory one context (with its Davidson
@@ -135,8 +138,9 @@ typedef struct fci_options {
  * tensor cores: every row of G_s and every row or column of C in 46-bit fixed
  * point relative to its own largest power of two, six 8-bit digits, exact
  * 64-bit integer sums; the diagonal of G_s in FP64.  Costs 12 bytes per
- * element of each G_s (141 MB at CAS(14,14), 2 GB at CAS(16,16)) at fci_init
- * and the same for two copies of C.  The results are bit-reproducible. */
+ * element of each G_s, all-zero 16-column steps of its 96- or 16-row blocks left out
+ * (128 MB at CAS(14,14), 1.3 GB at CAS(16,16)), at fci_init and 24 per determinant for
+ * two copies of C.  The results are bit-reproducible. */
 #define FCI_SS_AUTO 0
 #define FCI_SS_FAMILY 1
 
@@ -233,15 +237,18 @@ int fci_free_default(void);
  *  dtype     FCI_F64: FP64 vectors and FP64 accuracy (fci_options.f64_kernels
  *            and f64_same_spin say which kernels: tensor-core contractions of
  *            8-bit digit slices with exact integer sums, double-float FP32
- *            arithmetic, or FP64 FMAs).  FCI_F32: FP32 vectors;
- *            sigma_1/sigma_2 in FP32, sigma_3 on the tensor cores with bf16
- *            slices of the FP32 operands and FP32 accumulation (see
- *            fci_options.f32_splits); the low-precision phase of the mixed
- *            Davidson.  For large string spaces (or with
- *            fci_options.same_spin_tc = 1) sigma_1/sigma_2 also run on the
- *            tensor cores, through intermediate strings (Eq. 7 operators
- *            E_ij E_kl); their adds are atomic, so FP32 results may differ in
- *            the last bits between calls.  FCI_F32 needs the replacement lists
+ *            arithmetic, or FP64 FMAs).  FCI_F32: FP32 vectors, the
+ *            low-precision phase of the mixed Davidson: sigma_3 on the tensor
+ *            cores with bf16 slices of the FP32 operands (see
+ *            fci_options.f32_splits), sigma_1/sigma_2 up to 16384 strings per
+ *            spin as dense products with G_s, three bf16 slices per operand
+ *            (up to 400 strings of one space, and where their planes do not
+ *            fit, by FP32 kernels over the tables); small spaces in one
+ *            kernel of FP32 arithmetic.  For larger string spaces (or with
+ *            fci_options.same_spin_tc = 1) sigma_1/sigma_2 run through
+ *            intermediate strings on the tensor cores (Eq. 7 operators
+ *            E_ij E_kl); their adds are atomic, so those FP32 results may
+ *            differ in the last bits between calls.  FCI_F32 needs the replacement lists
  *            of both spins to have at most 96 entries (norb 18 at half
  *            filling) and at most 65408 strings per spin; FCI_F64 covers
  *            every space with at most 96 replacements per string and 255
@@ -251,8 +258,8 @@ int fci_free_default(void);
  *  stream    cudaStream_t or NULL.  Asynchronous; allocates nothing (the
  *            workspaces of the large-space FP32 path, 8N bytes, of the sliced
  *            FP64 sigma_3, 12N bytes, and of the dense same-spin products,
- *            24N bytes, are made at fci_init), so it can be captured in a
- *            CUDA graph.  The context's workspaces are shared
+ *            24N bytes (12N for FP32 alone), are made at fci_init), so it can
+ *            be captured in a CUDA graph.  The context's workspaces are shared
  *            by its calls: fci_sigma calls on one context must not overlap in
  *            time (issue them on one stream, or order the streams).
  * Errors: FCI_ERR_ARG (including the size limits above, reported on the host
@@ -322,9 +329,13 @@ int fci_rdm1(fci_ctx *ctx, const void *c, int dtype, double *gamma);
  *   <c|H|c> = sum h_pq gamma_pq + 1/2 sum (pq|rs) (Gamma_pqrs - delta_qr gamma_ps).
  * Gamma_pqrs = sum_K <K|E_qp|c> <K|E_rs|c> over the determinants K, computed
  * as the Gram matrices of (E_rs + E_sr)|c> and (E_rs - E_sr)|c>, and gamma, on
- * the tensor cores with FP64 accuracy (c in 45-bit fixed point relative to its largest element, six 8-bit digits, exact integer
- * accumulation): about 1e-14 of ||c||^2, bit-reproducible.  c need
- * not be normalised (both densities scale with ||c||^2).
+ * the tensor cores (c in 45-bit fixed point relative to its largest element, six
+ * 8-bit digits, exact integer accumulation), bit-reproducible.  The error of an
+ * element of Gamma is up to about 3e-14 N max|c|^2 + 4e-13 ||c||^2 for N
+ * determinants: 4e-13 of ||c||^2 for coefficients of one size, 1e-10 for a CI vector
+ * dominated by one determinant at CAS(12,12); gamma1's about a fifth of it (fci_rdm1
+ * is exact to FP64 rounding).  c need not be normalised (both densities scale with
+ * ||c||^2).
  *
  *  c       device vector (dtype FCI_F64 or FCI_F32) of N elements; the call
  *          first waits for all work on the device
@@ -346,12 +357,11 @@ int fci_rdm2(fci_ctx *ctx, const void *c, int dtype, double *gamma1, double *gam
  * any device memory.  The paper has no counterpart: this is an interface
  * convenience.
  *
- * fci_rdm1 allocates its scratch (one partial sum per replacement-list entry)
- * with cudaMalloc and releases it with cudaFree on every call.  Some callers
- * cannot do that: an application whose device memory is handed out entirely
+ * fci_rdm1 takes its scratch (lists of string pairs, and a partial sum per pair
+ * and block of rows) with cudaMalloc, on the first call or, beyond 64 MiB, on every
+ * call, and waits for all work on the device.  Some callers cannot do that: an application whose device memory is handed out entirely
  * by its own pool or by a framework's caching allocator, or one that keeps
- * other streams busy and cannot accept the device-wide synchronisation that
- * cudaFree implies.  This entry point serves them: it uses a fixed array in
+ * other streams busy and cannot accept a device-wide synchronisation.  This entry point serves them: it uses a fixed array in
  * the library's device memory and runs on the caller's stream.
  *
  *  c       device vector (dtype FCI_F64 or FCI_F32), ordered on `stream`

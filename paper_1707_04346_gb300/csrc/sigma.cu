@@ -16,7 +16,11 @@
 //    and beta-alpha halves coincide).  FP64: one CTA owns an output row; for
 //    each alpha replacement a it stages C(J_a, :) and W[p_a, :] in shared
 //    memory and accumulates the row of sigma in shared memory (diagonal
-//    replacements merged, see k_sigma3_exact).  FP32: sigma_tc.cu.
+//    replacements merged, see k_sigma3_exact).  FP32: sigma3_f32.cu, sigma_tc.cu.
+// These are the FP64 multiply-add and double-float kernels, the fused FP32 walk of few
+// strings, and the choice among all: small spaces run sigma_small.cu; else the default
+// FP64 terms are those of sigma3_sliced.cu or sigma_wide.cu with sigma_ss.cu, the FP32
+// same-spin terms those of sigma_ss32.cu (beyond 16384 strings sigma_tc.cu).
 #include "internal.cuh"
 
 namespace fci {

@@ -184,7 +184,7 @@ static double macs(const fci_ctx *ctx) {  // multiply-adds of the call
 // FP64 up to kSmall64 multiply-adds (CAS(9; 5,4), 1.1e7: 37 us against 81 us with
 // the sliced products; CAS(10; 5,3), 2.4e7: 89 with them).  FP32 up to kSmall32 for
 // unequal spins (CAS(10; 5,4): 51 us against 68 with the dense products; CAS(11;
-// 6,5), 3e8: 270 against 115) and kSmall32Same for one string space, whose same-spin
+// 6,5), 3.5e8: 270 against 115) and kSmall32Same for one string space, whose same-spin
 // terms the fused table walk of sigma.cu takes next (15876 determinants of CAS(9; 4,4):
 // 19 us against 28; CAS(11; 3,3), 2e7: 44 both; CAS(10; 4,4), 4e7: 50 against 44).
 // Both spins with replacements (the single-spin terms alone stay with the staged

@@ -32,7 +32,7 @@
 // 1190 cycles that a K-step of 48 columns took.)
 // G_s between strings that differ by more than two replacements is zero, and
 // strings in address order share their high orbitals: of the K-steps of a
-// 96-row block of G, 12 % (CAS(14,14)) and 34 % (CAS(16,16)) hold only zeros.
+// 96-row block of G, 9 % (CAS(14,14)) and 33 % (CAS(16,16)) hold only zeros.
 // B keeps the others, with their list per block; rows of G as the narrow side
 // of the tile skip more than as the 128-row side.
 // NB = 96 where the tiles fill the chip: the digit products run as MMAs of N =

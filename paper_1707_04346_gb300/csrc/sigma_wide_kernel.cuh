@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     *s_fail = 1;
             }
         } else if (warp < kMmaWarp) {
-            // ---- epilogue: lane m of the tile, 8-column chunks grp, grp + 2, ... ----
+            // ---- epilogue: lane m of the tile, 8-column chunks grp, grp + 3, ... ----
             const int quarter = warp & 3, grp = (warp - 4) >> 2;
             const int m = quarter * 32 + lane;
             const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
