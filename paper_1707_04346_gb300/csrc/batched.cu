@@ -445,13 +445,14 @@ __global__ void k_bpad(const int *__restrict__ on, const double *__restrict__ nr
 }
 
 // Eigenvalues and eigenvectors of each instance's projected matrix (small_dense.cuh).
+template <bool RESCALE>
 __global__ void __launch_bounds__(kBlock) k_bjacobi(const int *__restrict__ on, const double *__restrict__ Aall, int m,
                                                     double *__restrict__ wall, double *__restrict__ Vall) {
     const int i = blockIdx.x;
     if (!on[i]) return;
     __shared__ sd::EigShared S;
-    sd::eig_symmetric(Aall + (int64_t)i * kMaxSub * kMaxSub, kMaxSub, m, wall + (int64_t)i * kMaxSub,
-                      Vall + (int64_t)i * kMaxSub * kMaxSub, S);
+    sd::eig_symmetric<RESCALE>(Aall + (int64_t)i * kMaxSub * kMaxSub, kMaxSub, m, wall + (int64_t)i * kMaxSub,
+                               Vall + (int64_t)i * kMaxSub * kMaxSub, S);
 }
 
 // nroots smallest diagonal entries per instance (ties: lower index) -> unit vectors in B_k
@@ -1165,8 +1166,13 @@ static int batch_davidson_run(fci_batch *b, int nroots, double tol, double *ener
     // instances that expand (padding elsewhere).  Returns m after the iteration.
     const int keep = std::min(keepn, maxsub);
     const unsigned gi = (unsigned)((ninst + 127) / 128);
+    bool rescale = false;
+    for (const fci_ctx *c : b->ctx) rescale = rescale || c->eig_rescale;
     auto iteration = [&](int mi, bool can_refine, int *sig_launches) -> int {
-        k_bjacobi<<<ninst, kBlock, 0, s>>>(W.on, W.A, mi, W.w, W.V);
+        if (rescale)
+            k_bjacobi<true><<<ninst, kBlock, 0, s>>>(W.on, W.A, mi, W.w, W.V);
+        else
+            k_bjacobi<false><<<ninst, kBlock, 0, s>>>(W.on, W.A, mi, W.w, W.V);
         for (int k = 0; k < nroots; ++k) {
             k_blincomb<<<b->nchunks, kBlock, 0, s>>>(b->d_chunks, W.on, W.Bv, ntot, mi, W.V + k, kMaxSub * kMaxSub, mi,
                                                       1.0, 0.0, W.X + (size_t)k * ntot);

@@ -348,10 +348,11 @@ __global__ void k_scale(double *__restrict__ y, const double *__restrict__ nrm2,
 
 // Eigenvalues w (ascending) and eigenvectors (columns of V[m][m]) of the
 // projected matrix (small_dense.cuh).
+template <bool RESCALE>
 __global__ void __launch_bounds__(256) k_jacobi(const double *__restrict__ A, int lda, int m, double *__restrict__ w,
                                                 double *__restrict__ V) {
     __shared__ sd::EigShared S;
-    sd::eig_symmetric(A, lda, m, w, V, S);
+    sd::eig_symmetric<RESCALE>(A, lda, m, w, V, S);
 }
 
 // What the host reads per iteration, into pinned host memory: Ritz values,
@@ -790,6 +791,14 @@ int dots(Work &W, const double *X, int m, const double *y, double *out, int stri
     return dots2(W, DotSet{X, y, out, stride, m}, DotSet{nullptr, nullptr, nullptr, 0, 0}, m, gate);
 }
 
+// Eigenpairs of the projected matrix (m vectors).
+void eigenproblem(Work &W, int m) {
+    if (W.ctx->eig_rescale)
+        k_jacobi<true><<<1, 256, 0, W.s>>>(W.A, kMaxSub, m, W.w, W.V);
+    else
+        k_jacobi<false><<<1, 256, 0, W.s>>>(W.A, kMaxSub, m, W.w, W.V);
+}
+
 // project y onto the spin parity (y <- (y + p y^T) / 2), if one is set
 int project_parity(Work &W, void *y, int elem) {
     if (W.parity == 0) return FCI_OK;
@@ -1009,7 +1018,7 @@ static int run_davidson_f32basis(fci_ctx *ctx, int nroots, double tol, double *e
         return FCI_OK;
     };
     for (it = 1; it <= ctx->opt.max_iter; ++it) {
-        k_jacobi<<<1, 256, 0, s>>>(W.A, kMaxSub, m, W.w, W.V);
+        eigenproblem(W, m);
         FCI_CUDA(cudaGetLastError());
         const int nr = nroots < m ? nroots : m;
         for (int k = 0; k < nr; ++k) {
@@ -1237,7 +1246,7 @@ int run_davidson(fci_ctx *ctx, int nroots, double tol, double *energies, void *v
 
     for (it = 1; it <= ctx->opt.max_iter; ++it) {
         // (4) diagonalise the projected matrix
-        k_jacobi<<<1, 256, 0, s>>>(W.A, kMaxSub, m, W.w, W.V);
+        eigenproblem(W, m);
         FCI_CUDA(cudaGetLastError());
         const int nr = nroots < m ? nroots : m;
         // Ritz vectors, their sigma, residuals and (2)-(3) preconditioned corrections

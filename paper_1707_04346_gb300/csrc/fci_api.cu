@@ -254,6 +254,11 @@ int fci_init(fci_ctx **out, int norb, int nalpha, int nbeta, const double *h1, c
     cudaError_t e = cudaSetDevice(dev);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) { delete ctx; return cuda_fail(e, "device setup"); }
+    // with integrals up to wmax the norm of H is below norb^2 wmax + norb^4 wmax / 2 < 2^19 wmax
+    double wmax = 0.0;
+    for (int64_t i = 0; i < (int64_t)norb * norb; ++i) wmax = std::fmax(wmax, std::fabs(h1[i]));
+    for (int64_t i = 0; i < (int64_t)norb * norb * norb * norb; ++i) wmax = std::fmax(wmax, std::fabs(eri[i]));
+    ctx->eig_rescale = wmax > 0x1p80 || (wmax < 0x1p-40 && wmax > 0.0);
     int rc = FCI_OK;
     try {
         rc = build_tables(ctx, h1, eri);

@@ -154,6 +154,7 @@ struct fci_ctx {
     bool f32_captured = false;
     int *ssEr = nullptr, *ssEc = nullptr;
     double *hdiag = nullptr;        // [ndet]
+    bool eig_rescale = false;       // projected matrices of H may be out of FP32's range
     int *d_err = nullptr;           // device error word (bounded waits that gave up)
     std::atomic<size_t> bytes{0};   // calls of several threads allocate
     // Davidson bookkeeping

@@ -82,13 +82,14 @@ constexpr int kEigMax = 32;
 //     them in FP64, and FP64 sweeps finish on the nearly diagonal matrix until a
 //     sweep rotates nothing (|a_pq| <= 2^-46 max(|a_pp|, |a_qq|) is skipped).
 // A rotation's tangent is formed in FP32 (an inexact angle leaves 1e-7 of the
-// element for the next sweep), where FP32 does not reach from values scaled by the
-// power of two of the off-diagonal element; a matrix too large for FP32 enters the
-// first stage scaled, and what is too small for it waits for the second: no FP64
-// matrix is out of range.  Its cosine is 1 / sqrt(1 + t^2) to FP64
-// rounding by one third-order correction of the FP32 reciprocal root, so that
-// every rotation is orthogonal to FP64 rounding.  A non-finite matrix ends both
-// stages at once and comes back as non-finite eigenvalues.
+// element for the next sweep).  Where the matrix may be out of FP32's range (RESCALE,
+// told by the integrals, fci_ctx::eig_rescale) one whose largest element is not between 2^-40
+// and 2^100 is scaled by a power of two and its eigenvalues scaled back; elements below
+// 2^-100 are not rotated.  (With the look at the elements in every launch the kernel took
+// 2 us more of 103.)  The rotation's cosine is 1 / sqrt(1 + t^2) to FP64 rounding by
+// one third-order correction of the FP32 reciprocal root, so that every rotation is
+// orthogonal to FP64 rounding.  A non-finite matrix ends both stages at once and comes
+// back as non-finite eigenvalues.
 struct EigShared {
     double a[kEigMax][kEigMax + 1], v[kEigMax][kEigMax + 1], t[kEigMax][kEigMax + 1];
     float af[kEigMax][kEigMax + 1], vf[kEigMax][kEigMax + 1];
@@ -108,15 +109,6 @@ __device__ __forceinline__ void rr_pair(int k, int step, int n, int &p, int &q) 
     const int x = player(k), y = player(n - 1 - k);
     p = min(x, y);
     q = max(x, y);
-}
-
-// x 2^(1023 - e) as FP32, rounded toward zero: zero below the range, infinite above.
-__device__ __forceinline__ float scaled_float(double x, int e) {
-    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7FF, E = ex - e + 127;
-    uint32_t b = ((uint32_t)E << 23) | ((uint32_t)(hi & 0xFFFFF) << 3) | ((uint32_t)__double2loint(x) >> 29);
-    if (ex == 0 || E <= 0) b = 0u;
-    if (ex != 0 && E >= 255) b = 0x7F800000u;
-    return __uint_as_float(b | ((uint32_t)hi & 0x80000000u));
 }
 
 // Sweeps of rotations on a (m x m, symmetric) with the vectors in v; c and s:
@@ -147,24 +139,15 @@ __device__ __forceinline__ void jacobi_sweeps(T (*a)[kEigMax + 1], T (*v)[kEigMa
                 if (q < m) {
                     const T apq = a[p][q], app = a[p][p], aqq = a[q][q];
                     bool rot;
-                    float d, o;  // a_qq - a_pp and a_pq, to one scale
                     if constexpr (sizeof(T) == 8) {  // |a_pq| > 2^-46 max(|a_pp|, |a_qq|), on the exponents
                         const int h = __double2hiint(apq) & 0x7FFFFFFF;
                         const int g = max(__double2hiint(app) & 0x7FFFFFFF, __double2hiint(aqq) & 0x7FFFFFFF);
-                        rot = h > g - (46 << 20) && h < 0x7FF00000 && h >= 0x00100000;
-                        d = (float)(aqq - app);
-                        o = (float)apq;
-                        if ((uint32_t)(h - (923 << 20)) >= 200u << 20) {  // not within 2^+-100
-                            d = scaled_float(aqq - app, h >> 20);
-                            o = scaled_float(apq, h >> 20);
-                        }
+                        rot = h > g - (46 << 20) && h < 0x7FF00000 && h >= 923 << 20;
                     } else {
-                        rot = fabsf(apq) > 2e-7f * fmaxf(fabsf(app), fabsf(aqq)) && fabsf(apq) > 1e-36f;
-                        d = aqq - app;
-                        o = apq;
+                        rot = fabsf(apq) > fmaf(2e-7f, fmaxf(fabsf(app), fabsf(aqq)), 0x1p-100f);
                     }
                     if (rot) {
-                        const float th = __fdividef(d, 2.0f * o);
+                        const float th = __fdividef((float)(aqq - app), 2.0f * (float)apq);
                         const float tf = copysignf(1.0f, th) * __fdividef(1.0f, fabsf(th) + sqrtf(fmaf(th, th, 1.0f)));
                         const float yf = rsqrtf(fmaf(tf, tf, 1.0f));
                         if constexpr (sizeof(T) == 8) {
@@ -218,6 +201,32 @@ __device__ __forceinline__ void jacobi_sweeps(T (*a)[kEigMax + 1], T (*v)[kEigMa
     }
 }
 
+// S.t and S.af scaled to a largest element in [1, 2) where it is not between 2^-40 and
+// 2^100 (above the batch's padding of 1e30); the factor back.  Zero and non-finite matrices
+// stay as they are.
+__device__ __forceinline__ double eig_rescale(int m, EigShared &S) {
+    int ex = 0;
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) ex = max(ex, (__double2hiint(S.t[t / m][t % m]) >> 20) & 0x7FF);
+    if (threadIdx.x == 0) S.rotated = 0;
+    __syncthreads();
+    atomicMax(&S.rotated, ex);
+    __syncthreads();
+    ex = S.rotated;
+    double back = 1.0;
+    if (ex > 0 && ex < 0x7FF && (ex < 983 || ex > 1123)) {
+        const int e = max(2046 - ex, 1);
+        const double f = __hiloint2double(e << 20, 0);
+        back = __hiloint2double((2046 - e) << 20, 0);
+        for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+            S.t[t / m][t % m] *= f;
+            S.af[t / m][t % m] = (float)S.t[t / m][t % m];
+        }
+    }
+    __syncthreads();
+    return back;
+}
+
+template <bool RESCALE>
 __device__ __forceinline__ void eig_symmetric(const double *A, int lda, int m, double *w, double *V, EigShared &S) {
     const int tid = threadIdx.x;
     for (int t = tid; t < kEigMax * (kEigMax + 1); t += 256) {
@@ -225,24 +234,16 @@ __device__ __forceinline__ void eig_symmetric(const double *A, int lda, int m, d
         (&S.a[0][0])[t] = 0.0;
     }
     __syncthreads();
-    int ex = 0;
     for (int t = tid; t < m * m; t += blockDim.x) {
         const int i = t / m, j = t % m;
         const double x = 0.5 * (A[i * lda + j] + A[j * lda + i]);
         S.t[i][j] = x;
         S.af[i][j] = (float)x;
         S.vf[i][j] = i == j ? 1.0f : 0.0f;
-        ex = max(ex, (__double2hiint(x) >> 20) & 0x7FF);
     }
-    if (__syncthreads_or(ex > 1123)) {  // beyond 2^100 (the batch pads with 1e30): scaled to below two
-        if (tid == 0) S.rotated = 0;
-        __syncthreads();
-        atomicMax(&S.rotated, ex);
-        __syncthreads();
-        ex = S.rotated < 0x7FF ? S.rotated : 1023;
-        for (int t = tid; t < m * m; t += blockDim.x) S.af[t / m][t % m] = scaled_float(S.t[t / m][t % m], ex);
-        __syncthreads();
-    }
+    __syncthreads();
+    double back = 1.0;
+    if constexpr (RESCALE) back = eig_rescale(m, S);
     jacobi_sweeps<float>(S.af, S.vf, S.cf, S.sf, m, &S.rotated, 12);
     __syncthreads();
     for (int t = tid; t < m * m; t += blockDim.x) S.v[t / m][t % m] = (double)S.vf[t / m][t % m];
@@ -306,7 +307,7 @@ __device__ __forceinline__ void eig_symmetric(const double *A, int lda, int m, d
         }
     }
     __syncthreads();
-    for (int t = tid; t < m; t += blockDim.x) w[t] = S.a[S.order[t]][S.order[t]];
+    for (int t = tid; t < m; t += blockDim.x) w[t] = RESCALE ? S.a[S.order[t]][S.order[t]] * back : S.a[S.order[t]][S.order[t]];
     for (int t = tid; t < m * m; t += blockDim.x) V[t] = S.v[t / m][S.order[t % m]];
 }
 
