@@ -260,8 +260,9 @@ int fci_free_default(void);
  *            FP64 sigma_3, 12N bytes, and of the dense same-spin products,
  *            24N bytes (12N for FP32 alone), are made at fci_init), so it can
  *            be captured in a CUDA graph.  The context's workspaces are shared
- *            by its calls: fci_sigma calls on one context must not overlap in
- *            time (issue them on one stream, or order the streams).
+ *            by its calls: fci_sigma calls on one context, and fci_davidson,
+ *            which makes such calls, must not overlap in time (issue them on
+ *            one stream, or order the streams).
  * Errors: FCI_ERR_ARG (including the size limits above, reported on the host
  * before any launch), FCI_ERR_OOM, FCI_ERR_CUDA (launch failure).
  */
